@@ -164,156 +164,6 @@ __global__ void __launch_bounds__((TX3 + 1) * (TY3 + 1)) k_sweep3(const SweepArg
     if (MODE == kResidual && a.part) block_partial<NT>(ssq, a.part, red);
 }
 
-// FP64 3D sweep.  FP64 runs at ~1/72 of the FP32 rate on this GPU, so the kernel is
-// bound by FP64 instruction issue and is organised to keep the FP64 pipe fed:
-// a node plane's in-plane transform is computed once and shared by the two cell
-// layers it bounds, the forces a layer sends to its top plane are carried in the
-// transformed basis (one transposed in-plane butterfly per plane), and the 32 x 12
-// tile keeps the recomputed halo ring small.  No global load is waited on inside a
-// step: node planes arrive through a three-slot shared-memory ring filled by
-// cp.async two planes ahead, and the cell's psi and the node's right-hand side are
-// loaded into registers one step (psi) or one compute phase (f) before their use.
-// The last node plane of the grid is finalised by one extra step over an empty
-// (psi = 0) layer.
-constexpr int TXD = 32, TYD = 12;
-
-// 8-byte global -> shared copy; ok = false fills zeros (src must still be valid).
-__device__ __forceinline__ void cp_async8(void *sdst, const void *gsrc, bool ok)
-{
-    const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(sdst));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(sa), "l"(gsrc), "r"(ok ? 8 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-template <typename TO, int MODE>
-__global__ void __launch_bounds__((TXD + 1) * (TYD + 1)) k_sweep3_dp(const SweepArgs<double, TO> a)
-{
-    pdl_begin();
-    if (a.gate && *a.gate) return;
-    constexpr int BX = TXD + 1, BY = TYD + 1, NT = BX * BY;
-    constexpr int PX = TXD + 2, PY = TYD + 2, PP = PX * PY;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *up = reinterpret_cast<double *>(smem_raw);   // [3][3][PP] ring of node planes
-    double *fc = up + 3 * 3 * PP;                         // [3][4][PP] corner forces of one plane
-    double *ps = fc + 12 * PP;                            // [PP] psi of the cells below + above
-    __shared__ double red[((NT + 31) / 32) * 32];
-
-    const Geom &g = a.g;
-    static_assert(BX == 33, "row-aligned warps need 32-cell rows");
-    const int tid = threadIdx.x + BX * threadIdx.y;
-    int tx, ty;
-    row_warp_xy<BY>(tid, tx, ty);
-    for (int s = tid; s < PP; s += NT) {
-        const int lx = s % PX, ly = s / PX;
-        if (lx == BX || ly == BY) {
-            for (int q = 0; q < 12; ++q) fc[q * PP + s] = 0.0;
-            ps[s] = 0.0;
-        }
-    }
-    // Persistent: the units are (tile, node plane) pairs, tile-major; block b owns a
-    // contiguous range of them and streams it as one z segment per tile it touches.
-    const int ntx = (g.nx - 1 + TXD - 1) / TXD, nty = (g.ny - 1 + TYD - 1) / TYD;
-    const long long U = (long long)ntx * nty * g.nz;
-    const long long ub = U * blockIdx.x / gridDim.x, ue = U * (blockIdx.x + 1) / gridDim.x;
-    double ssq = 0.0;
-    for (long long su = ub; su < ue;) {
-        const int tile = (int)(su / g.nz), kz0 = (int)(su % g.nz);
-        const int kend = (int)min((long long)g.nz, kz0 + (ue - su)) - 1;   // last node plane finalised
-        su += kend + 1 - kz0;
-        const int x0 = (tile % ntx) * TXD, y0 = (tile / ntx) * TYD;
-        const int kfirst = kz0 > 0 ? kz0 - 1 : 0;
-        // node plane k into ring slot k % 3 (zeros outside the grid)
-        auto load_plane = [&](int k) {
-            double *dst = up + (k % 3) * 3 * PP;
-            for (int s = tid; s < PP; s += NT) {
-                const int lx = s % PX, ly = s / PX;
-                const int gx = x0 - 1 + lx, gy = y0 - 1 + ly;
-                const bool ok = gx >= 0 && gx < g.nx && gy >= 0 && gy < g.ny && k >= 0 && k < g.nz;
-                const long long o = ok ? gidx(g, gx, gy, k) : 0;
-#pragma unroll
-                for (int p = 0; p < 3; ++p) cp_async8(dst + p * PP + s, a.u + (ok ? p * g.cs + o : 0), ok);
-            }
-            cp_async_commit();
-        };
-        const int gx = x0 + tx, gy = y0 + ty;
-        const bool own = gx < g.nx && gy < g.ny && (tx < TXD || gx == g.nx - 1) && (ty < TYD || gy == g.ny - 1);
-        const int cx = gx - 1, cy = gy - 1;
-        const bool cell_ok = cx >= 0 && cx < g.nx - 1 && cy >= 0 && cy < g.ny - 1;
-        const int me = ty * PX + tx;
-        auto corners = [&](int k, double (&T)[3][4]) {
-            const double *pl = up + (k % 3) * 3 * PP;
-#pragma unroll
-            for (int p = 0; p < 3; ++p) {
-                T[p][0] = pl[p * PP + me];
-                T[p][1] = pl[p * PP + me + 1];
-                T[p][2] = pl[p * PP + me + PX];
-                T[p][3] = pl[p * PP + me + PX + 1];
-                bfly4xy(T[p]);
-            }
-        };
-        auto cell_psi = [&](int lz) { return (cell_ok && lz <= g.nz - 2) ? a.psi[gidx(g, cx, cy, lz)] : 0.0; };
-
-        double Tb[3][4], Cf[3][4];
-#pragma unroll
-        for (int p = 0; p < 3; ++p)
-#pragma unroll
-            for (int s = 0; s < 4; ++s) Cf[p][s] = 0.0;
-        double psi_prev = 0.0;
-        double psi = cell_psi(kfirst);
-        load_plane(kfirst);
-        load_plane(kfirst + 1);
-        cp_async_wait_all();
-        __syncthreads();
-        corners(kfirst, Tb);
-        for (int lz = kfirst; lz <= kend; ++lz) {
-            load_plane(lz + 2);                               // slot of plane lz - 1, free since the last barrier
-            const double psi_next = cell_psi(lz + 1);
-            const bool fin = own && lz >= kz0;
-            double fv[3];
-            const long long on = gidx(g, gx, gy, lz);
-#pragma unroll
-            for (int p = 0; p < 3; ++p) fv[p] = (MODE != kApply && fin) ? a.f[p * g.cs + on] : 0.0;
-            double Tt[3][4], Fb[3][4], Ft[3][4];
-            corners(lz + 1, Tt);
-            cell_faces3<double>(Tb, Tt, psi, a.c, Fb, Ft);
-#pragma unroll
-            for (int p = 0; p < 3; ++p) {
-#pragma unroll
-                for (int s = 0; s < 4; ++s) {
-                    Fb[p][s] += Cf[p][s];   // plane lz: top face of layer lz-1 + bottom face of layer lz
-                    Cf[p][s] = Ft[p][s];
-                    Tb[p][s] = Tt[p][s];
-                }
-                bfly4xyT(Fb[p]);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) fc[(p * 4 + q) * PP + me] = Fb[p][q];
-            }
-            ps[me] = psi_prev + psi;
-            psi_prev = psi;
-            psi = psi_next;
-            __syncthreads();
-            if (fin) {
-                double Ku[3], uv[3];
-                const double *pl = up + (lz % 3) * 3 * PP;
-#pragma unroll
-                for (int p = 0; p < 3; ++p) {
-                    Ku[p] = (fc[(p * 4 + 3) * PP + me] + fc[(p * 4 + 2) * PP + me + 1]) +
-                            (fc[(p * 4 + 1) * PP + me + PX] + fc[(p * 4 + 0) * PP + me + PX + 1]);
-                    uv[p] = pl[p * PP + me + PX + 1];
-                }
-                const double pss = (ps[me] + ps[me + 1]) + (ps[me + PX] + ps[me + PX + 1]);
-                body::finalize_f<double, TO, MODE>(a, gx, gy, lz, Ku, pss, uv, fv, ssq);
-            }
-            cp_async_wait_all();                              // plane lz + 2 in this thread's copies
-            __syncthreads();
-        }
-    }
-    if (MODE == kResidual && a.part) block_partial<NT>(ssq, a.part, red);
-}
-
-constexpr size_t smem_dp() { return sizeof(double) * (3 * 3 + 12 + 1) * (TXD + 2) * (TYD + 2); }
-
 template <typename T, typename TO, int MODE>
 __global__ void __launch_bounds__((TX2 + 1) * (TY2 + 1)) k_sweep2(const SweepArgs<T, TO> a)
 {
@@ -555,16 +405,6 @@ constexpr size_t smem_gs2()
 
 }  // namespace
 
-// Persistent FP64 sweep: one block per SM of the 152 (one fits per SM), at most one
-// per (tile, node plane) unit.
-static void sweep_grid_dp(const Geom &g, int *grid, int *kchunk)
-{
-    const long long units = (long long)((g.nx - 1 + TXD - 1) / TXD) * ((g.ny - 1 + TYD - 1) / TYD) * g.nz;
-    grid[0] = (int)std::min<long long>(152, units);
-    grid[1] = grid[2] = 1;
-    *kchunk = 0;
-}
-
 void sweep_grid(const Geom &g, int *grid, int *kchunk)
 {
     if (g.dim == 3) {
@@ -585,9 +425,9 @@ void sweep_grid(const Geom &g, int *grid, int *kchunk)
 
 long long sweep_blocks(const Geom &g, bool fp64)
 {
+    if (fp64 && g.dim == 3) return sweep_blocks_fix(g);
     int grid[3], ch;
-    if (fp64 && g.dim == 3) sweep_grid_dp(g, grid, &ch);
-    else sweep_grid(g, grid, &ch);
+    sweep_grid(g, grid, &ch);
     return (long long)grid[0] * grid[1] * grid[2];
 }
 
@@ -654,26 +494,17 @@ static cudaError_t launch_mode(const SweepArgs<T, TO> &a0, cudaStream_t s)
 {
     SweepArgs<T, TO> a = a0;
     int grid[3];
-    if (a.g.dim == 3 && sizeof(T) == 8) {
-        sweep_grid_dp(a.g, grid, &a.kchunk);
-        const size_t sm = smem_dp();
-        static std::atomic<unsigned long long> attr_dp{0};
-        cudaError_t ea = smem_attr_once(reinterpret_cast<const void *>(k_sweep3_dp<TO, MODE>), sm, attr_dp);
-        if (ea != cudaSuccess) return ea;
-        cudaError_t e = launch_pdl(k_sweep3_dp<TO, MODE>, dim3(grid[0], grid[1], grid[2]), dim3(TXD + 1, TYD + 1), sm, s,
-                                   reinterpret_cast<const SweepArgs<double, TO> &>(a));
-        if (e != cudaSuccess) return e;
-        ++g_launches;
-        return cudaGetLastError();
-    }
     sweep_grid(a.g, grid, &a.kchunk);
     if (a.g.dim == 3) {
-        const size_t sm = smem3<T>();
-        static std::atomic<unsigned long long> attr_done{0};
-        cudaError_t ea = smem_attr_once(reinterpret_cast<const void *>(k_sweep3<T, TO, MODE>), sm, attr_done);
-        if (ea != cudaSuccess) return ea;
-        cudaError_t e = launch_pdl(k_sweep3<T, TO, MODE>, dim3(grid[0], grid[1], grid[2]), dim3(TX3 + 1, TY3 + 1), sm, s, a);
-        if (e != cudaSuccess) return e;
+        if constexpr (sizeof(T) == 4) {            // FP64: launch_sweep_fix
+            const size_t sm = smem3<T>();
+            static std::atomic<unsigned long long> attr_done{0};
+            cudaError_t ea = smem_attr_once(reinterpret_cast<const void *>(k_sweep3<T, TO, MODE>), sm, attr_done);
+            if (ea != cudaSuccess) return ea;
+            cudaError_t e = launch_pdl(k_sweep3<T, TO, MODE>, dim3(grid[0], grid[1], grid[2]), dim3(TX3 + 1, TY3 + 1), sm,
+                                       s, a);
+            if (e != cudaSuccess) return e;
+        }
     } else {
         cudaError_t e = launch_pdl(k_sweep2<T, TO, MODE>, dim3(grid[0], grid[1], 1), dim3(TX2 + 1, TY2 + 1), 0, s, a);
         if (e != cudaSuccess) return e;
@@ -685,6 +516,8 @@ static cudaError_t launch_mode(const SweepArgs<T, TO> &a0, cudaStream_t s)
 template <typename T, typename TO>
 cudaError_t launch_sweep(int mode, const SweepArgs<T, TO> &a, cudaStream_t s)
 {
+    if constexpr (sizeof(T) == 8)
+        if (a.g.dim == 3) return launch_sweep_fix<TO>(mode, a, s);
     switch (mode) {
     case kApply: return launch_mode<T, TO, kApply>(a, s);
     case kResidual: return launch_mode<T, TO, kResidual>(a, s);

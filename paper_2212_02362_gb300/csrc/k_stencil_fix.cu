@@ -1,0 +1,433 @@
+// k_stencil_fix.cu — FP64 3D apply / residual / damped-Jacobi sweep with the cell
+// arithmetic in 64-bit integers (sbm_fix.cuh).
+//
+// What bounds it.  With FP64 instructions this sweep is bound by their issue rate (about
+// two lanes per SM and clock on GB300): some 180 of them per cell.  In block floating
+// point the same cell takes about 800 integer instructions, which issue 64 times as
+// fast, and leaves some ten FP64 instructions per node (the conversion of the node's
+// force, f - K u, the norm), which run on the FP64 pipe beside them.
+//
+// Work split.  A block owns a tile of 32 x 10 cells in x/y (33 x 11 threads, one per cell
+// column with the halo column and row; 12 warps, so 168 registers a thread) and a
+// contiguous range of (tile, node plane) units, which it streams along z, one cell layer
+// a step.  Node planes pass through a four-slot shared-memory ring in three stages, so
+// that nothing inside a step waits for global memory and two barriers a step suffice:
+//   plane lz+3  copied by cp.async while step lz computes; at the step's end each thread
+//               takes the largest exponent of the values it copied into the plane's key
+//   plane lz+2  turned into integers in place, each thread the values it copied
+//   plane lz+1  read by the cells of layer lz
+// The forces a layer sends to its top plane are carried in registers in the transformed
+// basis with their exponent; those of the four columns around a node are exchanged
+// through shared memory with the exponents beside them.
+//
+// A plane or a psi that the integer form does not take (sbm_fix.cuh) ends the integer
+// loop before any node that depends on it; the block finishes its range with the FP64
+// body below, which also runs when the level's constants do not fit.
+#include <algorithm>
+
+#include "sbm_common.cuh"
+#include "sbm_bodies.cuh"
+#include "sbm_fix.cuh"
+
+namespace sbm {
+
+namespace {
+
+using fix::i64;
+
+constexpr int TX = 32, TY = 10;                   // cells of a tile
+constexpr int BX = TX + 1, BY = TY + 1, NT = BX * BY;
+constexpr int PX = TX + 2, PY = TY + 2, PP = PX * PY;
+// ring of node planes (4 x 3 components), exchanged forces (12 for the FP64 body, 9 and
+// an exponent here), psi of the cells below + above
+constexpr size_t kSmem = sizeof(double) * (12 + 12 + 1) * PP + sizeof(int) * PP;
+
+// 8-byte global -> shared copy; ok = false fills zeros (src must still be valid).
+__device__ __forceinline__ void cp_async8(void *sdst, const void *gsrc, bool ok)
+{
+    const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(sdst));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(sa), "l"(gsrc), "r"(ok ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+
+// Deterministic block reduction of ssq into part[block].
+__device__ __forceinline__ void block_partial(double ssq, double *part, double *red)
+{
+    constexpr int NW = (NT + 31) / 32;
+    const int tid = threadIdx.x;
+    red[tid] = ssq;
+    if (tid < NW * 32 - NT) red[NT + tid] = 0.0;
+    __syncthreads();
+    if (tid < 32) {
+        double s = 0.0;
+        for (int w = 0; w < NW; ++w) s += red[w * 32 + tid];
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+        if (tid == 0) part[blockIdx.x] = s;
+    }
+}
+
+// One tile's share of the grid for this thread.
+struct Tile {
+    int x0, y0;            // first owned node
+    int gx, gy;            // the thread's node; its cell is (gx - 1, gy - 1)
+    bool own, cell_ok;
+};
+
+__device__ __forceinline__ Tile make_tile(const Geom &g, int t, int ntx, int tx, int ty)
+{
+    Tile T;
+    T.x0 = (t % ntx) * TX;
+    T.y0 = (t / ntx) * TY;
+    T.gx = T.x0 + tx;
+    T.gy = T.y0 + ty;
+    T.own = T.gx < g.nx && T.gy < g.ny && (tx < TX || T.gx == g.nx - 1) && (ty < TY || T.gy == g.ny - 1);
+    T.cell_ok = T.gx >= 1 && T.gx < g.nx && T.gy >= 1 && T.gy < g.ny;
+    return T;
+}
+
+// Node plane k of a tile into the shared array dst[3][PP] (zeros outside the grid).
+__device__ __forceinline__ void load_plane(const double *u, const Geom &g, const Tile &T, int k, double *dst)
+{
+    for (int s = threadIdx.x; s < PP; s += NT) {
+        const int lx = s % PX, ly = s / PX;
+        const int gx = T.x0 - 1 + lx, gy = T.y0 - 1 + ly;
+        const bool ok = gx >= 0 && gx < g.nx && gy >= 0 && gy < g.ny && k >= 0 && k < g.nz;
+        const long long o = ok ? gidx(g, gx, gy, k) : 0;
+#pragma unroll
+        for (int p = 0; p < 3; ++p) cp_async8(dst + p * PP + s, u + (ok ? p * g.cs + o : 0), ok);
+    }
+    cp_async_commit();
+}
+
+// The units [ub, ue) with FP64 instructions: what the integer form does not take.  A node
+// plane's in-plane transform is shared by the two cell layers it bounds, and planes come
+// through a three-slot ring two steps ahead.
+template <typename TO, int MODE>
+__device__ __noinline__ double sweep_dp(const SweepArgs<double, TO> &a, long long ub, long long ue, double *up)
+{
+    double *fc = up + 12 * PP, *ps = fc + 12 * PP;
+    const Geom &g = a.g;
+    const int tid = threadIdx.x;
+    int tx, ty;
+    row_warp_xy<BY>(tid, tx, ty);
+    __syncthreads();
+    for (int s = tid; s < PP; s += NT) {
+        const int lx = s % PX, ly = s / PX;
+        if (lx == BX || ly == BY) {
+            for (int q = 0; q < 12; ++q) fc[q * PP + s] = 0.0;
+            ps[s] = 0.0;
+        }
+    }
+    const int ntx = (g.nx - 1 + TX - 1) / TX;
+    double ssq = 0.0;
+    for (long long su = ub; su < ue;) {
+        const int kz0 = (int)(su % g.nz);
+        const int kend = (int)min((long long)g.nz, kz0 + (ue - su)) - 1;   // last node plane finalised
+        const Tile T = make_tile(g, (int)(su / g.nz), ntx, tx, ty);
+        su += kend + 1 - kz0;
+        const int kfirst = kz0 > 0 ? kz0 - 1 : 0;
+        const int me = ty * PX + tx;
+        auto corners = [&](int k, double (&C)[3][4]) {
+            const double *pl = up + (k % 3) * 3 * PP;
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                C[p][0] = pl[p * PP + me];
+                C[p][1] = pl[p * PP + me + 1];
+                C[p][2] = pl[p * PP + me + PX];
+                C[p][3] = pl[p * PP + me + PX + 1];
+                bfly4xy(C[p]);
+            }
+        };
+        auto cell_psi = [&](int lz) {
+            return (T.cell_ok && lz <= g.nz - 2) ? a.psi[gidx(g, T.gx - 1, T.gy - 1, lz)] : 0.0;
+        };
+        double Tb[3][4], Cf[3][4];
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int s = 0; s < 4; ++s) Cf[p][s] = 0.0;
+        double psi_prev = 0.0;
+        double psi = cell_psi(kfirst);
+        load_plane(a.u, g, T, kfirst, up + (kfirst % 3) * 3 * PP);
+        load_plane(a.u, g, T, kfirst + 1, up + ((kfirst + 1) % 3) * 3 * PP);
+        cp_async_wait_all();
+        __syncthreads();
+        corners(kfirst, Tb);
+        for (int lz = kfirst; lz <= kend; ++lz) {
+            load_plane(a.u, g, T, lz + 2, up + ((lz + 2) % 3) * 3 * PP);   // slot of plane lz - 1
+            const double psi_next = cell_psi(lz + 1);
+            const bool fin = T.own && lz >= kz0;
+            double fv[3];
+            const long long on = gidx(g, T.gx, T.gy, lz);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) fv[p] = (MODE != kApply && fin) ? a.f[p * g.cs + on] : 0.0;
+            double Tt[3][4], Fb[3][4], Ft[3][4];
+            corners(lz + 1, Tt);
+            cell_faces3<double>(Tb, Tt, psi, a.c, Fb, Ft);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    Fb[p][s] += Cf[p][s];   // plane lz: top face of layer lz-1 + bottom face of layer lz
+                    Cf[p][s] = Ft[p][s];
+                    Tb[p][s] = Tt[p][s];
+                }
+                bfly4xyT(Fb[p]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) fc[(p * 4 + q) * PP + me] = Fb[p][q];
+            }
+            ps[me] = psi_prev + psi;
+            psi_prev = psi;
+            psi = psi_next;
+            __syncthreads();
+            if (fin) {
+                double Ku[3], uv[3];
+                const double *pl = up + (lz % 3) * 3 * PP;
+#pragma unroll
+                for (int p = 0; p < 3; ++p) {
+                    Ku[p] = (fc[(p * 4 + 3) * PP + me] + fc[(p * 4 + 2) * PP + me + 1]) +
+                            (fc[(p * 4 + 1) * PP + me + PX] + fc[(p * 4 + 0) * PP + me + PX + 1]);
+                    uv[p] = pl[p * PP + me + PX + 1];
+                }
+                const double pss = (ps[me] + ps[me + 1]) + (ps[me + PX] + ps[me + PX + 1]);
+                body::finalize_f<double, TO, MODE>(a, T.gx, T.gy, lz, Ku, pss, uv, fv, ssq);
+            }
+            cp_async_wait_all();                              // plane lz + 2 in this thread's copies
+            __syncthreads();
+        }
+    }
+    return ssq;
+}
+
+template <typename TO, int MODE>
+__global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO> a, const fix::Consts fc)
+{
+    pdl_begin();
+    if (a.gate && *a.gate) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *up = reinterpret_cast<double *>(smem_raw);        // [4][3][PP]: doubles, then integers
+    i64 *X = reinterpret_cast<i64 *>(up + 12 * PP);            // [9][PP]: corner forces 0..2 of a plane
+    double *ps = up + 24 * PP;                                 // [PP]
+    int *Xe = reinterpret_cast<int *>(ps + PP);                // [PP]: their exponents
+    __shared__ double red[((NT + 31) / 32) * 32];
+    __shared__ unsigned keys[4];
+
+    const Geom &g = a.g;
+    const int tid = threadIdx.x;
+    int tx, ty;
+    row_warp_xy<BY>(tid, tx, ty);
+    for (int s = tid; s < PP; s += NT) {
+        const int lx = s % PX, ly = s / PX;
+        if (lx == BX || ly == BY) {                            // no cells there
+            for (int q = 0; q < 9; ++q) X[q * PP + s] = 0;
+            Xe[s] = fix::kNoExp;
+            ps[s] = 0.0;
+        }
+    }
+    const int ntx = (g.nx - 1 + TX - 1) / TX, nty = (g.ny - 1 + TY - 1) / TY;
+    const long long U = (long long)ntx * nty * g.nz;
+    const long long ub = U * blockIdx.x / gridDim.x, ue = U * (blockIdx.x + 1) / gridDim.x;
+    const int me = ty * PX + tx;
+    double ssq = 0.0;
+    long long rest = fc.ok ? ue : ub;          // units from here on are left to the FP64 body
+
+    auto slot = [&](int k) { return up + (k & 3) * 3 * PP; };
+    // the largest exponent key of the values this thread copied, into the plane's key
+    auto take_key = [&](int k) {
+        const double *pl = slot(k);
+        unsigned m = 0;
+        for (int s = tid; s < PP; s += NT)
+#pragma unroll
+            for (int p = 0; p < 3; ++p) m = max(m, fix::exp_key(pl[p * PP + s]));
+        const unsigned w = (tid | 31) < NT ? 0xffffffffu : (1u << (NT & 31)) - 1u;   // the last warp is partial
+        m = __reduce_max_sync(w, m);
+        if ((tid & 31) == 0) atomicMax(&keys[k & 3], m);
+    };
+    auto exp_of = [&](int k) { return max((int)(keys[k & 3] >> 20), fix::kExpLo); };
+    auto to_ints = [&](int k) {
+        double *pl = slot(k);
+        const int E = exp_of(k);
+        for (int s = tid; s < PP; s += NT)
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                const i64 v = fix::to_fix(pl[p * PP + s], E);
+                pl[p * PP + s] = fix::of_bits(v);
+            }
+    };
+    auto corners = [&](int k, i64 (&C)[3][4]) {
+        const i64 *pl = reinterpret_cast<const i64 *>(slot(k));
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+            C[p][0] = pl[p * PP + me];
+            C[p][1] = pl[p * PP + me + 1];
+            C[p][2] = pl[p * PP + me + PX];
+            C[p][3] = pl[p * PP + me + PX + 1];
+            bfly4xy(C[p]);
+        }
+    };
+
+    for (long long su = ub; su < ue && rest == ue;) {
+        const int t = (int)(su / g.nz), kz0 = (int)(su % g.nz);
+        const int kend = (int)min((long long)g.nz, kz0 + (ue - su)) - 1;   // last node plane finalised
+        const long long seg = su - kz0;                                    // unit of the tile's plane 0
+        const Tile T = make_tile(g, t, ntx, tx, ty);
+        su += kend + 1 - kz0;
+        const int kfirst = kz0 > 0 ? kz0 - 1 : 0;
+        auto cell_psi = [&](int lz) {
+            return (T.cell_ok && lz <= g.nz - 2) ? a.psi[gidx(g, T.gx - 1, T.gy - 1, lz)] : 0.0;
+        };
+        // planes kfirst, kfirst + 1 as integers, kfirst + 2 with its key
+        for (int k = kfirst; k < kfirst + 3; ++k) load_plane(a.u, g, T, k, slot(k));
+        if (tid < 4) keys[tid] = 0u;
+        double psi = cell_psi(kfirst), psi_prev = 0.0;
+        cp_async_wait_all();
+        __syncthreads();
+        for (int k = kfirst; k < kfirst + 3; ++k) take_key(k);
+        bool bad = __syncthreads_or(!fix::psi_ok(psi));
+        for (int k = kfirst; k < kfirst + 3; ++k) bad = bad || !fix::key_ok(keys[k & 3]);
+        if (bad) {
+            rest = seg + kz0;
+            break;
+        }
+        to_ints(kfirst);
+        to_ints(kfirst + 1);
+        __syncthreads();
+        i64 Tb[3][4], Cf[3][4];
+        int Eb = exp_of(kfirst), ecf = fix::kNoExp;
+        corners(kfirst, Tb);
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) Cf[p][q] = 0;
+#pragma unroll 1
+        for (int lz = kfirst; lz <= kend; ++lz) {
+            if (!fix::key_ok(keys[(lz + 2) & 3])) {            // the same for the whole block
+                rest = seg + max(lz, kz0);
+                break;
+            }
+            load_plane(a.u, g, T, lz + 3, slot(lz + 3));       // slot of plane lz - 1
+            const double psi_next = cell_psi(lz + 1);
+            const bool fin = T.own && lz >= kz0;
+            double fv[3], uv[3];
+            const long long on = fin ? gidx(g, T.gx, T.gy, lz) : 0;
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                fv[p] = (MODE != kApply && fin) ? a.f[p * g.cs + on] : 0.0;
+                uv[p] = (MODE == kJacobi && fin) ? a.u[p * g.cs + on] : 0.0;
+            }
+            to_ints(lz + 2);
+            // the cell of layer lz, both faces on the larger of their planes' units
+            const int Et = exp_of(lz + 1);
+            const int E = max(Eb, Et);
+            i64 Tt[3][4], Fb[3][4], Ft[3][4];
+            corners(lz + 1, Tt);
+            if (Eb != Et) {
+#pragma unroll
+                for (int p = 0; p < 3; ++p)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        Tb[p][q] = fix::down(Tb[p][q], E - Eb);
+                        Tt[p][q] = fix::down(Tt[p][q], E - Et);
+                    }
+            }
+            int e;
+            fix::cell_faces3(Tb, Tt, E, psi, fc, Fb, Ft, e);
+            if (E != Et) {
+                corners(lz + 1, Tb);
+            } else {
+#pragma unroll
+                for (int p = 0; p < 3; ++p)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) Tb[p][q] = Tt[p][q];
+            }
+            Eb = Et;
+            // plane lz: top face of layer lz - 1 + bottom face of layer lz
+            const int en = max(e, ecf), s0 = en - ecf, s1 = en - e;
+            i64 N[3][4];
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    N[p][q] = fix::down(Cf[p][q], s0) + fix::down(Fb[p][q], s1);
+                    Cf[p][q] = Ft[p][q];
+                }
+                bfly4xyT(N[p]);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) X[(p * 3 + q) * PP + me] = N[p][q];
+            }
+            Xe[me] = en;
+            ecf = e;
+            if (MODE == kJacobi) ps[me] = psi_prev + psi;
+            psi_prev = psi;
+            psi = psi_next;
+            __syncthreads();
+            if (tid == 0) keys[lz & 3] = 0u;                   // for plane lz + 4
+            if (fin) {
+                const int e1 = Xe[me + 1], e2 = Xe[me + PX], e3 = Xe[me + PX + 1];
+                const int ee = max(max(en, e1), max(e2, e3));
+                const int d0 = ee - en, d1 = ee - e1, d2 = ee - e2, d3 = ee - e3;
+                double Ku[3];
+#pragma unroll
+                for (int p = 0; p < 3; ++p) {
+                    const i64 s = (fix::down(N[p][3], d0) + fix::down(X[(p * 3 + 2) * PP + me + 1], d1)) +
+                                  (fix::down(X[(p * 3 + 1) * PP + me + PX], d2) +
+                                   fix::down(X[(p * 3 + 0) * PP + me + PX + 1], d3));
+                    Ku[p] = fix::to_double(s, ee);
+                }
+                double pss = 0.0;
+                if (MODE == kJacobi) pss = (ps[me] + ps[me + 1]) + (ps[me + PX] + ps[me + PX + 1]);
+                body::finalize_f<double, TO, MODE>(a, T.gx, T.gy, lz, Ku, pss, uv, fv, ssq);
+            }
+            cp_async_wait_all();                               // plane lz + 3 in this thread's copies
+            take_key(lz + 3);
+            if (__syncthreads_or(!fix::psi_ok(psi)) && lz < kend) {
+                rest = seg + max(lz + 1, kz0);
+                break;
+            }
+        }
+    }
+    if (rest < ue) ssq += sweep_dp<TO, MODE>(a, rest, ue, up);
+    if (MODE == kResidual && a.part) {
+        __syncthreads();
+        block_partial(ssq, a.part, red);
+    }
+}
+
+template <typename TO, int MODE>
+cudaError_t launch_fix_mode(const SweepArgs<double, TO> &a, cudaStream_t s)
+{
+    static std::atomic<unsigned long long> attr_done{0};
+    cudaError_t e = smem_attr_once(reinterpret_cast<const void *>(k_sweep3_fix<TO, MODE>), kSmem, attr_done);
+    if (e != cudaSuccess) return e;
+    const fix::Consts fc = fix::make_consts(3, a.c);
+    e = launch_pdl(k_sweep3_fix<TO, MODE>, dim3((unsigned)sweep_blocks_fix(a.g)), dim3(NT), kSmem, s, a, fc);
+    if (e != cudaSuccess) return e;
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// One block per SM of the 152, at most one per (tile, node plane) unit.
+long long sweep_blocks_fix(const Geom &g)
+{
+    const long long units = (long long)((g.nx - 1 + TX - 1) / TX) * ((g.ny - 1 + TY - 1) / TY) * g.nz;
+    return std::min<long long>(152, units);
+}
+
+template <typename TO>
+cudaError_t launch_sweep_fix(int mode, const SweepArgs<double, TO> &a, cudaStream_t s)
+{
+    switch (mode) {
+    case kApply: return launch_fix_mode<TO, kApply>(a, s);
+    case kResidual: return launch_fix_mode<TO, kResidual>(a, s);
+    case kJacobi: return launch_fix_mode<TO, kJacobi>(a, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+template cudaError_t launch_sweep_fix<double>(int, const SweepArgs<double, double> &, cudaStream_t);
+template cudaError_t launch_sweep_fix<float>(int, const SweepArgs<double, float> &, cudaStream_t);
+
+}  // namespace sbm

@@ -171,6 +171,12 @@ long long sweep_blocks(const Geom &g, bool fp64);
 template <typename T, typename TO>
 cudaError_t launch_sweep(int mode, const SweepArgs<T, TO> &a, cudaStream_t s);
 
+// FP64 3D sweep with the cell arithmetic in 64-bit integers (k_stencil_fix.cu) and its
+// blocks (= partial sums).
+template <typename TO>
+cudaError_t launch_sweep_fix(int mode, const SweepArgs<double, TO> &a, cudaStream_t s);
+long long sweep_blocks_fix(const Geom &g);
+
 // FP32 3D sweep with TMA plane staging and packed FP32x2 arithmetic, one
 // persistent CTA per SM (k_stencil_tma.cu).  tmap: three CUtensorMaps of the
 // storage that a.g's grid sits in at offset org (>= 0; zero for a whole level):

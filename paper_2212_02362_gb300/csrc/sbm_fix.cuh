@@ -1,0 +1,257 @@
+// sbm_fix.cuh — the FP64 cell arithmetic of the operator in 64-bit integers.
+//
+// GB300 issues about one FP64 instruction for every 64 integer ones, so the FP64 stencil,
+// evaluated with FP64 instructions, is bound by the FP64 pipe.  Here the same cell
+// formula (sbm_cell.cuh) is evaluated in block floating point: a 64-bit integer mantissa
+// per value and one power of two per cell.
+//
+//   1. The nodal values around a cell become integers |u| < 2^60 on a common power of
+//      two, the largest one in the staged node plane: a double keeps all of its 53 bits
+//      down to 2^-7 of that largest value.
+//   2. The mean/difference transform is exact (additions of integers).
+//   3. The cell's 21 transformed values are shifted left until the largest reaches
+//      2^60, so the products below keep the cell's own leading digits, however small
+//      its strain is beside its displacement.
+//   4. The constants psi C / h^2 are 60-bit fractions (psi as mantissa and exponent);
+//      a product keeps its upper 64 bits.  The sum of the 8 cells of a node is bounded
+//      by 2^63, so the smallest unit is 2^-57 of the largest force the cell could have.
+//   5. Forces of neighbouring cells are added after a shift to the larger of their
+//      exponents; the sum is converted to a double once per node.
+//
+// Against the formula in FP64 every rounding (2^-53 of each partial result there) is
+// replaced by one of at most 2^-55 of the cell's largest term; measured errors stand at
+// the kernels.  Values that do not fit the scheme (infinities, NaN, exponents beyond the
+// range below, negative psi) are recognised while they are staged, and the caller
+// evaluates those planes with FP64 instructions.
+#pragma once
+
+#include <math.h>
+#include <stdint.h>
+#include <string.h>
+
+#include "sbm_cell.cuh"
+
+namespace sbm {
+namespace fix {
+
+typedef long long i64;
+
+#if defined(__CUDA_ARCH__)
+__device__ __forceinline__ int mulhi_s(int a, int b) { return __mulhi(a, b); }
+__device__ __forceinline__ unsigned mulhi_u(unsigned a, unsigned b) { return __umulhi(a, b); }
+__device__ __forceinline__ int clz64(unsigned long long v) { return __clzll((long long)v); }
+__device__ __forceinline__ i64 bits_of(double v) { return __double_as_longlong(v); }
+__device__ __forceinline__ double of_bits(i64 b) { return __longlong_as_double(b); }
+#else
+inline int mulhi_s(int a, int b) { return (int)(((int64_t)a * b) >> 32); }
+inline unsigned mulhi_u(unsigned a, unsigned b) { return (unsigned)(((uint64_t)a * b) >> 32); }
+inline int clz64(unsigned long long v) { return v ? __builtin_clzll(v) : 64; }
+inline i64 bits_of(double v) { i64 b; memcpy(&b, &v, 8); return b; }
+inline double of_bits(i64 b) { double v; memcpy(&v, &b, 8); return v; }
+#endif
+
+// Biased exponents a staged value may have; with the bounds on the constants below, every
+// result is then a normal number.  Zero is allowed as well.
+constexpr int kExpLo = 600, kExpHi = 1500;
+constexpr int kNoExp = -(1 << 20);      // exponent of a cell without force
+
+// The exponent field of a value's magnitude as an ordered key: 0 for zero, key >> 20 the
+// biased exponent otherwise (a denormal, with exponent 0, gives a key of at least 1).
+__host__ __device__ __forceinline__ unsigned exp_key(double v)
+{
+    const i64 b = bits_of(v);
+    return ((unsigned)(b >> 32) & 0x7fffffffu) | ((unsigned)b != 0u ? 1u : 0u);
+}
+__host__ __device__ __forceinline__ bool key_ok(unsigned key)
+{
+    return key == 0u || (key >= ((unsigned)kExpLo << 20) && key < ((unsigned)kExpHi << 20));
+}
+
+// v as an integer on the unit 2^(E - 1023 - 59), E >= the biased exponent of v.
+__host__ __device__ __forceinline__ i64 to_fix(double v, int E)
+{
+    const i64 b = bits_of(v);
+    const int ex = (int)((unsigned)(b >> 52) & 0x7ffu);
+    const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
+    const int sh = E - ex;
+    const i64 a = sh > 63 ? 0 : (i64)((m << 7) >> sh);
+    return b < 0 ? -a : a;
+}
+constexpr int kFixUnit = 1023 + 59;     // to_fix's unit is 2^(E - kFixUnit)
+
+// a * 2^e as a double (e such that the result is normal; a may be zero).
+__host__ __device__ __forceinline__ double to_double(i64 a, int e)
+{
+    const double v = (double)a;
+    return a == 0 ? 0.0 : of_bits(bits_of(v) + ((i64)e << 52));
+}
+
+// A constant below 2^60 in two signed 32-bit parts, hi 2^32 + lo.
+struct Frac {
+    int hi, lo;
+};
+__host__ __device__ __forceinline__ Frac split(i64 k)
+{
+    Frac f;
+    f.lo = (int)(unsigned)(unsigned long long)k;
+    f.hi = (int)(k >> 32) + (f.lo < 0 ? 1 : 0);
+    return f;
+}
+
+// (a k) / 2^64 to within two units: the parts a_lo k_lo and the low halves of the cross
+// products are dropped.
+__host__ __device__ __forceinline__ i64 mul(i64 a, Frac k)
+{
+    const int ah = (int)(a >> 32);
+    const unsigned al = (unsigned)(unsigned long long)a;
+    const int s = mulhi_s(ah, k.lo) + (int)mulhi_u(al, (unsigned)k.hi);
+    return (i64)ah * k.hi + s;
+}
+
+// Moduli constants of a level, prepared on the host: 2^60-fractions of 2^ec.
+// n[]: ad, |a12|, a44, (b1 + b12)/2, (b1 - b12)/2, b44, c2 of Coef (2D: a11 - a12, |a12|,
+// a44, b1), each at most 2^61 in the stored unit; neg12: a12 < 0.
+struct Consts {
+    Frac c[7];
+    int neg12;
+    int ec;                 // value = c 2^(ec - 64) before the product with psi
+    int ok;                 // the constants fit; otherwise the FP64 kernel is used
+};
+
+// Scale: the largest row of the stress map, times the headroom of the sums that follow
+// (8 cells x 7 terms of at most 2^61 in 3D, 4 x 3 in 2D), must stay below 2^63.
+inline Consts make_consts(int dim, const Coef<double> &c)
+{
+    Consts r;
+    memset(&r, 0, sizeof(r));
+    const double a12 = fabs(c.a12);
+    double v[7], bound;
+    if (dim == 3) {
+        v[0] = c.ad; v[1] = a12; v[2] = c.a44;
+        v[3] = 0.5 * (c.b1 + c.b12); v[4] = 0.5 * (c.b1 - c.b12);
+        v[5] = c.b44; v[6] = c.c2;
+        bound = fmax(fmax(c.ad + 3.0 * a12, 2.0 * c.a44), fmax(c.b1 + fabs(c.b12), fmax(4.0 * c.b44, c.c2)));
+    } else {
+        v[0] = c.a11 - c.a12; v[1] = a12; v[2] = c.a44; v[3] = c.b1;
+        v[4] = v[5] = v[6] = 0.0;
+        bound = fmax(fmax(v[0] + 2.0 * a12, 2.0 * c.a44), c.b1);
+    }
+    r.neg12 = c.a12 < 0.0;
+    if (!(bound > ldexp(1.0, -200)) || !(bound < ldexp(1.0, 200))) return r;
+    int eb;
+    frexp(bound, &eb);                       // bound < 2^eb
+    for (int i = 0; i < 7; ++i) {
+        if (!(v[i] >= 0.0)) return r;
+        // c <= 2^61 for v = 2^eb: with psi's mantissa below 2^63 the product's upper half
+        // is below 2^60, which is 1/16 of the fraction 1
+        r.c[i] = split((i64)rint(ldexp(v[i], 61 - eb)));
+    }
+    r.ec = eb + 4;
+    r.ok = 1;
+    return r;
+}
+
+// psi the scheme takes: 0, or positive and within 2^+-200.
+__host__ __device__ __forceinline__ bool psi_ok(double psi)
+{
+    const unsigned h = (unsigned)(bits_of(psi) >> 52);      // sign and exponent
+    return psi == 0.0 || (h >= 823u && h < 1223u);
+}
+
+// psi > 0 as mantissa in [2^62, 2^63) and exponent: psi = m 2^(e - 63).
+__host__ __device__ __forceinline__ i64 psi_mantissa(double psi, int &e)
+{
+    const i64 b = bits_of(psi);
+    e = (int)((unsigned)(b >> 52) & 0x7ffu) - 1022;
+    return (i64)((((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull) << 10);
+}
+
+// The upper word of v's magnitude (less one for v < 0).
+__host__ __device__ __forceinline__ unsigned mag_hi(i64 v)
+{
+    const int h = (int)(v >> 32);
+    return (unsigned)(h ^ (h >> 31));
+}
+
+// Shift of the transformed values: all of them below 2^61 in magnitude afterwards.
+// m: the OR of their magnitudes.
+__host__ __device__ __forceinline__ int norm_shift(unsigned long long m) { return clz64(m) - 3; }
+
+__host__ __device__ __forceinline__ i64 shift_by(i64 v, int s)
+{
+    return s >= 0 ? (i64)((unsigned long long)v << s) : v >> -s;
+}
+
+__host__ __device__ __forceinline__ i64 down(i64 v, int s) { return v >> (s > 63 ? 63 : s); }
+
+// One 3D cell: in-plane transforms (bfly4xy of the integers) of its bottom and top faces
+// on the unit 2^(E - kFixUnit), its psi.  Returns the transformed face forces, the
+// unit of which is 2^e (e = kNoExp: no force, Fb = Ft = 0).
+__host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], const i64 (&Tt)[3][4], int E, double psi,
+                                                     const Consts &c, i64 (&Fb)[3][4], i64 (&Ft)[3][4], int &e)
+{
+    i64 U[3][8];
+    unsigned mh = 0;
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            U[p][s] = Tb[p][s] + Tt[p][s];
+            U[p][s + 4] = Tt[p][s] - Tb[p][s];
+            if (s > 0) mh |= mag_hi(U[p][s]);
+            mh |= mag_hi(U[p][s + 4]);
+        }
+    unsigned long long m = (unsigned long long)mh << 32 | 0xffffffffu;
+    if (mh == 0u) {                          // all below 2^32: the low words decide
+        m = 0;
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int s = 1; s < 8; ++s) m |= (unsigned long long)(U[p][s] ^ (U[p][s] >> 63));
+    }
+    int ep;
+    const i64 pm = psi_mantissa(psi, ep);
+    const int sh = norm_shift(m);
+    const bool none = m == 0ull || psi == 0.0;
+    e = none ? kNoExp : E - kFixUnit - sh + ep + c.ec;
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int s = 1; s < 8; ++s) U[p][s] = none ? 0 : shift_by(U[p][s], sh);
+    Frac k[7];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) k[i] = split(mul(pm, c.c[i]));
+    i64 ltr = mul(U[0][1] + U[1][2] + U[2][4], k[1]);
+    ltr = c.neg12 ? -ltr : ltr;
+    const i64 sxx = mul(U[0][1], k[0]) + ltr, syy = mul(U[1][2], k[0]) + ltr, szz = mul(U[2][4], k[0]) + ltr;
+    const i64 sxy = mul(U[1][1] + U[0][2], k[2]);
+    const i64 sxz = mul(U[2][1] + U[0][4], k[2]);
+    const i64 syz = mul(U[2][2] + U[1][4], k[2]);
+    const i64 S = U[2][3] + U[1][5] + U[0][6];
+    // (b1 x + b12 y, b1 y + b12 x) from the sum and the difference of x and y
+    i64 a, d;
+    a = mul(U[0][3] + U[2][6], k[3]); d = mul(U[0][3] - U[2][6], k[4]);
+    const i64 d03 = a + d, d26 = a - d;
+    a = mul(U[1][3] + U[2][5], k[3]); d = mul(U[1][3] - U[2][5], k[4]);
+    const i64 d13 = a + d, d25 = a - d;
+    a = mul(U[0][5] + U[1][6], k[3]); d = mul(U[0][5] - U[1][6], k[4]);
+    const i64 d05 = a + d, d16 = a - d;
+    const i64 d23 = mul(S + U[2][3], k[5]), d15 = mul(S + U[1][5], k[5]), d06 = mul(S + U[0][6], k[5]);
+    const i64 d07 = mul(U[0][7], k[6]), d17 = mul(U[1][7], k[6]), d27 = mul(U[2][7], k[6]);
+    const i64 dU[3][8] = {{0, sxx, sxy, d03, sxz, d05, d06, d07},
+                          {0, sxy, syy, d13, syz, d15, d16, d17},
+                          {0, sxz, syz, d23, szz, d25, d26, d27}};
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        Fb[p][0] = -dU[p][4];
+        Ft[p][0] = dU[p][4];
+#pragma unroll
+        for (int s = 1; s < 4; ++s) {
+            Fb[p][s] = dU[p][s] - dU[p][s + 4];
+            Ft[p][s] = dU[p][s] + dU[p][s + 4];
+        }
+    }
+}
+
+}  // namespace fix
+}  // namespace sbm

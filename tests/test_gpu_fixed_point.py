@@ -1,0 +1,94 @@
+"""The FP64 3D sweep in integer arithmetic (k_sweep3_fix) against the oracle where its
+tiles, its plane ring and its hand-over to FP64 instructions can go wrong."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+from _sbm import cuda, gpu_grid, host, oracle_problem, random_workload
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2212_02362_gb300 import build
+    build.build()
+    oracle.build()
+
+
+def _rel(a, b):
+    return np.abs(a - b).max() / np.abs(b).max()
+
+
+# one tile holds 32 x 10 cells: one cell, exactly a tile, a tile and a remainder of one
+# cell on either axis, one plane per block and long segments
+@pytest.mark.parametrize("n", [(2, 2, 2), (3, 2, 17), (33, 11, 2), (34, 12, 3), (33, 11, 15), (66, 12, 6), (9, 31, 33)])
+def test_tile_edges(n):
+    wk = random_workload(3, n, 90)
+    g, P = gpu_grid(wk), oracle_problem(wk)
+    u = wk.u0 + W.uniform(91, P.ndofs, -1e-2, 1e-2) * ~oracle.dirichlet_mask(P)
+    psi = oracle.floor_psi(wk.psi, wk.psi_min)
+    assert _rel(host(g.apply(g.finest, cuda(u))), oracle.apply(P, psi, u)) <= 1e-13
+    r, nrm = g.residual(g.finest, cuda(wk.f), cuda(u))
+    ref = oracle.residual(P, psi, wk.f, u)
+    assert _rel(host(r), ref) <= 1e-13 and np.isclose(nrm, oracle.norm_free(P, ref), rtol=1e-13)
+    got = host(g.smooth(g.finest, cuda(wk.f), cuda(u), "jacobi", 0.6))
+    assert _rel(got - u, oracle.jacobi_sweep(P, psi, wk.f, u, 0.6) - u) <= 1e-12
+
+
+@pytest.mark.parametrize("scale", [1e-200, 1e-130, 1e-100, 1.0, 1e140, 1e150])
+def test_magnitudes(scale):
+    """In and beyond the range of the integer form (2^-423 to 2^477)."""
+    wk = random_workload(3, (35, 13, 12), 92)
+    g, P = gpu_grid(wk), oracle_problem(wk)
+    u = scale * W.uniform(93, P.ndofs, -1, 1)
+    assert _rel(host(g.apply(g.finest, cuda(u))) / scale, oracle.apply(P, oracle.floor_psi(wk.psi, wk.psi_min), u) / scale) <= 1e-13
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan, 1e250, 1e-250])
+@pytest.mark.parametrize("plane", [0, 9, 20])
+def test_planes_that_do_not_fit(value, plane):
+    """One node's value sends the rest of its block's planes to FP64 instructions: every
+    other value is as before, and the neighbourhood of a NaN or infinity is not finite."""
+    wk = random_workload(3, (35, 13, 21), 94)
+    g, P = gpu_grid(wk), oracle_problem(wk)
+    u = W.uniform(95, P.ndofs, -1, 1)
+    v = u.reshape(3, 21, 13, 35)
+    if value == 1e-250:
+        v[:, plane] = 0.0
+    v[1, plane, 6, 17] = value
+    with np.errstate(invalid="ignore", over="ignore"):
+        ref = oracle.apply(P, oracle.floor_psi(wk.psi, wk.psi_min), u)
+    got = host(g.apply(g.finest, cuda(u)))
+    fin = np.isfinite(ref)
+    assert np.array_equal(fin, np.isfinite(got))
+    fin &= np.abs(ref) < 1e10
+    assert fin.sum() > 20000 and np.abs(got - ref)[fin].max() <= 1e-12 * np.abs(ref[fin]).max()
+
+
+def test_planes_of_different_size():
+    """Each plane has its own unit: neighbouring planes nine decades apart."""
+    wk = random_workload(3, (37, 13, 31), 96)
+    g, P = gpu_grid(wk), oracle_problem(wk)
+    u = W.uniform(97, P.ndofs, -1, 1).reshape(3, 31, 13, 37)
+    u *= (10.0 ** np.array([0, -9, -3, 0, 6, 6, -2, 0, 0, 3] * 3 + [0]))[None, :, None, None]
+    ref = oracle.apply(P, oracle.floor_psi(wk.psi, wk.psi_min), u.reshape(-1)).reshape(3, 31, -1)
+    got = host(g.apply(g.finest, cuda(u.reshape(-1)))).reshape(3, 31, -1)
+    big = np.abs(ref).max(axis=(0, 2))
+    near = np.maximum(big, np.maximum(np.roll(big, 1), np.roll(big, -1)))
+    assert np.all(np.abs(got - ref).max(axis=(0, 2)) <= 1e-13 * near)
+
+
+def test_zero_psi_and_wide_psi():
+    """Cells without force beside cells of full stiffness, psi over eight decades."""
+    wk = random_workload(3, (35, 13, 11), 98, psi_lo=1e-8)
+    wk.psi = 10.0 ** W.uniform(99, wk.ncells, -8, 0)
+    g, P = gpu_grid(wk), oracle_problem(wk)
+    u = W.uniform(100, P.ndofs, -1, 1)
+    assert _rel(host(g.apply(g.finest, cuda(u))), oracle.apply(P, oracle.floor_psi(wk.psi, 1e-8), u)) <= 1e-13
+    assert np.all(host(g.apply(g.finest, cuda(np.repeat([0.3, -0.7, 1.1], P.nnodes)))) == 0.0)
