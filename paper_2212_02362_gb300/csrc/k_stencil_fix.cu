@@ -10,15 +10,17 @@
 // Work split.  A block owns a tile of 32 x 10 cells in x/y (33 x 11 threads, one per cell
 // column with the halo column and row; 12 warps, so 168 registers a thread) and a
 // contiguous range of (tile, node plane) units, which it streams along z, one cell layer
-// a step.  Node planes pass through a four-slot shared-memory ring in three stages, so
-// that nothing inside a step waits for global memory and two barriers a step suffice:
-//   plane lz+3  copied by cp.async while step lz computes; at the step's end each thread
-//               takes the largest exponent of the values it copied into the plane's key
-//   plane lz+2  turned into integers in place, each thread the values it copied
-//   plane lz+1  read by the cells of layer lz
+// a step.  Node planes pass through a four-slot shared-memory ring in four stages, so
+// that nothing inside a step waits for global memory and one barrier a step suffices.  In
+// step lz
+//   plane lz+4  is copied by cp.async (into the slot that plane lz left in step lz - 1)
+//   plane lz+3  has arrived: each thread takes the largest exponent of the values it
+//               copied into the plane's key
+//   plane lz+2  is turned into integers in place, each thread the values it copied
+//   plane lz+1  is read by the cells of layer lz
 // The forces a layer sends to its top plane are carried in registers in the transformed
 // basis with their exponent; those of the four columns around a node are exchanged
-// through shared memory with the exponents beside them.
+// through a double-buffered shared array with the exponents beside them.
 //
 // A plane or a psi that the integer form does not take (sbm_fix.cuh) ends the integer
 // loop before any node that depends on it; the block finishes its range with the FP64
@@ -38,9 +40,9 @@ using fix::i64;
 constexpr int TX = 32, TY = 10;                   // cells of a tile
 constexpr int BX = TX + 1, BY = TY + 1, NT = BX * BY;
 constexpr int PX = TX + 2, PY = TY + 2, PP = PX * PY;
-// ring of node planes (4 x 3 components), exchanged forces (12 for the FP64 body, 9 and
-// an exponent here), psi of the cells below + above
-constexpr size_t kSmem = sizeof(double) * (12 + 12 + 1) * PP + sizeof(int) * PP;
+// ring of node planes (4 x 3 components); two buffers of 9 exchanged forces, psi of the
+// cells below + above and the exponent (the FP64 body: 12 forces and psi)
+constexpr size_t kSmem = sizeof(double) * (12 + 2 * (9 + 1)) * PP + 2 * sizeof(int) * PP;
 
 // 8-byte global -> shared copy; ok = false fills zeros (src must still be valid).
 __device__ __forceinline__ void cp_async8(void *sdst, const void *gsrc, bool ok)
@@ -86,17 +88,35 @@ __device__ __forceinline__ Tile make_tile(const Geom &g, int t, int ntx, int tx,
     return T;
 }
 
-// Node plane k of a tile into the shared array dst[3][PP] (zeros outside the grid).
-__device__ __forceinline__ void load_plane(const double *u, const Geom &g, const Tile &T, int k, double *dst)
+// The staged nodes of this thread (tid and, for the first few threads, tid + NT): their
+// offset within a plane, -1 outside the grid.
+struct Stage {
+    int o0, o1;
+};
+
+__device__ __forceinline__ Stage make_stage(const Geom &g, const Tile &T)
 {
-    for (int s = threadIdx.x; s < PP; s += NT) {
-        const int lx = s % PX, ly = s / PX;
-        const int gx = T.x0 - 1 + lx, gy = T.y0 - 1 + ly;
-        const bool ok = gx >= 0 && gx < g.nx && gy >= 0 && gy < g.ny && k >= 0 && k < g.nz;
-        const long long o = ok ? gidx(g, gx, gy, k) : 0;
+    auto off = [&](int s) {
+        const int gx = T.x0 - 1 + s % PX, gy = T.y0 - 1 + s / PX;
+        return (s < PP && gx >= 0 && gx < g.nx && gy >= 0 && gy < g.ny) ? gx + g.sx * gy : -1;
+    };
+    return {off(threadIdx.x), off(threadIdx.x + NT)};
+}
+static_assert(PP <= 2 * NT, "two staged nodes a thread at most");
+
+// Node plane k of a tile into the shared array dst[3][PP] (zeros outside the grid).
+__device__ __forceinline__ void load_plane(const double *u, const Geom &g, const Stage &S, int k, double *dst)
+{
+    const bool in = k >= 0 && k < g.nz;
+    const double *pl = u + (in ? g.sy * k : 0);
+    auto node = [&](int o, int s) {
+        const bool ok = in && o >= 0;
+        const double *q = ok ? pl + o : u;
 #pragma unroll
-        for (int p = 0; p < 3; ++p) cp_async8(dst + p * PP + s, u + (ok ? p * g.cs + o : 0), ok);
-    }
+        for (int p = 0; p < 3; ++p) cp_async8(dst + p * PP + s, q + (ok ? p * g.cs : 0), ok);
+    };
+    node(S.o0, threadIdx.x);
+    if (threadIdx.x + NT < PP) node(S.o1, threadIdx.x + NT);
     cp_async_commit();
 }
 
@@ -111,6 +131,7 @@ __device__ __noinline__ double sweep_dp(const SweepArgs<double, TO> &a, long lon
     const int tid = threadIdx.x;
     int tx, ty;
     row_warp_xy<BY>(tid, tx, ty);
+    cp_async_wait_all();
     __syncthreads();
     for (int s = tid; s < PP; s += NT) {
         const int lx = s % PX, ly = s / PX;
@@ -125,6 +146,7 @@ __device__ __noinline__ double sweep_dp(const SweepArgs<double, TO> &a, long lon
         const int kz0 = (int)(su % g.nz);
         const int kend = (int)min((long long)g.nz, kz0 + (ue - su)) - 1;   // last node plane finalised
         const Tile T = make_tile(g, (int)(su / g.nz), ntx, tx, ty);
+        const Stage S = make_stage(g, T);
         su += kend + 1 - kz0;
         const int kfirst = kz0 > 0 ? kz0 - 1 : 0;
         const int me = ty * PX + tx;
@@ -149,13 +171,13 @@ __device__ __noinline__ double sweep_dp(const SweepArgs<double, TO> &a, long lon
             for (int s = 0; s < 4; ++s) Cf[p][s] = 0.0;
         double psi_prev = 0.0;
         double psi = cell_psi(kfirst);
-        load_plane(a.u, g, T, kfirst, up + (kfirst % 3) * 3 * PP);
-        load_plane(a.u, g, T, kfirst + 1, up + ((kfirst + 1) % 3) * 3 * PP);
+        load_plane(a.u, g, S, kfirst, up + (kfirst % 3) * 3 * PP);
+        load_plane(a.u, g, S, kfirst + 1, up + ((kfirst + 1) % 3) * 3 * PP);
         cp_async_wait_all();
         __syncthreads();
         corners(kfirst, Tb);
         for (int lz = kfirst; lz <= kend; ++lz) {
-            load_plane(a.u, g, T, lz + 2, up + ((lz + 2) % 3) * 3 * PP);   // slot of plane lz - 1
+            load_plane(a.u, g, S, lz + 2, up + ((lz + 2) % 3) * 3 * PP);   // slot of plane lz - 1
             const double psi_next = cell_psi(lz + 1);
             const bool fin = T.own && lz >= kz0;
             double fv[3];
@@ -207,9 +229,9 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
     if (a.gate && *a.gate) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *up = reinterpret_cast<double *>(smem_raw);        // [4][3][PP]: doubles, then integers
-    i64 *X = reinterpret_cast<i64 *>(up + 12 * PP);            // [9][PP]: corner forces 0..2 of a plane
-    double *ps = up + 24 * PP;                                 // [PP]
-    int *Xe = reinterpret_cast<int *>(ps + PP);                // [PP]: their exponents
+    i64 *X2 = reinterpret_cast<i64 *>(up + 12 * PP);           // [2][9][PP]: corner forces 0..2 of a plane
+    double *ps2 = up + 30 * PP;                                // [2][PP]
+    int *Xe2 = reinterpret_cast<int *>(ps2 + 2 * PP);          // [2][PP]: exponents of the forces
     __shared__ double red[((NT + 31) / 32) * 32];
     __shared__ unsigned keys[4];
 
@@ -220,9 +242,9 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
     for (int s = tid; s < PP; s += NT) {
         const int lx = s % PX, ly = s / PX;
         if (lx == BX || ly == BY) {                            // no cells there
-            for (int q = 0; q < 9; ++q) X[q * PP + s] = 0;
-            Xe[s] = fix::kNoExp;
-            ps[s] = 0.0;
+            for (int q = 0; q < 18; ++q) X2[q * PP + s] = 0;
+            Xe2[s] = Xe2[PP + s] = fix::kNoExp;
+            ps2[s] = ps2[PP + s] = 0.0;
         }
     }
     const int ntx = (g.nx - 1 + TX - 1) / TX, nty = (g.ny - 1 + TY - 1) / TY;
@@ -230,6 +252,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
     const long long ub = U * blockIdx.x / gridDim.x, ue = U * (blockIdx.x + 1) / gridDim.x;
     const int me = ty * PX + tx;
     double ssq = 0.0;
+    int buf = 0;
     long long rest = fc.ok ? ue : ub;          // units from here on are left to the FP64 body
 
     auto slot = [&](int k) { return up + (k & 3) * 3 * PP; };
@@ -237,9 +260,11 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
     auto take_key = [&](int k) {
         const double *pl = slot(k);
         unsigned m = 0;
-        for (int s = tid; s < PP; s += NT)
 #pragma unroll
-            for (int p = 0; p < 3; ++p) m = max(m, fix::exp_key(pl[p * PP + s]));
+        for (int p = 0; p < 3; ++p) m = max(m, fix::exp_key(pl[p * PP + tid]));
+        if (tid + NT < PP)
+#pragma unroll
+            for (int p = 0; p < 3; ++p) m = max(m, fix::exp_key(pl[p * PP + tid + NT]));
         const unsigned w = (tid | 31) < NT ? 0xffffffffu : (1u << (NT & 31)) - 1u;   // the last warp is partial
         m = __reduce_max_sync(w, m);
         if ((tid & 31) == 0) atomicMax(&keys[k & 3], m);
@@ -248,12 +273,12 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
     auto to_ints = [&](int k) {
         double *pl = slot(k);
         const int E = exp_of(k);
-        for (int s = tid; s < PP; s += NT)
 #pragma unroll
-            for (int p = 0; p < 3; ++p) {
-                const i64 v = fix::to_fix(pl[p * PP + s], E);
-                pl[p * PP + s] = fix::of_bits(v);
-            }
+        for (int p = 0; p < 3; ++p) pl[p * PP + tid] = fix::of_bits(fix::to_fix(pl[p * PP + tid], E));
+        if (tid + NT < PP)
+#pragma unroll
+            for (int p = 0; p < 3; ++p)
+                pl[p * PP + tid + NT] = fix::of_bits(fix::to_fix(pl[p * PP + tid + NT], E));
     };
     auto corners = [&](int k, i64 (&C)[3][4]) {
         const i64 *pl = reinterpret_cast<const i64 *>(slot(k));
@@ -277,12 +302,14 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
         auto cell_psi = [&](int lz) {
             return (T.cell_ok && lz <= g.nz - 2) ? a.psi[gidx(g, T.gx - 1, T.gy - 1, lz)] : 0.0;
         };
-        // planes kfirst, kfirst + 1 as integers, kfirst + 2 with its key
-        for (int k = kfirst; k < kfirst + 3; ++k) load_plane(a.u, g, T, k, slot(k));
+        const Stage S = make_stage(g, T);
+        // planes kfirst, kfirst + 1 as integers, kfirst + 2 with its key, kfirst + 3 on its way
+        for (int k = kfirst; k < kfirst + 3; ++k) load_plane(a.u, g, S, k, slot(k));
         if (tid < 4) keys[tid] = 0u;
         double psi = cell_psi(kfirst), psi_prev = 0.0;
         cp_async_wait_all();
         __syncthreads();
+        load_plane(a.u, g, S, kfirst + 3, slot(kfirst + 3));
         for (int k = kfirst; k < kfirst + 3; ++k) take_key(k);
         bool bad = __syncthreads_or(!fix::psi_ok(psi));
         for (int k = kfirst; k < kfirst + 3; ++k) bad = bad || !fix::key_ok(keys[k & 3]);
@@ -300,13 +327,20 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
         for (int p = 0; p < 3; ++p)
 #pragma unroll
             for (int q = 0; q < 4; ++q) Cf[p][q] = 0;
+        __syncthreads();                                       // plane kfirst's slot is free
 #pragma unroll 1
         for (int lz = kfirst; lz <= kend; ++lz) {
             if (!fix::key_ok(keys[(lz + 2) & 3])) {            // the same for the whole block
                 rest = seg + max(lz, kz0);
                 break;
             }
-            load_plane(a.u, g, T, lz + 3, slot(lz + 3));       // slot of plane lz - 1
+            cp_async_wait_all();                               // plane lz + 3 in this thread's copies
+            take_key(lz + 3);
+            load_plane(a.u, g, S, lz + 4, slot(lz + 4));
+            if (tid == 0) keys[lz & 3] = 0u;                   // for plane lz + 4
+            i64 *X = X2 + buf * 9 * PP;
+            int *Xe = Xe2 + buf * PP;
+            double *ps = ps2 + buf * PP;
             const double psi_next = cell_psi(lz + 1);
             const bool fin = T.own && lz >= kz0;
             double fv[3], uv[3];
@@ -361,8 +395,8 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
             if (MODE == kJacobi) ps[me] = psi_prev + psi;
             psi_prev = psi;
             psi = psi_next;
-            __syncthreads();
-            if (tid == 0) keys[lz & 3] = 0u;                   // for plane lz + 4
+            const int bad_next = __syncthreads_or(!fix::psi_ok(psi));
+            buf ^= 1;
             if (fin) {
                 const int e1 = Xe[me + 1], e2 = Xe[me + PX], e3 = Xe[me + PX + 1];
                 const int ee = max(max(en, e1), max(e2, e3));
@@ -379,9 +413,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
                 if (MODE == kJacobi) pss = (ps[me] + ps[me + 1]) + (ps[me + PX] + ps[me + PX + 1]);
                 body::finalize_f<double, TO, MODE>(a, T.gx, T.gy, lz, Ku, pss, uv, fv, ssq);
             }
-            cp_async_wait_all();                               // plane lz + 3 in this thread's copies
-            take_key(lz + 3);
-            if (__syncthreads_or(!fix::psi_ok(psi)) && lz < kend) {
+            if (bad_next && lz < kend) {
                 rest = seg + max(lz + 1, kz0);
                 break;
             }

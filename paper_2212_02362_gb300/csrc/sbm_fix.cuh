@@ -158,12 +158,12 @@ __host__ __device__ __forceinline__ bool psi_ok(double psi)
     return psi == 0.0 || (h >= 823u && h < 1223u);
 }
 
-// psi > 0 as mantissa in [2^62, 2^63) and exponent: psi = m 2^(e - 63).
+// psi > 0 as mantissa in [2^62, 2^63) and exponent: psi = m 2^(e - 63); mantissa 0 for 0.
 __host__ __device__ __forceinline__ i64 psi_mantissa(double psi, int &e)
 {
     const i64 b = bits_of(psi);
     e = (int)((unsigned)(b >> 52) & 0x7ffu) - 1022;
-    return (i64)((((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull) << 10);
+    return b == 0 ? 0 : (i64)((((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull) << 10);
 }
 
 // The upper word of v's magnitude (less one for v < 0).
@@ -176,11 +176,6 @@ __host__ __device__ __forceinline__ unsigned mag_hi(i64 v)
 // Shift of the transformed values: all of them below 2^61 in magnitude afterwards.
 // m: the OR of their magnitudes.
 __host__ __device__ __forceinline__ int norm_shift(unsigned long long m) { return clz64(m) - 3; }
-
-__host__ __device__ __forceinline__ i64 shift_by(i64 v, int s)
-{
-    return s >= 0 ? (i64)((unsigned long long)v << s) : v >> -s;
-}
 
 __host__ __device__ __forceinline__ i64 down(i64 v, int s) { return v >> (s > 63 ? 63 : s); }
 
@@ -211,13 +206,19 @@ __host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], cons
     }
     int ep;
     const i64 pm = psi_mantissa(psi, ep);
-    const int sh = norm_shift(m);
-    const bool none = m == 0ull || psi == 0.0;
-    e = none ? kNoExp : E - kFixUnit - sh + ep + c.ec;
+    int sh = norm_shift(m);
+    e = (m == 0ull || pm == 0) ? kNoExp : E - kFixUnit - sh + ep + c.ec;
+    if (sh < 0) {                            // sums of opposite corners near the bound
+        sh += 3;
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int s = 1; s < 8; ++s) U[p][s] >>= 3;
+    }
 #pragma unroll
     for (int p = 0; p < 3; ++p)
 #pragma unroll
-        for (int s = 1; s < 8; ++s) U[p][s] = none ? 0 : shift_by(U[p][s], sh);
+        for (int s = 1; s < 8; ++s) U[p][s] = (i64)((unsigned long long)U[p][s] << (sh & 63));
     Frac k[7];
 #pragma unroll
     for (int i = 0; i < 7; ++i) k[i] = split(mul(pm, c.c[i]));
