@@ -425,7 +425,7 @@ void sweep_grid(const Geom &g, int *grid, int *kchunk)
 
 long long sweep_blocks(const Geom &g, bool fp64)
 {
-    if (fp64 && g.dim == 3) return sweep_blocks_fix(g);
+    if (fp64) return sweep_blocks_fix(g);
     int grid[3], ch;
     sweep_grid(g, grid, &ch);
     return (long long)grid[0] * grid[1] * grid[2];
@@ -489,24 +489,22 @@ cudaError_t launch_sweep_node(int mode, const SweepArgs<float, float> &a, cudaSt
     return cudaGetLastError();
 }
 
-template <typename T, typename TO, int MODE>
-static cudaError_t launch_mode(const SweepArgs<T, TO> &a0, cudaStream_t s)
+template <int MODE>
+static cudaError_t launch_mode(const SweepArgs<float, float> &a0, cudaStream_t s)
 {
-    SweepArgs<T, TO> a = a0;
+    SweepArgs<float, float> a = a0;
     int grid[3];
     sweep_grid(a.g, grid, &a.kchunk);
     if (a.g.dim == 3) {
-        if constexpr (sizeof(T) == 4) {            // FP64: launch_sweep_fix
-            const size_t sm = smem3<T>();
-            static std::atomic<unsigned long long> attr_done{0};
-            cudaError_t ea = smem_attr_once(reinterpret_cast<const void *>(k_sweep3<T, TO, MODE>), sm, attr_done);
-            if (ea != cudaSuccess) return ea;
-            cudaError_t e = launch_pdl(k_sweep3<T, TO, MODE>, dim3(grid[0], grid[1], grid[2]), dim3(TX3 + 1, TY3 + 1), sm,
-                                       s, a);
-            if (e != cudaSuccess) return e;
-        }
+        const size_t sm = smem3<float>();
+        static std::atomic<unsigned long long> attr_done{0};
+        cudaError_t ea = smem_attr_once(reinterpret_cast<const void *>(k_sweep3<float, float, MODE>), sm, attr_done);
+        if (ea != cudaSuccess) return ea;
+        cudaError_t e = launch_pdl(k_sweep3<float, float, MODE>, dim3(grid[0], grid[1], grid[2]), dim3(TX3 + 1, TY3 + 1), sm,
+                                   s, a);
+        if (e != cudaSuccess) return e;
     } else {
-        cudaError_t e = launch_pdl(k_sweep2<T, TO, MODE>, dim3(grid[0], grid[1], 1), dim3(TX2 + 1, TY2 + 1), 0, s, a);
+        cudaError_t e = launch_pdl(k_sweep2<float, float, MODE>, dim3(grid[0], grid[1], 1), dim3(TX2 + 1, TY2 + 1), 0, s, a);
         if (e != cudaSuccess) return e;
     }
     ++g_launches;
@@ -516,13 +514,15 @@ static cudaError_t launch_mode(const SweepArgs<T, TO> &a0, cudaStream_t s)
 template <typename T, typename TO>
 cudaError_t launch_sweep(int mode, const SweepArgs<T, TO> &a, cudaStream_t s)
 {
-    if constexpr (sizeof(T) == 8)
-        if (a.g.dim == 3) return launch_sweep_fix<TO>(mode, a, s);
-    switch (mode) {
-    case kApply: return launch_mode<T, TO, kApply>(a, s);
-    case kResidual: return launch_mode<T, TO, kResidual>(a, s);
-    case kJacobi: return launch_mode<T, TO, kJacobi>(a, s);
-    default: return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 8) {
+        return launch_sweep_fix<TO>(mode, a, s);
+    } else {
+        switch (mode) {
+        case kApply: return launch_mode<kApply>(a, s);
+        case kResidual: return launch_mode<kResidual>(a, s);
+        case kJacobi: return launch_mode<kJacobi>(a, s);
+        default: return cudaErrorInvalidValue;
+        }
     }
 }
 
@@ -550,25 +550,29 @@ cudaError_t launch_gs(const Geom &g, const T *psi, const T *Ke, const T *f, T *u
 }
 
 template <typename T>
-cudaError_t launch_gs2_sweep(const Geom &g, const T *psi, const T *Ke, const T *f, const T *uin, T *uout,
+cudaError_t launch_gs2_sweep(const Geom &g, const Coef<T> &c, const T *psi, const T *Ke, const T *f, const T *uin, T *uout,
                              int descending, cudaStream_t s, const int *gate)
 {
     if (g.dim != 2 || uin == uout) return cudaErrorInvalidValue;
-    const size_t sm = smem_gs2<T>();
-    static std::atomic<unsigned long long> attr_done{0};
-    cudaError_t ea = smem_attr_once(reinterpret_cast<const void *>(k_gs2_tile<T>), sm, attr_done);
-    if (ea != cudaSuccess) return ea;
-    dim3 gr((g.nx + GST - 1) / GST, (g.ny + GST - 1) / GST, 1);
-    cudaError_t e = launch_pdl(k_gs2_tile<T>, gr, dim3(kGsThreads), sm, s, g, psi, Ke, f, uin, uout, descending, gate);
-    if (e != cudaSuccess) return e;
-    ++g_launches;
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 8) {
+        return launch_gs2_fix(g, c, psi, Ke, f, uin, uout, descending, s, gate);
+    } else {
+        const size_t sm = smem_gs2<T>();
+        static std::atomic<unsigned long long> attr_done{0};
+        cudaError_t ea = smem_attr_once(reinterpret_cast<const void *>(k_gs2_tile<T>), sm, attr_done);
+        if (ea != cudaSuccess) return ea;
+        dim3 gr((g.nx + GST - 1) / GST, (g.ny + GST - 1) / GST, 1);
+        cudaError_t e = launch_pdl(k_gs2_tile<T>, gr, dim3(kGsThreads), sm, s, g, psi, Ke, f, uin, uout, descending, gate);
+        if (e != cudaSuccess) return e;
+        ++g_launches;
+        return cudaGetLastError();
+    }
 }
 
-template cudaError_t launch_gs2_sweep<double>(const Geom &, const double *, const double *, const double *,
-                                              const double *, double *, int, cudaStream_t, const int *);
-template cudaError_t launch_gs2_sweep<float>(const Geom &, const float *, const float *, const float *,
-                                             const float *, float *, int, cudaStream_t, const int *);
+template cudaError_t launch_gs2_sweep<double>(const Geom &, const Coef<double> &, const double *, const double *,
+                                              const double *, const double *, double *, int, cudaStream_t, const int *);
+template cudaError_t launch_gs2_sweep<float>(const Geom &, const Coef<float> &, const float *, const float *,
+                                             const float *, const float *, float *, int, cudaStream_t, const int *);
 
 template cudaError_t launch_gs<double>(const Geom &, const double *, const double *, const double *, double *, int, cudaStream_t,
                                        const int *);

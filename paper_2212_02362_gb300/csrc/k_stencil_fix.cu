@@ -1,7 +1,7 @@
-// k_stencil_fix.cu — FP64 3D apply / residual / damped-Jacobi sweep with the cell
-// arithmetic in 64-bit integers (sbm_fix.cuh).
+// k_stencil_fix.cu — FP64 apply / residual / damped-Jacobi sweep and the 2D FP64 colour
+// Gauss-Seidel sweep with the cell arithmetic in 64-bit integers (sbm_fix.cuh).
 //
-// What bounds it.  With FP64 instructions this sweep is bound by their issue rate (about
+// What bounds it (3D).  With FP64 instructions the sweep is bound by their issue rate (about
 // two lanes per SM and clock on GB300): some 180 of them per cell.  In block floating
 // point the same cell takes about 800 integer instructions, which issue 64 times as
 // fast, and leaves some ten FP64 instructions per node (the conversion of the node's
@@ -53,19 +53,20 @@ __device__ __forceinline__ void cp_async8(void *sdst, const void *gsrc, bool ok)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-// Deterministic block reduction of ssq into part[block].
-__device__ __forceinline__ void block_partial(double ssq, double *part, double *red)
+// Deterministic block reduction of ssq into *out.
+template <int N>
+__device__ __forceinline__ void block_partial(double ssq, double *out, double *red)
 {
-    constexpr int NW = (NT + 31) / 32;
+    constexpr int NW = (N + 31) / 32;
     const int tid = threadIdx.x;
     red[tid] = ssq;
-    if (tid < NW * 32 - NT) red[NT + tid] = 0.0;
+    if (tid < NW * 32 - N) red[N + tid] = 0.0;
     __syncthreads();
     if (tid < 32) {
         double s = 0.0;
         for (int w = 0; w < NW; ++w) s += red[w * 32 + tid];
         for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-        if (tid == 0) part[blockIdx.x] = s;
+        if (tid == 0) *out = s;
     }
 }
 
@@ -212,8 +213,8 @@ __device__ __noinline__ double sweep_dp(const SweepArgs<double, TO> &a, long lon
                             (fc[(p * 4 + 1) * PP + me + PX] + fc[(p * 4 + 0) * PP + me + PX + 1]);
                     uv[p] = pl[p * PP + me + PX + 1];
                 }
-                const double pss = (ps[me] + ps[me + 1]) + (ps[me + PX] + ps[me + PX + 1]);
-                body::finalize_f<double, TO, MODE>(a, T.gx, T.gy, lz, Ku, pss, uv, fv, ssq);
+                const double ip = MODE == kJacobi ? 1.0 / ((ps[me] + ps[me + 1]) + (ps[me + PX] + ps[me + PX + 1])) : 0.0;
+                body::finalize_f<double, TO, MODE>(a, T.gx, T.gy, lz, Ku, ip, uv, fv, ssq);
             }
             cp_async_wait_all();                              // plane lz + 2 in this thread's copies
             __syncthreads();
@@ -350,6 +351,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
                 fv[p] = (MODE != kApply && fin) ? a.f[p * g.cs + on] : 0.0;
                 uv[p] = (MODE == kJacobi && fin) ? a.u[p * g.cs + on] : 0.0;
             }
+            double ip = (MODE == kJacobi && a.dinv && fin) ? a.dinv[on] : 0.0;
             to_ints(lz + 2);
             // the cell of layer lz, both faces on the larger of their planes' units
             const int Et = exp_of(lz + 1);
@@ -392,7 +394,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
             }
             Xe[me] = en;
             ecf = e;
-            if (MODE == kJacobi) ps[me] = psi_prev + psi;
+            if (MODE == kJacobi && !a.dinv) ps[me] = psi_prev + psi;
             psi_prev = psi;
             psi = psi_next;
             const int bad_next = __syncthreads_or(!fix::psi_ok(psi));
@@ -409,9 +411,9 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
                                    fix::down(X[(p * 3 + 0) * PP + me + PX + 1], d3));
                     Ku[p] = fix::to_double(s, ee);
                 }
-                double pss = 0.0;
-                if (MODE == kJacobi) pss = (ps[me] + ps[me + 1]) + (ps[me + PX] + ps[me + PX + 1]);
-                body::finalize_f<double, TO, MODE>(a, T.gx, T.gy, lz, Ku, pss, uv, fv, ssq);
+                if (MODE == kJacobi && !a.dinv)
+                    ip = 1.0 / ((ps[me] + ps[me + 1]) + (ps[me + PX] + ps[me + PX + 1]));
+                body::finalize_f<double, TO, MODE>(a, T.gx, T.gy, lz, Ku, ip, uv, fv, ssq);
             }
             if (bad_next && lz < kend) {
                 rest = seg + max(lz + 1, kz0);
@@ -422,18 +424,311 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
     if (rest < ue) ssq += sweep_dp<TO, MODE>(a, rest, ue, up);
     if (MODE == kResidual && a.part) {
         __syncthreads();
-        block_partial(ssq, a.part, red);
+        block_partial<NT>(ssq, a.part + blockIdx.x, red);
     }
+}
+
+// ------------------------------------------------------------------------- 2D
+//
+// One thread per cell of a 32 x TY2 tile (the first row and column the halo), which
+// turns its own four corners into integers on their largest exponent: no staging and no
+// block-wide unit, one barrier for the exchange of the corner forces.  A block with a
+// value that does not fit evaluates its cells with FP64 instructions.  What is left is
+// latency (one round of loads, one barrier), so small grids take the flat tile, which
+// spreads the FP64 instructions of the update over twice as many SMs.
+constexpr int TX2 = 32;
+
+template <typename TO, int MODE, int TY2>
+__global__ void __launch_bounds__((TX2 + 1) * (TY2 + 1)) k_sweep2_fix(const SweepArgs<double, TO> a, const fix::Consts fc)
+{
+    pdl_begin();
+    if (a.gate && *a.gate) return;
+    constexpr int BX2 = TX2 + 1, BY2 = TY2 + 1, NT2 = BX2 * BY2, PX2 = TX2 + 2, PP2 = PX2 * (TY2 + 2);
+    __shared__ i64 X[2][4][PP2];                   // corner forces (integers, or doubles where they do not fit)
+    __shared__ int Xe[PP2];
+    __shared__ double ps[PP2];
+    __shared__ double red[((NT2 + 31) / 32) * 32];
+    const Geom &g = a.g;
+    const int tid = threadIdx.x;
+    int tx, ty;
+    row_warp_xy<BY2>(tid, tx, ty);
+    for (int s = tid; s < PP2; s += NT2) {
+        if (s % PX2 == BX2 || s / PX2 == BY2) {
+            for (int q = 0; q < 8; ++q) (&X[0][0][0])[q * PP2 + s] = 0;
+            Xe[s] = fix::kNoExp;
+            ps[s] = 0.0;
+        }
+    }
+    const int gx = blockIdx.x * TX2 + tx, gy = blockIdx.y * TY2 + ty;
+    const bool own = gx < g.nx && gy < g.ny && (tx < TX2 || gx == g.nx - 1) && (ty < TY2 || gy == g.ny - 1);
+    const bool cell_ok = gx >= 1 && gx < g.nx && gy >= 1 && gy < g.ny;
+    const long long on = gidx(g, gx, gy, 0);
+    double D[2][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = gx - 1 + (q & 1), j = gy - 1 + (q >> 1);
+        const bool ok = i >= 0 && i < g.nx && j >= 0 && j < g.ny;
+        const long long o = ok ? gidx(g, i, j, 0) : 0;
+#pragma unroll
+        for (int p = 0; p < 2; ++p) D[p][q] = ok ? a.u[p * g.cs + o] : 0.0;
+    }
+    const double psi = cell_ok ? a.psi[gidx(g, gx - 1, gy - 1, 0)] : 0.0;
+    double fv[2] = {0.0, 0.0};
+    if (MODE != kApply && own) {
+        fv[0] = a.f[on];
+        fv[1] = a.f[g.cs + on];
+    }
+    double ip = (MODE == kJacobi && a.dinv && own) ? a.dinv[on] : 0.0;
+    const double uv[2] = {D[0][3], D[1][3]};
+    const int me = ty * PX2 + tx;
+    unsigned key = 0;
+    i64 I[2][4], F[2][4];
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) key = max(key, fix::exp_key(D[p][q]));
+    const bool ok = fc.ok && fix::key_ok(key) && fix::psi_ok(psi);
+    const int E = max((int)(key >> 20), fix::kExpLo);
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) I[p][q] = fix::to_fix(D[p][q], E);
+    int e;
+    fix::cell_forces2(I, E, psi, fc, F, e);
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) X[p][q][me] = F[p][q];
+    Xe[me] = e;
+    ps[me] = psi;
+    const bool all = __syncthreads_and(ok) != 0;
+    double Ku[2] = {0.0, 0.0};
+    if (all) {
+        if (own) {
+            const int e1 = Xe[me + 1], e2 = Xe[me + PX2], e3 = Xe[me + PX2 + 1];
+            const int ee = max(max(e, e1), max(e2, e3));
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+                Ku[p] = fix::to_double((fix::down(F[p][3], ee - e) + fix::down(X[p][2][me + 1], ee - e1)) +
+                                           (fix::down(X[p][1][me + PX2], ee - e2) +
+                                            fix::down(X[p][0][me + PX2 + 1], ee - e3)),
+                                       ee);
+        }
+    } else {
+        cell_forces2<double>(D, psi, a.c);
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) X[p][q][me] = fix::bits_of(D[p][q]);
+        __syncthreads();
+        if (own)
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+                Ku[p] = fix::of_bits(X[p][3][me]) + fix::of_bits(X[p][2][me + 1]) + fix::of_bits(X[p][1][me + PX2]) +
+                        fix::of_bits(X[p][0][me + PX2 + 1]);
+    }
+    double ssq = 0.0;
+    if (own) {
+        if (MODE == kJacobi && !a.dinv) ip = 1.0 / (ps[me] + ps[me + 1] + ps[me + PX2] + ps[me + PX2 + 1]);
+        body::finalize_f<double, TO, MODE>(a, gx, gy, 0, Ku, ip, uv, fv, ssq);
+    }
+    if (MODE == kResidual && a.part)
+        block_partial<NT2>(ssq, a.part + blockIdx.x + (long long)gridDim.x * blockIdx.y, red);
+}
+
+// Rows of cells per block: 8, on grids that would give fewer blocks than SMs 4.
+int rows2(const Geom &g)
+{
+    return ((g.nx + 30) / 32) * (long long)((g.ny + 6) / 8) >= 152 ? 8 : 4;
+}
+
+// 2D colour Gauss-Seidel in FP64, one launch per sweep.  A block owns a TILE x TILE tile of
+// nodes and stages u, f and psi on the tile plus a four-node halo; the four colour phases
+// then run in shared memory, phase q relaxing its colour on the tile grown by 3 - q nodes,
+// so every value a phase reads was produced by the phases before it exactly as in four
+// separate colour passes.  Only the tile is written, to a second buffer.  A thread turns
+// the 3 x 3 neighbourhood of its node into integers and evaluates the node's corner of its
+// four cells; a neighbourhood that does not fit takes the row of K in FP64.  The diagonal
+// blocks follow from psi sums: every corner of the unit-psi cell matrix has the same
+// diagonal entry, and the same coupling up to its sign (+ at corners 0 and 3).
+template <int TILE>
+__global__ void __launch_bounds__(256) k_gs2_fix(const Geom g, const fix::Consts fc, const double *__restrict__ psi,
+                                                 const double *__restrict__ Ke, const double *__restrict__ f,
+                                                 const double *__restrict__ uin, double *__restrict__ uout,
+                                                 int descending, const int *gate)
+{
+    pdl_begin();
+    if (gate && *gate) return;
+    constexpr int H = 4, SN = TILE + 2 * H, SC = SN - 1, SF = SN - 2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *su = reinterpret_cast<double *>(smem_raw);   // [2][SN][SN] staged nodes
+    double *sf = su + 2 * SN * SN;                        // [2][SF][SF] right-hand side of staged nodes 1 .. SN-2
+    double *sp = sf + 2 * SF * SF;                        // [SC][SC] psi of the staged cells (0 outside the grid)
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int x0 = blockIdx.x * TILE - H, y0 = blockIdx.y * TILE - H;   // global node of staged (0, 0)
+    for (int s = tid; s < SN * SN; s += nt) {
+        const int i = x0 + s % SN, j = y0 + s / SN;
+        const bool ok = i >= 0 && i < g.nx && j >= 0 && j < g.ny;
+        const long long o = ok ? gidx(g, i, j, 0) : 0;
+        su[s] = ok ? uin[o] : 0.0;
+        su[SN * SN + s] = ok ? uin[g.cs + o] : 0.0;
+    }
+    for (int s = tid; s < SF * SF; s += nt) {
+        const int i = x0 + 1 + s % SF, j = y0 + 1 + s / SF;
+        const bool ok = i >= 0 && i < g.nx && j >= 0 && j < g.ny;
+        const long long o = ok ? gidx(g, i, j, 0) : 0;
+        sf[s] = ok ? f[o] : 0.0;
+        sf[SF * SF + s] = ok ? f[g.cs + o] : 0.0;
+    }
+    for (int s = tid; s < SC * SC; s += nt) {
+        const int i = x0 + s % SC, j = y0 + s / SC;
+        const bool ok = i >= 0 && i < g.nx - 1 && j >= 0 && j < g.ny - 1;
+        sp[s] = ok ? psi[gidx(g, i, j, 0)] : 0.0;
+    }
+    const double kd = Ke[0], k01 = Ke[1];                 // corner 0: diagonal and coupling
+    __syncthreads();
+    for (int q = 0; q < 4; ++q) {
+        const int c = descending ? 3 - q : q;
+        const int h = 3 - q;                              // halo still relaxed in this phase
+        const int lo = H - h, nr = (TILE + 2 * h) / 2;    // first staged index, colour nodes per row
+        const int lx0 = lo + (((c & 1) - lo) & 1), ly0 = lo + (((c >> 1) - lo) & 1);
+        for (int n = tid; n < nr * nr; n += nt) {
+            const int lx = lx0 + 2 * (n % nr), ly = ly0 + 2 * (n / nr);
+            const int i = x0 + lx, j = y0 + ly;
+            if (i < 0 || j < 0 || i >= g.nx || j >= g.ny) continue;
+            const int me = ly * SN + lx, mf = (ly - 1) * SF + lx - 1;
+            double pc[4];                                 // cell a: the node is its corner a
+            bool ok = fc.ok;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                pc[a] = sp[(ly - (a >> 1)) * SC + lx - (a & 1)];
+                ok = ok && fix::psi_ok(pc[a]);
+            }
+            unsigned key = 0;
+            i64 I[2][9];
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+#pragma unroll
+                for (int m = 0; m < 9; ++m) {
+                    const double v = su[p * SN * SN + me + (m / 3 - 1) * SN + m % 3 - 1];
+                    key = max(key, fix::exp_key(v));
+                    I[p][m] = fix::bits_of(v);
+                }
+            ok = ok && fix::key_ok(key);
+            const int E = max((int)(key >> 20), fix::kExpLo);
+            double Ku[2] = {0.0, 0.0};
+            if (ok) {
+#pragma unroll
+                for (int p = 0; p < 2; ++p)
+#pragma unroll
+                    for (int m = 0; m < 9; ++m) I[p][m] = fix::to_fix(fix::of_bits(I[p][m]), E);
+                i64 F[4][2];
+                int e[4], ee = fix::kNoExp;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    i64 u4[2][4];
+#pragma unroll
+                    for (int p = 0; p < 2; ++p)
+#pragma unroll
+                        for (int b = 0; b < 4; ++b)
+                            u4[p][b] = I[p][(1 - (a >> 1) + (b >> 1)) * 3 + 1 - (a & 1) + (b & 1)];
+                    fix::corner_force2(u4, a, E, pc[a], fc, F[a], e[a]);
+                    ee = max(ee, e[a]);
+                }
+#pragma unroll
+                for (int p = 0; p < 2; ++p)
+                    Ku[p] = fix::to_double((fix::down(F[0][p], ee - e[0]) + fix::down(F[1][p], ee - e[1])) +
+                                               (fix::down(F[2][p], ee - e[2]) + fix::down(F[3][p], ee - e[3])),
+                                           ee);
+            } else {
+                for (int a = 0; a < 4; ++a)
+                    for (int p = 0; p < 2; ++p) {
+                        double t = 0.0;
+                        for (int b = 0; b < 4; ++b)
+                            for (int r = 0; r < 2; ++r)
+                                t = madd(Ke[(a * 2 + p) * 8 + b * 2 + r],
+                                         su[r * SN * SN + me + ((b >> 1) - (a >> 1)) * SN + (b & 1) - (a & 1)], t);
+                        Ku[p] = madd(pc[a], t, Ku[p]);
+                    }
+            }
+            const double w = 1.0 / (kd * ((pc[0] + pc[1]) + (pc[2] + pc[3])));
+            const double s01 = k01 * ((pc[0] + pc[3]) - (pc[1] + pc[2]));
+            if (!is_dir(g, 0, i, j, 0)) {
+                const double du = (sf[mf] - Ku[0]) * w;
+                su[me] += du;
+                Ku[1] = madd(s01, du, Ku[1]);
+            }
+            if (!is_dir(g, 1, i, j, 0)) su[SN * SN + me] += (sf[SF * SF + mf] - Ku[1]) * w;
+        }
+        __syncthreads();
+    }
+    for (int s = tid; s < TILE * TILE; s += nt) {
+        const int lx = H + s % TILE, ly = H + s / TILE;
+        const int i = x0 + lx, j = y0 + ly;
+        if (i >= g.nx || j >= g.ny) continue;
+        const long long o = gidx(g, i, j, 0);
+        uout[o] = su[ly * SN + lx];
+        uout[g.cs + o] = su[SN * SN + ly * SN + lx];
+    }
+}
+
+template <int TILE>
+cudaError_t launch_gs2_tile(const Geom &g, const fix::Consts &fc, const double *psi, const double *Ke, const double *f,
+                            const double *uin, double *uout, int descending, cudaStream_t s, const int *gate)
+{
+    constexpr int SN = TILE + 8;
+    constexpr size_t sm = sizeof(double) * (2 * SN * SN + 2 * (SN - 2) * (SN - 2) + (SN - 1) * (SN - 1));
+    static std::atomic<unsigned long long> attr_done{0};
+    cudaError_t e = smem_attr_once(reinterpret_cast<const void *>(k_gs2_fix<TILE>), sm, attr_done);
+    if (e != cudaSuccess) return e;
+    // the largest phase relaxes ((TILE + 6) / 2)^2 nodes
+    const int nt = TILE >= 32 ? 256 : TILE >= 16 ? 128 : 64;
+    const dim3 gr((g.nx + TILE - 1) / TILE, (g.ny + TILE - 1) / TILE, 1);
+    e = launch_pdl(k_gs2_fix<TILE>, gr, dim3(nt), sm, s, g, fc, psi, Ke, f, uin, uout, descending, gate);
+    if (e != cudaSuccess) return e;
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+__global__ void k_inv_psi(const Geom g, const double *__restrict__ psi, double *__restrict__ dinv)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    const int k = blockIdx.z * blockDim.z + threadIdx.z;
+    if (i >= g.nx || j >= g.ny || k >= g.nz) return;
+    double c[4];                                          // cells (i-1,j-1), (i,j-1), (i-1,j), (i,j), summed over z
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int ci = i - 1 + (q & 1), cj = j - 1 + (q >> 1);
+        const bool ok = ci >= 0 && cj >= 0 && ci < g.nx - 1 && cj < g.ny - 1;
+        if (g.dim == 3) {
+            const double lo = ok && k > 0 ? psi[gidx(g, ci, cj, k - 1)] : 0.0;
+            const double hi = ok && k < g.nz - 1 ? psi[gidx(g, ci, cj, k)] : 0.0;
+            c[q] = lo + hi;
+        } else {
+            c[q] = ok ? psi[gidx(g, ci, cj, 0)] : 0.0;
+        }
+    }
+    const double s = g.dim == 3 ? (c[0] + c[1]) + (c[2] + c[3]) : c[0] + c[1] + c[2] + c[3];
+    dinv[gidx(g, i, j, k)] = 1.0 / s;
 }
 
 template <typename TO, int MODE>
 cudaError_t launch_fix_mode(const SweepArgs<double, TO> &a, cudaStream_t s)
 {
-    static std::atomic<unsigned long long> attr_done{0};
-    cudaError_t e = smem_attr_once(reinterpret_cast<const void *>(k_sweep3_fix<TO, MODE>), kSmem, attr_done);
-    if (e != cudaSuccess) return e;
-    const fix::Consts fc = fix::make_consts(3, a.c);
-    e = launch_pdl(k_sweep3_fix<TO, MODE>, dim3((unsigned)sweep_blocks_fix(a.g)), dim3(NT), kSmem, s, a, fc);
+    const fix::Consts fc = fix::make_consts(a.g.dim, a.c);
+    cudaError_t e;
+    if (a.g.dim == 3) {
+        static std::atomic<unsigned long long> attr_done{0};
+        e = smem_attr_once(reinterpret_cast<const void *>(k_sweep3_fix<TO, MODE>), kSmem, attr_done);
+        if (e != cudaSuccess) return e;
+        e = launch_pdl(k_sweep3_fix<TO, MODE>, dim3((unsigned)sweep_blocks_fix(a.g)), dim3(NT), kSmem, s, a, fc);
+    } else {
+        const int ty = rows2(a.g);
+        const dim3 gr((a.g.nx + 30) / 32, (a.g.ny - 2 + ty) / ty), b(33 * (ty + 1));
+        e = ty == 8 ? launch_pdl(k_sweep2_fix<TO, MODE, 8>, gr, b, 0, s, a, fc)
+                    : launch_pdl(k_sweep2_fix<TO, MODE, 4>, gr, b, 0, s, a, fc);
+    }
     if (e != cudaSuccess) return e;
     ++g_launches;
     return cudaGetLastError();
@@ -441,11 +736,32 @@ cudaError_t launch_fix_mode(const SweepArgs<double, TO> &a, cudaStream_t s)
 
 }  // namespace
 
-// One block per SM of the 152, at most one per (tile, node plane) unit.
+// 3D: one block per SM of the 152, at most one per (tile, node plane) unit.  2D: the tiles.
 long long sweep_blocks_fix(const Geom &g)
 {
+    if (g.dim == 2) {
+        const int ty = rows2(g);
+        return ((g.nx + 30) / 32) * (long long)((g.ny - 2 + ty) / ty);
+    }
     const long long units = (long long)((g.nx - 1 + TX - 1) / TX) * ((g.ny - 1 + TY - 1) / TY) * g.nz;
     return std::min<long long>(152, units);
+}
+
+cudaError_t launch_inv_psi(const Geom &g, const double *psi, double *dinv, cudaStream_t s)
+{
+    const dim3 b(32, 4, 2), gr((g.nx + 31) / 32, (g.ny + 3) / 4, (g.nz + 1) / 2);
+    k_inv_psi<<<gr, b, 0, s>>>(g, psi, dinv);
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gs2_fix(const Geom &g, const Coef<double> &c, const double *psi, const double *Ke, const double *f,
+                           const double *uin, double *uout, int descending, cudaStream_t s, const int *gate)
+{
+    const fix::Consts fc = fix::make_consts(2, c);
+    const long long b32 = ((g.nx + 31) / 32) * (long long)((g.ny + 31) / 32);
+    if (b32 >= 304) return launch_gs2_tile<32>(g, fc, psi, Ke, f, uin, uout, descending, s, gate);
+    return launch_gs2_tile<16>(g, fc, psi, Ke, f, uin, uout, descending, s, gate);
 }
 
 template <typename TO>

@@ -44,6 +44,7 @@ struct Level {
     double h = 0;
     double *psi64 = nullptr;
     float *psi32 = nullptr;
+    double *dinv = nullptr;   // FP64 Jacobi scaling (ensure_dinv), or null
     double *du[2] = {nullptr, nullptr}, *df = nullptr, *dr = nullptr;
     float *su[2] = {nullptr, nullptr}, *sf = nullptr, *sr = nullptr;
     Coef<double> c64{};
@@ -129,6 +130,7 @@ struct sbm_grid_s {
     float *A32 = nullptr;
     int *gather = nullptr;
     bool bottom_ready = false;
+    bool dinv_ready = false;    // the levels' dinv belongs to their psi
     unsigned version = 1;
     GraphSlot slots[2];
     GraphSlot amr_slot;         // one outer iteration of the composite solve
@@ -225,6 +227,7 @@ cudaError_t sweep(sbm_grid G, int l, int mode, const T *u, const T *f, T *out, d
     for (int p = 0; p < 3; ++p) a.wk[p] = (L.c64.kdiag[p] != 0.0) ? T(omega / L.c64.kdiag[p]) : T(0);
     a.kchunk = 0;
     a.gate = G->cur_gate;
+    if constexpr (std::is_same<T, double>::value) a.dinv = G->dinv_ready ? L.dinv : nullptr;
     return launch_sweep<T, T>(mode, a, G->st);
 }
 
@@ -321,7 +324,7 @@ cudaError_t smooth(sbm_grid G, int l, int &cur, const sbm_opts &o, int nsweeps, 
     const int ncol = 1 << L.g.dim;
     for (int s = 0; s < nsweeps; ++s) {
         if (o.smoother == SBM_MCGS && L.g.dim == 2) {
-            CKE(launch_gs2_sweep<T>(L.g, P<T>::psi(L), P<T>::Ke(L), f, P<T>::u(L, cur), P<T>::u(L, 1 - cur),
+            CKE(launch_gs2_sweep<T>(L.g, P<T>::c(L), P<T>::psi(L), P<T>::Ke(L), f, P<T>::u(L, cur), P<T>::u(L, 1 - cur),
                                     descending ? 1 : 0, G->st, G->cur_gate));
             cur ^= 1;
         } else if (o.smoother == SBM_MCGS) {
@@ -449,6 +452,28 @@ cudaError_t enqueue_fp64_batch(sbm_grid G, const sbm_opts &o, const double *rhs,
     return e;
 }
 
+// The FP64 Jacobi scaling of every smoothed level, formed once per psi: in the sweep the
+// FP64 division costs as much FP64 issue as the rest of the node's update.  A level
+// whose array cannot be allocated goes without (the sweep then divides).
+cudaError_t ensure_dinv(sbm_grid G)
+{
+    if (G->dinv_ready) return cudaSuccess;
+    for (int l = 1; l < G->nl; ++l) {
+        Level &L = G->L[l];
+        if (!L.dinv) {
+            if (gmalloc(G, (void **)&L.dinv, sizeof(double) * L.g.cs) != cudaSuccess) {
+                cudaGetLastError();
+                L.dinv = nullptr;
+                continue;
+            }
+            ++G->version;            // graphs captured without it are captured again
+        }
+        CKE(launch_inv_psi(L.g, L.psi64, L.dinv, G->st));
+    }
+    G->dinv_ready = true;
+    return cudaSuccess;
+}
+
 sbm_status setup_bottom(sbm_grid G)
 {
     if (G->bottom_ready) return SBM_OK;
@@ -542,6 +567,7 @@ sbm_status run_solve(sbm_grid G, const sbm_opts &o, const double *rhs, sbm_info 
     sbm_status st = setup_bottom(G);
     if (st != SBM_OK) return st;
     const int mixed = G->desc.precision == SBM_MIXED;
+    if (!mixed && o.smoother == SBM_JACOBI) CK(ensure_dinv(G));
     const long long launches0 = g_launches;
     long long replayed = 0;
     CK(cudaEventRecord(G->ev0, G->st));
@@ -863,7 +889,7 @@ cudaError_t patch_smooth(sbm_grid G, Patch &Pt, int &cur, const sbm_opts &o, int
     const int ncol = 1 << Pt.v.dim;
     for (int s = 0; s < n; ++s) {
         if (o.smoother == SBM_MCGS && Pt.v.dim == 2) {
-            CKE(launch_gs2_sweep<T>(Pt.v, PP<T>::psi(Pt) + Pt.voff, PP<T>::Ke(Pt), PP<T>::rhs(Pt) + Pt.voff,
+            CKE(launch_gs2_sweep<T>(Pt.v, PP<T>::c(Pt), PP<T>::psi(Pt) + Pt.voff, PP<T>::Ke(Pt), PP<T>::rhs(Pt) + Pt.voff,
                                     PP<T>::e(Pt, cur) + Pt.voff, PP<T>::e(Pt, 1 - cur) + Pt.voff, desc ? 1 : 0, G->st));
             cur ^= 1;
         } else if (o.smoother == SBM_MCGS) {
@@ -1260,6 +1286,7 @@ sbm_status amr_prepare(sbm_grid G)
             CK(launch_coarsen_psi(G->L[l].g, G->L[l - 1].g, G->L[l].psi64, G->L[l - 1].psi64, G->st));
         for (int l = 0; l < G->nl; ++l) CK(launch_round_cells(G->L[l].g, G->L[l].psi64, G->L[l].psi32, G->st));
         G->bottom_ready = false;
+        G->dinv_ready = false;
         G->amr_psi_dirty = false;
     }
     return SBM_OK;
@@ -1270,6 +1297,7 @@ sbm_status amr_run(sbm_grid G, const sbm_opts &o, sbm_info *info)
 {
     sbm_status st = setup_bottom(G);
     if (st != SBM_OK) return st;
+    if (std::is_same<T, double>::value && o.smoother == SBM_JACOBI) CK(ensure_dinv(G));
     const long long launches0 = g_launches;
     CK(cudaEventRecord(G->ev0, G->st));
     CK(amr_residual<T>(G, 0));
@@ -1466,7 +1494,7 @@ sbm_status sbm_grid_destroy(sbm_grid G)
     if (G->fork_ev) cudaEventDestroy(G->fork_ev);
     for (int l = 0; l < G->nl; ++l) {
         Level &L = G->L[l];
-        void *ptrs[] = {L.psi64, L.psi32, L.du[0], L.du[1], L.df, L.dr, L.su[0], L.su[1], L.sf, L.sr, L.Ke64, L.Ke32};
+        void *ptrs[] = {L.psi64, L.psi32, L.dinv, L.du[0], L.du[1], L.df, L.dr, L.su[0], L.su[1], L.sf, L.sr, L.Ke64, L.Ke32};
         for (void *p : ptrs)
             if (p) cudaFree(p);
     }
@@ -1681,6 +1709,7 @@ static sbm_status finish_psi(sbm_grid G)
     }
     G->has_psi = true;
     G->bottom_ready = false;
+    G->dinv_ready = false;
     return SBM_OK;
 }
 

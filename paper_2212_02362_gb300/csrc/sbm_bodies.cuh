@@ -34,15 +34,15 @@ __device__ __forceinline__ void finalize(const SweepArgs<T, TO> &a, int gx, int 
     }
 }
 
-// finalize with the node's right-hand side already loaded (fv[p] = f[p] at the node).
+// finalize with the node's right-hand side already loaded (fv[p] = f[p] at the node) and
+// the Jacobi scaling ip = 1 / psi sum.
 template <typename T, typename TO, int MODE>
 __device__ __forceinline__ void finalize_f(const SweepArgs<T, TO> &a, int gx, int gy, int gz, const T *Ku,
-                                           T psisum, const T *uval, const T *fv, double &ssq)
+                                           T ip, const T *uval, const T *fv, double &ssq)
 {
     const Geom &g = a.g;
     const long long o = gidx(g, gx, gy, gz);
     if (MODE == kJacobi) {
-        const T ip = T(1) / psisum;
         for (int p = 0; p < g.dim; ++p) {
             T v = uval[p];
             if (!is_dir(g, p, gx, gy, gz)) v += (fv[p] - Ku[p]) * ip * a.wk[p];

@@ -101,6 +101,7 @@ struct SweepArgs {
     T wk[3];               // Jacobi: omega / kdiag[p]
     int kchunk;            // node planes per block along z (3D)
     const int *gate = nullptr;   // device flag: when set, the launch does nothing
+    const T *dinv = nullptr;     // FP64 Jacobi: 1 / (psi sum of the node's cells), or null (formed in the sweep)
 };
 
 // Number of z chunks for a z-streaming stencil launch: minimises
@@ -171,11 +172,16 @@ long long sweep_blocks(const Geom &g, bool fp64);
 template <typename T, typename TO>
 cudaError_t launch_sweep(int mode, const SweepArgs<T, TO> &a, cudaStream_t s);
 
-// FP64 3D sweep with the cell arithmetic in 64-bit integers (k_stencil_fix.cu) and its
+// FP64 sweeps with the cell arithmetic in 64-bit integers (k_stencil_fix.cu) and their
 // blocks (= partial sums).
 template <typename TO>
 cudaError_t launch_sweep_fix(int mode, const SweepArgs<double, TO> &a, cudaStream_t s);
 long long sweep_blocks_fix(const Geom &g);
+// dinv[node] = 1 / (sum of psi over the node's cells), summed in the sweeps' order.
+cudaError_t launch_inv_psi(const Geom &g, const double *psi, double *dinv, cudaStream_t s);
+// One 2D FP64 colour Gauss-Seidel sweep (see launch_gs2_sweep); c: the level's constants.
+cudaError_t launch_gs2_fix(const Geom &g, const Coef<double> &c, const double *psi, const double *Ke, const double *f,
+                           const double *uin, double *uout, int descending, cudaStream_t s, const int *gate);
 
 // FP32 3D sweep with TMA plane staging and packed FP32x2 arithmetic, one
 // persistent CTA per SM (k_stencil_tma.cu).  tmap: three CUtensorMaps of the
@@ -199,7 +205,7 @@ cudaError_t launch_gs(const Geom &g, const T *psi, const T *Ke, const T *f, T *u
 // One 2D colour Gauss-Seidel sweep (all four colours, ascending or descending) in one
 // launch, reading uin and writing every node of the grid to uout (uout != uin).
 template <typename T>
-cudaError_t launch_gs2_sweep(const Geom &g, const T *psi, const T *Ke, const T *f, const T *uin, T *uout,
+cudaError_t launch_gs2_sweep(const Geom &g, const Coef<T> &c, const T *psi, const T *Ke, const T *f, const T *uin, T *uout,
                              int descending, cudaStream_t s, const int *gate = nullptr);
 
 template <typename T>

@@ -140,13 +140,14 @@ inline Consts make_consts(int dim, const Coef<double> &c)
     if (!(bound > ldexp(1.0, -200)) || !(bound < ldexp(1.0, 200))) return r;
     int eb;
     frexp(bound, &eb);                       // bound < 2^eb
+    const int lg = dim == 3 ? 61 : 62;
     for (int i = 0; i < 7; ++i) {
         if (!(v[i] >= 0.0)) return r;
-        // c <= 2^61 for v = 2^eb: with psi's mantissa below 2^63 the product's upper half
-        // is below 2^60, which is 1/16 of the fraction 1
-        r.c[i] = split((i64)rint(ldexp(v[i], 61 - eb)));
+        // 3D: c <= 2^61 for v = 2^eb, so with psi's mantissa below 2^63 the product's upper
+        // half is below 2^60 (1/16 of the fraction 1); 2D, with fewer terms, twice that
+        r.c[i] = split((i64)rint(ldexp(v[i], lg - eb)));
     }
-    r.ec = eb + 4;
+    r.ec = eb + 65 - lg;
     r.ok = 1;
     return r;
 }
@@ -252,6 +253,72 @@ __host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], cons
             Ft[p][s] = dU[p][s] + dU[p][s + 4];
         }
     }
+}
+
+// The six transformed values of a 2D cell that carry force, in the order U[0][1..3],
+// U[1][1..3] of bfly4, shifted up to 2^61 at most.  Returns the shift; m = 0: all zero.
+__host__ __device__ __forceinline__ int transform2(const i64 (&u)[2][4], i64 (&U)[2][4], bool &none)
+{
+    unsigned long long m = 0;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) U[p][q] = u[p][q];
+        bfly4(U[p]);
+#pragma unroll
+        for (int q = 1; q < 4; ++q) m |= (unsigned long long)(U[p][q] ^ (U[p][q] >> 63));
+    }
+    none = m == 0ull;
+    const int sh = norm_shift(m);            // |U| <= 4 2^60: at least -2
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int q = 1; q < 4; ++q)
+            U[p][q] = sh >= 0 ? (i64)((unsigned long long)U[p][q] << (sh & 63)) : U[p][q] >> (-sh & 63);
+    return sh;
+}
+
+// One 2D cell: nodal integers on the unit 2^(E - kFixUnit) -> corner forces on 2^e.
+__host__ __device__ __forceinline__ void cell_forces2(const i64 (&u)[2][4], int E, double psi, const Consts &c,
+                                                      i64 (&F)[2][4], int &e)
+{
+    i64 U[2][4];
+    bool none;
+    const int sh = transform2(u, U, none);
+    int ep;
+    const i64 pm = psi_mantissa(psi, ep);
+    e = (none || pm == 0) ? kNoExp : E - kFixUnit - sh + ep + c.ec;
+    Frac k[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) k[i] = split(mul(pm, c.c[i]));
+    i64 ltr = mul(U[0][1] + U[1][2], k[1]);
+    ltr = c.neg12 ? -ltr : ltr;
+    const i64 sxy = mul(U[1][1] + U[0][2], k[2]);
+    F[0][0] = 0; F[0][1] = mul(U[0][1], k[0]) + ltr; F[0][2] = sxy; F[0][3] = mul(U[0][3], k[3]);
+    F[1][0] = 0; F[1][1] = sxy; F[1][2] = mul(U[1][2], k[0]) + ltr; F[1][3] = mul(U[1][3], k[3]);
+    bfly4T(F[0]);
+    bfly4T(F[1]);
+}
+
+// The same for the force on corner a alone; psi multiplies the two forces.
+__host__ __device__ __forceinline__ void corner_force2(const i64 (&u)[2][4], int a, int E, double psi, const Consts &c,
+                                                       i64 (&F)[2], int &e)
+{
+    i64 U[2][4];
+    bool none;
+    const int sh = transform2(u, U, none);
+    int ep;
+    const i64 pm = psi_mantissa(psi, ep);
+    e = (none || pm == 0) ? kNoExp : E - kFixUnit - sh + ep + c.ec + 1;
+    i64 ltr = mul(U[0][1] + U[1][2], c.c[1]);
+    ltr = c.neg12 ? -ltr : ltr;
+    const i64 sxx = mul(U[0][1], c.c[0]) + ltr, syy = mul(U[1][2], c.c[0]) + ltr;
+    const i64 sxy = mul(U[1][1] + U[0][2], c.c[2]);
+    const i64 d0 = mul(U[0][3], c.c[3]), d1 = mul(U[1][3], c.c[3]);
+    const bool px = (a & 1) != 0, py = (a & 2) != 0;
+    const Frac k = split(pm >> 1);
+    F[0] = mul((px ? sxx : -sxx) + (py ? sxy : -sxy) + (px == py ? d0 : -d0), k);
+    F[1] = mul((px ? sxy : -sxy) + (py ? syy : -syy) + (px == py ? d1 : -d1), k);
 }
 
 }  // namespace fix

@@ -92,3 +92,57 @@ def test_zero_psi_and_wide_psi():
     u = W.uniform(100, P.ndofs, -1, 1)
     assert _rel(host(g.apply(g.finest, cuda(u))), oracle.apply(P, oracle.floor_psi(wk.psi, 1e-8), u)) <= 1e-13
     assert np.all(host(g.apply(g.finest, cuda(np.repeat([0.3, -0.7, 1.1], P.nnodes)))) == 0.0)
+
+
+# 2D: tiles of 32 x 8 or 32 x 4 cells (from 152 tiles on the taller ones), colour tiles of
+# 16 or (from 304 tiles of 32 on) 32 nodes
+@pytest.mark.parametrize("n", [(2, 2), (33, 5), (34, 6), (17, 16), (16, 33), (65, 49), (609, 521)])
+def test_2d_tile_edges(n):
+    wk = random_workload(2, n, 110)
+    g, P = gpu_grid(wk), oracle_problem(wk)
+    u = wk.u0 + W.uniform(111, P.ndofs, -1e-2, 1e-2) * ~oracle.dirichlet_mask(P)
+    psi = oracle.floor_psi(wk.psi, wk.psi_min)
+    assert _rel(host(g.apply(g.finest, cuda(u))), oracle.apply(P, psi, u)) <= 1e-13
+    r, nrm = g.residual(g.finest, cuda(wk.f), cuda(u))
+    ref = oracle.residual(P, psi, wk.f, u)
+    assert _rel(host(r), ref) <= 1e-13 and np.isclose(nrm, oracle.norm_free(P, ref), rtol=1e-13)
+    got = host(g.smooth(g.finest, cuda(wk.f), cuda(u), "jacobi", 0.6))
+    assert _rel(got - u, oracle.jacobi_sweep(P, psi, wk.f, u, 0.6) - u) <= 1e-12
+    for desc in (False, True):
+        got = host(g.smooth(g.finest, cuda(wk.f), cuda(u), "gs", descending=desc))
+        assert _rel(got - u, oracle.gs_sweep(P, psi, wk.f, u, desc) - u) <= 1e-11
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan, 1e250, 1e-250])
+def test_2d_values_that_do_not_fit(value):
+    wk = random_workload(2, (49, 33), 112)
+    g, P = gpu_grid(wk), oracle_problem(wk)
+    u = W.uniform(113, P.ndofs, -1, 1)
+    v = u.reshape(2, 33, 49)
+    if value == 1e-250:
+        v[:, 13:20, 20:27] = 0.0
+    v[1, 16, 23] = value
+    psi = oracle.floor_psi(wk.psi, wk.psi_min)
+    with np.errstate(invalid="ignore", over="ignore"):
+        pairs = [(oracle.apply(P, psi, u), host(g.apply(g.finest, cuda(u)))),
+                 (oracle.gs_sweep(P, psi, wk.f, u), host(g.smooth(g.finest, cuda(wk.f), cuda(u), "gs")))]
+    for ref, got in pairs:
+        fin = np.isfinite(ref)
+        assert np.array_equal(fin, np.isfinite(got))
+        fin &= np.abs(ref) < 1e10
+        assert fin.sum() > 3000 and np.abs((got - ref)[fin]).max() <= 1e-11 * np.abs(ref[fin]).max()
+
+
+@pytest.mark.parametrize("dim,n", [(2, (65, 41)), (3, (17, 17, 21))])
+def test_solve_after_a_new_psi(dim, n):
+    """The FP64 Jacobi scaling kept per level follows the psi: solves on one grid with a
+    first and a second psi equal solves on fresh grids."""
+    wk, w2 = random_workload(dim, n, 114, moduli=W.iso_cubic(1.0, 0.2)), random_workload(dim, n, 115, moduli=W.iso_cubic(1.0, 0.2))
+    g = gpu_grid(wk)
+    for psi in (wk.psi, w2.psi, wk.psi):
+        g.set_psi(cuda(psi), wk.psi_min)
+        fresh = gpu_grid(wk)
+        fresh.set_psi(cuda(psi), wk.psi_min)
+        u, v = cuda(wk.u0), cuda(wk.u0)
+        a, b = g.solve(u, omega=0.5), fresh.solve(v, omega=0.5)
+        assert a.cycles == b.cycles and np.array_equal(host(u), host(v))
