@@ -191,10 +191,14 @@ __global__ void k_amr_ghost(const Geom sc, const AmrInfo Lc, const Geom sp, cons
 #pragma unroll
         for (int p = 0; p < D; ++p) v[c][p] = in ? up[p * sp.cs + o] : T(0);
     }
+    // the child nodes: offset (-1: none to write), and in mode 1 the solved ones' values,
+    // all loaded before the first store (a load behind a store waits for it)
+    long long oc[1 << D];
+    bool solved[1 << D];
+    T old[1 << D][D];
 #pragma unroll
     for (int d = 0; d < (1 << D); ++d) {
-        const int dl[3] = {d & 1, (d >> 1) & 1, D == 3 ? d >> 2 : 0};
-        const int g[3] = {2 * B[0] + dl[0], 2 * B[1] + dl[1], 2 * B[2] + dl[2]};
+        const int g[3] = {2 * B[0] + (d & 1), 2 * B[1] + ((d >> 1) & 1), 2 * B[2] + (D == 3 ? d >> 2 : 0)};
         int l[3];
         bool in = true;
 #pragma unroll
@@ -202,9 +206,16 @@ __global__ void k_amr_ghost(const Geom sc, const AmrInfo Lc, const Geom sp, cons
             l[ax] = g[ax] - Lc.org[ax];
             if (l[ax] < 0 || l[ax] >= cn[ax]) in = false;
         }
-        if (!in) continue;
-        const bool solved = axes_owned(Lc, g);
-        if (solved && mode != 1) continue;
+        solved[d] = axes_owned(Lc, g);
+        oc[d] = in && !(solved[d] && mode != 1) ? gidx(sc, l[0], l[1], l[2]) : -1;
+#pragma unroll
+        for (int p = 0; p < D; ++p) old[d][p] = (oc[d] >= 0 && solved[d]) ? uc[p * sc.cs + oc[d]] : T(0);
+    }
+#pragma unroll
+    for (int d = 0; d < (1 << D); ++d) {
+        if (oc[d] < 0) continue;
+        const int dl[3] = {d & 1, (d >> 1) & 1, D == 3 ? d >> 2 : 0};
+        const int g[3] = {2 * B[0] + dl[0], 2 * B[1] + dl[1], 2 * B[2] + dl[2]};
         T val[D];
 #pragma unroll
         for (int p = 0; p < D; ++p) val[p] = T(0);
@@ -226,39 +237,45 @@ __global__ void k_amr_ghost(const Geom sc, const AmrInfo Lc, const Geom sp, cons
 #pragma unroll
             for (int p = 0; p < D; ++p) val[p] *= sc_;
         }
-        const long long o = gidx(sc, l[0], l[1], l[2]);
 #pragma unroll
         for (int p = 0; p < D; ++p) {
-            if (!solved) uc[p * sc.cs + o] = val[p];
-            else if (!domain_dirichlet(Lc, g, p)) uc[p * sc.cs + o] += val[p];
+            if (!solved[d]) uc[p * sc.cs + oc[d]] = val[p];
+            else if (!domain_dirichlet(Lc, g, p)) uc[p * sc.cs + oc[d]] = old[d][p] + val[p];
         }
     }
 }
 
 // rhs_parent at the parent nodes covered by this child <- full weighting of the
-// child residual (the child nodes of the stencil are all inside the child box).
-template <typename T>
-__global__ void k_amr_restrict(const Geom sc, const AmrInfo Lc, const Geom sp, const AmrInfo Lp, const T *rc, T *rhsp)
+// child residual (the child nodes of the stencil are all inside the child box).  The
+// 3^D loads of a component are independent (clamped index, zero weight outside).
+template <typename T, int D>
+__global__ void k_amr_restrict(const Geom sc, const AmrInfo Lc, const Geom sp, const AmrInfo Lp, const T *rc, T *rhsp,
+                               int3 b0)
 {
-    int i, j, k, g[3];
-    if (!thread_node(sp, Lp, i, j, k, g)) return;
+    // storage node of the parent; the launch covers the nodes under the child's box from b0
+    const int i = b0.x + blockIdx.x * blockDim.x + threadIdx.x, j = b0.y + blockIdx.y * blockDim.y + threadIdx.y,
+              k = b0.z + blockIdx.z * blockDim.z + threadIdx.z;
+    if (i >= sp.nx || j >= sp.ny || k >= sp.nz) return;
+    const int g[3] = {i + Lp.org[0], j + Lp.org[1], k + Lp.org[2]};
     if (!covered_by(Lc, g)) return;
-    const bool d3 = Lp.dim == 3;
-    const T w[3] = {T(0.5), T(1), T(0.5)};
-    const T scale = d3 ? T(0.125) : T(0.25);
+    const T scale = D == 3 ? T(0.125) : T(0.25);
     const long long op = gidx(sp, i, j, k);
-    T s[3] = {T(0), T(0), T(0)};
-    for (int dk = (d3 ? -1 : 0); dk <= (d3 ? 1 : 0); ++dk)
-        for (int dj = -1; dj <= 1; ++dj)
-            for (int di = -1; di <= 1; ++di) {
-                const int li = 2 * g[0] + di - Lc.org[0], lj = 2 * g[1] + dj - Lc.org[1];
-                const int lk = d3 ? 2 * g[2] + dk - Lc.org[2] : 0;
-                if (li < 0 || lj < 0 || lk < 0 || li >= sc.nx || lj >= sc.ny || lk >= sc.nz) continue;
-                const T wt = w[di + 1] * w[dj + 1] * (d3 ? w[dk + 1] : T(1));
-                const long long oc = gidx(sc, li, lj, lk);
-                for (int p = 0; p < Lp.dim; ++p) s[p] += wt * rc[p * sc.cs + oc];
-            }
-    for (int p = 0; p < Lp.dim; ++p) rhsp[p * sp.cs + op] = domain_dirichlet(Lp, g, p) ? T(0) : s[p] * scale;
+    const int l0[3] = {2 * g[0] - Lc.org[0], 2 * g[1] - Lc.org[1], D == 3 ? 2 * g[2] - Lc.org[2] : 0};
+    T s[D];
+#pragma unroll
+    for (int p = 0; p < D; ++p) s[p] = T(0);
+#pragma unroll
+    for (int m = 0; m < (D == 3 ? 27 : 9); ++m) {
+        const int di = m % 3 - 1, dj = m / 3 % 3 - 1, dk = D == 3 ? m / 9 - 1 : 0;
+        const int li = l0[0] + di, lj = l0[1] + dj, lk = l0[2] + dk;
+        const bool in = li >= 0 && lj >= 0 && lk >= 0 && li < sc.nx && lj < sc.ny && lk < sc.nz;
+        const T wt = in ? T(1) / T(1 << ((di != 0) + (dj != 0) + (dk != 0))) : T(0);
+        const long long oc = in ? gidx(sc, li, lj, lk) : 0;
+#pragma unroll
+        for (int p = 0; p < D; ++p) s[p] += wt * (in ? rc[p * sc.cs + oc] : T(0));
+    }
+#pragma unroll
+    for (int p = 0; p < D; ++p) rhsp[p * sp.cs + op] = domain_dirichlet(Lp, g, p) ? T(0) : s[p] * scale;
 }
 
 // u += e on owned free dofs.
@@ -756,7 +773,14 @@ template <typename T>
 cudaError_t launch_amr_restrict(const Geom &sc, const AmrInfo &Lc, const Geom &sp, const AmrInfo &Lp, const T *rc,
                                 T *rhsp, cudaStream_t st)
 {
-    k_amr_restrict<T><<<amr_grid(sp), kAmrBlock, 0, st>>>(sc, Lc, sp, Lp, rc, rhsp);
+    const int3 b0 = make_int3(Lc.lo[0] / 2 - Lp.org[0], Lc.lo[1] / 2 - Lp.org[1],
+                              sc.dim == 3 ? Lc.lo[2] / 2 - Lp.org[2] : 0);
+    Geom box = sp;
+    box.nx = (Lc.hi[0] - Lc.lo[0]) / 2 + 1;
+    box.ny = (Lc.hi[1] - Lc.lo[1]) / 2 + 1;
+    box.nz = sc.dim == 3 ? (Lc.hi[2] - Lc.lo[2]) / 2 + 1 : 1;
+    if (sc.dim == 3) k_amr_restrict<T, 3><<<amr_grid(box), kAmrBlock, 0, st>>>(sc, Lc, sp, Lp, rc, rhsp, b0);
+    else k_amr_restrict<T, 2><<<amr_grid(box), kAmrBlock, 0, st>>>(sc, Lc, sp, Lp, rc, rhsp, b0);
     ++g_launches;
     return cudaGetLastError();
 }

@@ -546,25 +546,32 @@ int rows2(const Geom &g)
 // nodes and stages u, f and psi on the tile plus a four-node halo; the four colour phases
 // then run in shared memory, phase q relaxing its colour on the tile grown by 3 - q nodes,
 // so every value a phase reads was produced by the phases before it exactly as in four
-// separate colour passes.  Only the tile is written, to a second buffer.  A thread turns
-// the 3 x 3 neighbourhood of its node into integers and evaluates the node's corner of its
-// four cells; a neighbourhood that does not fit takes the row of K in FP64.  The diagonal
-// blocks follow from psi sums: every corner of the unit-psi cell matrix has the same
-// diagonal entry, and the same coupling up to its sign (+ at corners 0 and 3).
+// separate colour passes.  Only the tile is written, to a second buffer.  A phase is a
+// chain of one node's update, so its work is spread: a thread takes one of a node's four
+// cells (the corner force in integers), then, after a barrier, one thread per node adds
+// the four and updates.  A node with a value that does not fit takes its row of K in FP64.
+// The diagonal blocks follow from psi sums: every corner of the unit-psi cell matrix has
+// the same diagonal entry, and the same coupling up to its sign (+ at corners 0 and 3).
+constexpr int kGsThreads = 512;
+
 template <int TILE>
-__global__ void __launch_bounds__(256) k_gs2_fix(const Geom g, const fix::Consts fc, const double *__restrict__ psi,
-                                                 const double *__restrict__ Ke, const double *__restrict__ f,
-                                                 const double *__restrict__ uin, double *__restrict__ uout,
-                                                 int descending, const int *gate)
+__global__ void __launch_bounds__(kGsThreads) k_gs2_fix(const Geom g, const fix::Consts fc,
+                                                        const double *__restrict__ psi, const double *__restrict__ Ke,
+                                                        const double *__restrict__ f, const double *__restrict__ uin,
+                                                        double *__restrict__ uout, int descending, const int *gate)
 {
     pdl_begin();
     if (gate && *gate) return;
     constexpr int H = 4, SN = TILE + 2 * H, SC = SN - 1, SF = SN - 2;
+    constexpr int NQ = (TILE + 6) / 2 * ((TILE + 6) / 2);  // nodes of the largest phase
+    constexpr int kBad = 1 << 20;                          // exponent of a cell that does not fit
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *su = reinterpret_cast<double *>(smem_raw);   // [2][SN][SN] staged nodes
     double *sf = su + 2 * SN * SN;                        // [2][SF][SF] right-hand side of staged nodes 1 .. SN-2
     double *sp = sf + 2 * SF * SF;                        // [SC][SC] psi of the staged cells (0 outside the grid)
-    const int tid = threadIdx.x, nt = blockDim.x;
+    i64 *X = reinterpret_cast<i64 *>(sp + SC * SC);       // [4][2][NQ] corner forces of a phase
+    int *Xe = reinterpret_cast<int *>(X + 8 * NQ);        // [4][NQ] their exponents
+    const int tid = threadIdx.x, nt = kGsThreads;
     const int x0 = blockIdx.x * TILE - H, y0 = blockIdx.y * TILE - H;   // global node of staged (0, 0)
     for (int s = tid; s < SN * SN; s += nt) {
         const int i = x0 + s % SN, j = y0 + s / SN;
@@ -591,55 +598,57 @@ __global__ void __launch_bounds__(256) k_gs2_fix(const Geom g, const fix::Consts
         const int c = descending ? 3 - q : q;
         const int h = 3 - q;                              // halo still relaxed in this phase
         const int lo = H - h, nr = (TILE + 2 * h) / 2;    // first staged index, colour nodes per row
+        const int nq = nr * nr;
         const int lx0 = lo + (((c & 1) - lo) & 1), ly0 = lo + (((c >> 1) - lo) & 1);
-        for (int n = tid; n < nr * nr; n += nt) {
+        for (int t = tid; t < 4 * nq; t += nt) {
+            const int a = t / nq, n = t - a * nq;         // the node is corner a of the cell
+            const int cx = lx0 + 2 * (n % nr) - (a & 1), cy = ly0 + 2 * (n / nr) - (a >> 1);
+            const double pc = sp[cy * SC + cx];
+            double v[2][4];
+            unsigned key = 0;
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    v[p][b] = su[p * SN * SN + (cy + (b >> 1)) * SN + cx + (b & 1)];
+                    key = max(key, fix::exp_key(v[p][b]));
+                }
+            int e = kBad;
+            if (fc.ok && fix::key_ok(key) && fix::psi_ok(pc)) {
+                const int E = max((int)(key >> 20), fix::kExpLo);
+                i64 I[2][4], F[2];
+#pragma unroll
+                for (int p = 0; p < 2; ++p)
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) I[p][b] = fix::to_fix(v[p][b], E);
+                fix::corner_force2(I, a, E, pc, fc, F, e);
+                X[(a * 2) * NQ + n] = F[0];
+                X[(a * 2 + 1) * NQ + n] = F[1];
+            }
+            Xe[a * NQ + n] = e;
+        }
+        __syncthreads();
+        for (int n = tid; n < nq; n += nt) {
             const int lx = lx0 + 2 * (n % nr), ly = ly0 + 2 * (n / nr);
             const int i = x0 + lx, j = y0 + ly;
             if (i < 0 || j < 0 || i >= g.nx || j >= g.ny) continue;
             const int me = ly * SN + lx, mf = (ly - 1) * SF + lx - 1;
             double pc[4];                                 // cell a: the node is its corner a
-            bool ok = fc.ok;
+            int e[4], ee = fix::kNoExp;
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
                 pc[a] = sp[(ly - (a >> 1)) * SC + lx - (a & 1)];
-                ok = ok && fix::psi_ok(pc[a]);
+                e[a] = Xe[a * NQ + n];
+                ee = max(ee, e[a]);
             }
-            unsigned key = 0;
-            i64 I[2][9];
-#pragma unroll
-            for (int p = 0; p < 2; ++p)
-#pragma unroll
-                for (int m = 0; m < 9; ++m) {
-                    const double v = su[p * SN * SN + me + (m / 3 - 1) * SN + m % 3 - 1];
-                    key = max(key, fix::exp_key(v));
-                    I[p][m] = fix::bits_of(v);
-                }
-            ok = ok && fix::key_ok(key);
-            const int E = max((int)(key >> 20), fix::kExpLo);
             double Ku[2] = {0.0, 0.0};
-            if (ok) {
+            if (ee != kBad) {
 #pragma unroll
                 for (int p = 0; p < 2; ++p)
-#pragma unroll
-                    for (int m = 0; m < 9; ++m) I[p][m] = fix::to_fix(fix::of_bits(I[p][m]), E);
-                i64 F[4][2];
-                int e[4], ee = fix::kNoExp;
-#pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    i64 u4[2][4];
-#pragma unroll
-                    for (int p = 0; p < 2; ++p)
-#pragma unroll
-                        for (int b = 0; b < 4; ++b)
-                            u4[p][b] = I[p][(1 - (a >> 1) + (b >> 1)) * 3 + 1 - (a & 1) + (b & 1)];
-                    fix::corner_force2(u4, a, E, pc[a], fc, F[a], e[a]);
-                    ee = max(ee, e[a]);
-                }
-#pragma unroll
-                for (int p = 0; p < 2; ++p)
-                    Ku[p] = fix::to_double((fix::down(F[0][p], ee - e[0]) + fix::down(F[1][p], ee - e[1])) +
-                                               (fix::down(F[2][p], ee - e[2]) + fix::down(F[3][p], ee - e[3])),
-                                           ee);
+                    Ku[p] = fix::to_double(
+                        (fix::down(X[p * NQ + n], ee - e[0]) + fix::down(X[(2 + p) * NQ + n], ee - e[1])) +
+                            (fix::down(X[(4 + p) * NQ + n], ee - e[2]) + fix::down(X[(6 + p) * NQ + n], ee - e[3])),
+                        ee);
             } else {
                 for (int a = 0; a < 4; ++a)
                     for (int p = 0; p < 2; ++p) {
@@ -676,15 +685,14 @@ template <int TILE>
 cudaError_t launch_gs2_tile(const Geom &g, const fix::Consts &fc, const double *psi, const double *Ke, const double *f,
                             const double *uin, double *uout, int descending, cudaStream_t s, const int *gate)
 {
-    constexpr int SN = TILE + 8;
-    constexpr size_t sm = sizeof(double) * (2 * SN * SN + 2 * (SN - 2) * (SN - 2) + (SN - 1) * (SN - 1));
+    constexpr int SN = TILE + 8, NQ = (TILE + 6) / 2 * ((TILE + 6) / 2);
+    constexpr size_t sm = sizeof(double) * (2 * SN * SN + 2 * (SN - 2) * (SN - 2) + (SN - 1) * (SN - 1) + 8 * NQ) +
+                          sizeof(int) * 4 * NQ;
     static std::atomic<unsigned long long> attr_done{0};
     cudaError_t e = smem_attr_once(reinterpret_cast<const void *>(k_gs2_fix<TILE>), sm, attr_done);
     if (e != cudaSuccess) return e;
-    // the largest phase relaxes ((TILE + 6) / 2)^2 nodes
-    const int nt = TILE >= 32 ? 256 : TILE >= 16 ? 128 : 64;
     const dim3 gr((g.nx + TILE - 1) / TILE, (g.ny + TILE - 1) / TILE, 1);
-    e = launch_pdl(k_gs2_fix<TILE>, gr, dim3(nt), sm, s, g, fc, psi, Ke, f, uin, uout, descending, gate);
+    e = launch_pdl(k_gs2_fix<TILE>, gr, dim3(kGsThreads), sm, s, g, fc, psi, Ke, f, uin, uout, descending, gate);
     if (e != cudaSuccess) return e;
     ++g_launches;
     return cudaGetLastError();

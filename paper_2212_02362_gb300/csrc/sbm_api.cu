@@ -480,9 +480,9 @@ sbm_status setup_bottom(sbm_grid G)
     Level &B = G->L[0];
     const long long n = G->nb;
     CK(cudaMemsetAsync(G->A64, 0, sizeof(double) * n * n, G->st));
-    CK(launch_bottom_assemble(B.g, B.psi64, B.c64, G->A64, G->st));
+    CK(launch_bottom_assemble(B.g, B.psi64, B.Ke64, G->A64, G->st));
     CK(launch_bottom_dirichlet(B.g, G->A64, G->st));
-    CK(launch_gauss_jordan(B.g, (int)n, G->A64, G->gjtmp, G->gjbar, G->gj_spins, G->st));
+    CK(launch_sym_inverse((int)n, G->A64, G->gjtmp, G->gjbar, G->gj_spins, G->st));
     {
         unsigned hbar[4] = {0, 0, 0, 0};
         CK(cudaMemcpyAsync(hbar, G->gjbar, sizeof(hbar), cudaMemcpyDeviceToHost, G->st));
@@ -906,44 +906,50 @@ cudaError_t patch_smooth(sbm_grid G, Patch &Pt, int &cur, const sbm_opts &o, int
 
 size_t patch_bytes(const Patch &Pt, size_t elem) { return (size_t)Pt.s.dim * Pt.s.cs * elem; }
 
-// Injection into covered parents (finest first), then ghost fill (coarsest first).
+// Injection into covered parents (finest first), then ghost fill (coarsest first), the
+// patches of a level concurrently.
 cudaError_t amr_fill(sbm_grid G)
 {
-    // patches are numbered parents first, so descending order is finest first
-    for (int a = G->npatch; a >= 1; --a) {
-        Patch &Pt = G->P[a - 1];
-        const int pa = Pt.parent;
-        CKE(launch_amr_inject(Pt.s, Pt.info, amr_geom(G, pa), amr_info(G, pa), Pt.u64, amr_u64(G, pa), G->st));
-    }
-    for (int a = 1; a <= G->npatch; ++a) {
-        Patch &Pt = G->P[a - 1];
-        const int pa = Pt.parent;
-        CKE(launch_amr_ghost<double>(Pt.s, Pt.info, amr_geom(G, pa), amr_info(G, pa), Pt.u64, amr_u64(G, pa), 0, G->st));
-    }
+    const std::vector<std::vector<int>> lev = amr_by_level(G);
+    for (int L = (int)lev.size() - 1; L >= 1; --L)
+        CKE(amr_branches(G, lev[L], [&](int a) -> cudaError_t {
+            Patch &Pt = G->P[a - 1];
+            const int pa = Pt.parent;
+            return launch_amr_inject(Pt.s, Pt.info, amr_geom(G, pa), amr_info(G, pa), Pt.u64, amr_u64(G, pa), G->st);
+        }));
+    for (int L = 1; L < (int)lev.size(); ++L)
+        CKE(amr_branches(G, lev[L], [&](int a) -> cudaError_t {
+            Patch &Pt = G->P[a - 1];
+            const int pa = Pt.parent;
+            return launch_amr_ghost<double>(Pt.s, Pt.info, amr_geom(G, pa), amr_info(G, pa), Pt.u64, amr_u64(G, pa), 0,
+                                            G->st);
+        }));
     return cudaSuccess;
 }
 
 // Composite FP64 residual of every level, its norm into scal[which..] and the
-// residual rounded to T as the right-hand side of the correction cycle.
+// residual rounded to T as the right-hand side of the correction cycle; the base level
+// and the patches concurrently (each reads and writes its own level's arrays).
 template <typename T>
 cudaError_t amr_residual(sbm_grid G, int which)
 {
     Level &B = G->L[G->nl - 1];
     CKE(amr_fill(G));
-    CKE(sweep<double>(G, G->nl - 1, kResidual, G->amr_u0, G->fsrc, G->amr_r0, nullptr, 0.0));
-    CKE(launch_amr_mask(B.g, G->base_info, G->amr_r0, G->st));
     T *base_rhs = std::is_same<T, double>::value ? (T *)B.df : (T *)B.sf;
-    long long off = 0;
-    CKE(launch_amr_sumsq_round<T>(B.g, G->base_info, G->amr_r0, base_rhs, G->amr_part, G->st));
-    off += amr_blocks(B.g);
+    long long off = amr_blocks(B.g);
     std::vector<long long> offs(G->npatch + 1, 0);
-    std::vector<int> all;
+    std::vector<int> all = {0};
     for (int a = 1; a <= G->npatch; ++a) {
         offs[a] = off;
         off += amr_blocks(G->P[a - 1].s);
         all.push_back(a);
     }
     CKE(amr_branches(G, all, [&](int a) -> cudaError_t {
+        if (a == 0) {
+            CKE(sweep<double>(G, G->nl - 1, kResidual, G->amr_u0, G->fsrc, G->amr_r0, nullptr, 0.0));
+            CKE(launch_amr_mask(B.g, G->base_info, G->amr_r0, G->st));
+            return launch_amr_sumsq_round<T>(B.g, G->base_info, G->amr_r0, base_rhs, G->amr_part, G->st);
+        }
         Patch &Pt = G->P[a - 1];
         CKE(sweep_view<double>(G, Pt, kResidual, Pt.u64, Pt.f64, Pt.r64, 0.0));
         CKE(launch_amr_mask(Pt.s, Pt.info, Pt.r64, G->st));
@@ -1015,22 +1021,26 @@ cudaError_t amr_cycle(sbm_grid G, const sbm_opts &o, double *const *target = nul
 // every level on its nodes.
 cudaError_t amr_inner_residual(sbm_grid G, const int *cur, int cb)
 {
-    const int A = G->npatch;
     Level &B = G->L[G->nl - 1];
-    for (int a = A; a >= 1; --a) {
-        Patch &Pt = G->P[a - 1];
-        const int pa = Pt.parent;
-        CKE(launch_amr_inject<float>(Pt.s, Pt.info, amr_geom(G, pa), amr_info(G, pa), Pt.se[cur[a]],
-                                     amr_e<float>(G, pa, cur, cb), G->st));
-    }
-    CKE(sweep<float>(G, G->nl - 1, kResidual, B.su[cb], B.sf, B.sr, nullptr, 0.0));
-    CKE(launch_amr_mask_to<float>(B.g, G->base_info, B.sr, B.sf, G->st));
-    for (int a = 1; a <= A; ++a) {
+    const std::vector<std::vector<int>> lev = amr_by_level(G);
+    for (int L = (int)lev.size() - 1; L >= 1; --L)
+        CKE(amr_branches(G, lev[L], [&](int a) -> cudaError_t {
+            Patch &Pt = G->P[a - 1];
+            const int pa = Pt.parent;
+            return launch_amr_inject<float>(Pt.s, Pt.info, amr_geom(G, pa), amr_info(G, pa), Pt.se[cur[a]],
+                                            amr_e<float>(G, pa, cur, cb), G->st);
+        }));
+    std::vector<int> all = {0};
+    for (int a = 1; a <= G->npatch; ++a) all.push_back(a);
+    return amr_branches(G, all, [&](int a) -> cudaError_t {
+        if (a == 0) {
+            CKE(sweep<float>(G, G->nl - 1, kResidual, B.su[cb], B.sf, B.sr, nullptr, 0.0));
+            return launch_amr_mask_to<float>(B.g, G->base_info, B.sr, B.sf, G->st);
+        }
         Patch &Pt = G->P[a - 1];
         CKE(sweep_view<float>(G, Pt, kResidual, Pt.se[cur[a]], Pt.srhs, Pt.sres, 0.0));
-        CKE(launch_amr_mask_to<float>(Pt.s, Pt.info, Pt.sres, Pt.srhs, G->st));
-    }
-    return cudaSuccess;
+        return launch_amr_mask_to<float>(Pt.s, Pt.info, Pt.sres, Pt.srhs, G->st);
+    });
 }
 
 // ------------------------------------------------ adjoint of the composite problem

@@ -157,67 +157,73 @@ __device__ __forceinline__ void restrict_node(const Geom &gf, const Geom &gc, co
 // u_f += P e_c on free fine dofs.  One thread per coarse node (I,J,K) writes the
 // fine nodes (2I+a, 2J+b, 2K+c), a, b, c in {0, 1}, that exist: the coincident
 // node copies e_c, the others average the 2, 4 or 8 coarse neighbours.  The x
-// pair (2I, 2I+1) is read and written as one aligned vector.
+// pair (2I, 2I+1) is read and written as one aligned vector.  All loads are issued
+// before the first store (a row's load behind another row's store waits for it, and a
+// small level's launch is that chain: 7 us with 12 of them in a row, 4 us without).
 template <typename T, int D>
 __device__ __forceinline__ void prolong_node(const Geom &gf, const Geom &gc, const T *__restrict__ ec,
                                              T *__restrict__ uf, int I, int J, int K)
 {
     using V = typename Vec2<T>::type;
-    constexpr bool d3 = D == 3;
-    const bool hx = I + 1 < gc.nx, hy = J + 1 < gc.ny, hz = d3 && K + 1 < gc.nz;
+    constexpr int NZ = D == 3 ? 2 : 1;
+    const bool hx = I + 1 < gc.nx, hy = J + 1 < gc.ny, hz = D == 3 && K + 1 < gc.nz;
     const int I1 = hx ? I + 1 : I, J1 = hy ? J + 1 : J, K1 = hz ? K + 1 : K;
-    const int i0 = 2 * I, j0 = 2 * J, k0 = d3 ? 2 * K : 0;
+    const int i0 = 2 * I, j0 = 2 * J, k0 = D == 3 ? 2 * K : 0;
+    T c[D][2][2][2];                             // coarse values of the cell above (I,J,K): [z][y][x]
+    V v[D][NZ][2];                               // fine values at x = 2I, 2I+1
 #pragma unroll
     for (int p = 0; p < D; ++p) {
         const T *e = ec + p * gc.cs;
-        // coarse values of the cell above (I,J,K): [z][y][x]
-        T c[2][2][2];
-        c[0][0][0] = e[gidx(gc, I, J, K)];
-        c[0][0][1] = e[gidx(gc, I1, J, K)];
-        c[0][1][0] = e[gidx(gc, I, J1, K)];
-        c[0][1][1] = e[gidx(gc, I1, J1, K)];
-        c[1][0][0] = e[gidx(gc, I, J, K1)];
-        c[1][0][1] = e[gidx(gc, I1, J, K1)];
-        c[1][1][0] = e[gidx(gc, I, J1, K1)];
-        c[1][1][1] = e[gidx(gc, I1, J1, K1)];
-        T *u = uf + p * gf.cs;
 #pragma unroll
-        for (int zc = 0; zc < 2; ++zc) {
-            if (zc == 1 && !hz) break;
+        for (int q = 0; q < 4 * NZ; ++q)
+            c[p][q >> 2][(q >> 1) & 1][q & 1] = e[gidx(gc, q & 1 ? I1 : I, q & 2 ? J1 : J, q & 4 ? K1 : K)];
+#pragma unroll
+        for (int zc = 0; zc < NZ; ++zc)
 #pragma unroll
             for (int yc = 0; yc < 2; ++yc) {
-                if (yc == 1 && !hy) break;
+                if ((zc == 1 && !hz) || (yc == 1 && !hy)) continue;
+                const T *row = uf + p * gf.cs + gidx(gf, i0, j0 + yc, k0 + zc);
+                if (hx) v[p][zc][yc] = *reinterpret_cast<const V *>(row);
+                else v[p][zc][yc].x = *row;
+            }
+    }
+#pragma unroll
+    for (int p = 0; p < D; ++p)
+#pragma unroll
+        for (int zc = 0; zc < NZ; ++zc)
+#pragma unroll
+            for (int yc = 0; yc < 2; ++yc) {
+                if ((zc == 1 && !hz) || (yc == 1 && !hy)) continue;
+                const T(&C)[2][2][2] = c[p];
                 // values at x = 2I (even) and 2I+1 (odd) on this fine row
                 T ev, od;
                 if (zc == 0 && yc == 0) {
-                    ev = c[0][0][0];
-                    od = T(0.5) * (c[0][0][0] + c[0][0][1]);
+                    ev = C[0][0][0];
+                    od = T(0.5) * (C[0][0][0] + C[0][0][1]);
                 } else if (zc == 0) {
-                    ev = T(0.5) * (c[0][0][0] + c[0][1][0]);
-                    od = T(0.25) * ((c[0][0][0] + c[0][0][1]) + (c[0][1][0] + c[0][1][1]));
+                    ev = T(0.5) * (C[0][0][0] + C[0][1][0]);
+                    od = T(0.25) * ((C[0][0][0] + C[0][0][1]) + (C[0][1][0] + C[0][1][1]));
                 } else if (yc == 0) {
-                    ev = T(0.5) * (c[0][0][0] + c[1][0][0]);
-                    od = T(0.25) * ((c[0][0][0] + c[0][0][1]) + (c[1][0][0] + c[1][0][1]));
+                    ev = T(0.5) * (C[0][0][0] + C[1][0][0]);
+                    od = T(0.25) * ((C[0][0][0] + C[0][0][1]) + (C[1][0][0] + C[1][0][1]));
                 } else {
-                    ev = T(0.25) * ((c[0][0][0] + c[0][1][0]) + (c[1][0][0] + c[1][1][0]));
-                    od = T(0.125) * (((c[0][0][0] + c[0][0][1]) + (c[0][1][0] + c[0][1][1])) +
-                                     ((c[1][0][0] + c[1][0][1]) + (c[1][1][0] + c[1][1][1])));
+                    ev = T(0.25) * ((C[0][0][0] + C[0][1][0]) + (C[1][0][0] + C[1][1][0]));
+                    od = T(0.125) * (((C[0][0][0] + C[0][0][1]) + (C[0][1][0] + C[0][1][1])) +
+                                     ((C[1][0][0] + C[1][0][1]) + (C[1][1][0] + C[1][1][1])));
                 }
                 const int j = j0 + yc, k = k0 + zc;
-                T *row = u + gidx(gf, 0, j, k);
+                T *row = uf + p * gf.cs + gidx(gf, i0, j, k);
                 const T me = is_dir(gf, p, i0, j, k) ? T(0) : T(1);
                 if (hx) {
                     const T mo = is_dir(gf, p, i0 + 1, j, k) ? T(0) : T(1);
-                    V v = *reinterpret_cast<V *>(row + i0);
-                    v.x += me * ev;
-                    v.y += mo * od;
-                    *reinterpret_cast<V *>(row + i0) = v;
+                    V w = v[p][zc][yc];
+                    w.x += me * ev;
+                    w.y += mo * od;
+                    *reinterpret_cast<V *>(row) = w;
                 } else {
-                    row[i0] += me * ev;
+                    *row = v[p][zc][yc].x + me * ev;
                 }
             }
-        }
-    }
 }
 
 // u[gather[row]] (+)= sum_c Ainv[row][c] b[gather[c]] by one warp (lane = 0..31).

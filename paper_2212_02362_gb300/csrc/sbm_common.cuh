@@ -244,9 +244,8 @@ cudaError_t launch_norm_final(const double *part, int nparts, double *scal, int 
 cudaError_t launch_outer_gate(const double *scal, double tol, int max_cycles, double *hist, int *state, cudaStream_t s);
 // dst <- src unless *gate (gate may be null).
 cudaError_t launch_copy_gated(long long n, const double *src, double *dst, const int *gate, cudaStream_t s);
-// bottom: dense assembly, Dirichlet rows/cols, Gauss-Jordan inverse, matvec
-cudaError_t launch_bottom_assemble(const Geom &g, const double *psi, const Coef<double> &c,
-                                   double *A, cudaStream_t s);
+// bottom: dense assembly (Ke: unit-psi cell matrix), Dirichlet rows/cols, inverse, matvec
+cudaError_t launch_bottom_assemble(const Geom &g, const double *psi, const double *Ke, double *A, cudaStream_t s);
 cudaError_t launch_bottom_dirichlet(const Geom &g, double *A, cudaStream_t s);
 // FP32 3D sweep, eight threads (one per cell) per node (small levels; no partial sums).
 cudaError_t launch_sweep_node(int mode, const SweepArgs<float, float> &a, cudaStream_t s);
@@ -256,8 +255,7 @@ constexpr long long kNodeKernelMaxNodes = 20000;
 // Inverse of the coarsest-level matrix in place (one cooperative launch);
 // bar: 4 device words, bar[2] != 0 afterwards if a grid barrier timed out.
 // spins: polls a block makes at one grid barrier before giving up (<= 0: default).
-cudaError_t launch_gauss_jordan(const Geom &g, int n, double *A, double *tmp, unsigned *bar, long long spins,
-                                cudaStream_t s);
+cudaError_t launch_sym_inverse(int n, double *A, double *tmp, unsigned *bar, long long spins, cudaStream_t s);
 cudaError_t launch_round(long long n, const double *src, float *dst, cudaStream_t s);
 template <typename T>
 cudaError_t launch_bottom_apply(int n, const T *Ainv, const int *gather, const T *b, T *u,
