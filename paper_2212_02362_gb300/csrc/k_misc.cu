@@ -396,19 +396,17 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned nblocks, un
 // Measured with the assembly: 375 dofs 0.76 -> 0.23 ms, 720 dofs 2.15 -> 0.65 ms.
 constexpr int kGJB = 16;
 
-// 1 / d, d > 0, to an ulp: the FP32 reciprocal of the significand and two Newton steps
-// (r <- r + r (1 - m r)), the exponent by integer arithmetic.  The inversion below is a
-// chain of these; extreme exponents take the division.
+// 1 / d, d > 0, to an ulp: the hardware's approximate reciprocal (PTX rcp.approx.ftz.f64,
+// 2^-20) and two Newton steps r <- r + r (1 - d r).  The inversion below is a chain of
+// these; extreme exponents take the division.
 __device__ __forceinline__ double pivot_rcp(double d)
 {
-    const long long bits = __double_as_longlong(d);
-    const int ex = (int)(bits >> 52);
+    const int ex = (int)(__double_as_longlong(d) >> 52);
     if (ex < 64 || ex > 1980) return 1.0 / d;
-    const double m = __longlong_as_double((bits & 0xfffffffffffffll) | 0x3ff0000000000000ll);
-    double r = (double)__frcp_rn((float)m);
-    r = fma(r, fma(-m, r, 1.0), r);
-    r = fma(r, fma(-m, r, 1.0), r);
-    return __longlong_as_double(__double_as_longlong(r) - ((long long)(ex - 1023) << 52));
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    r = fma(r, fma(-d, r, 1.0), r);
+    return fma(r, fma(-d, r, 1.0), r);
 }
 
 // Inverse of the kGJB x kGJB SPD matrix in shared memory by one warp: lane (r, h) keeps
@@ -438,19 +436,21 @@ __device__ __forceinline__ void invert_pivot(double (*P)[kGJB + 1], int lane)
     for (int c = 0; c < 8; ++c) P[r][8 * h + c] = -v[c];
 }
 
+// PAN: the panel is staged in shared memory (else read from L2); in_smem: the block's
+// rows stay in shared memory.  kRowsMax rows a block at most have their B in shared memory
+// at once.
+constexpr int kRowsMax = 16;
+
+template <bool PAN>
 __global__ void __launch_bounds__(kThreads) k_sym_inverse(int n, double *A, double *tmp, unsigned *bar, int in_smem,
                                                           long long limit)
 {
-    // dynamic shared memory: the panel (in_smem bit 1, else read from L2), then, when
-    // in_smem bit 0, the block's rows
-    extern __shared__ double smem_gj[];
-    const bool pan_smem = (in_smem & 2) != 0;
-    in_smem &= 1;
-    double *srow = smem_gj + (pan_smem ? (long long)kGJB * n : 0);
+    extern __shared__ double smem_gj[];           // the panel (PAN), then the block's rows (in_smem)
+    double *srow = smem_gj + (PAN ? (long long)kGJB * n : 0);
     __shared__ double G[kGJB][kGJB + 1];
-    __shared__ double Brow[kThreads / 32][kGJB];
+    __shared__ double Brow[kRowsMax][kGJB];
     const unsigned nb = gridDim.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = kThreads / 32;
     const long long xb = (long long)kGJB * n;     // one exchange buffer: panel[r][i] = S[i][k0 + r]
     if (in_smem)
         for (int i = blockIdx.x, m = 0; i < n; i += gridDim.x, ++m)
@@ -479,47 +479,48 @@ __global__ void __launch_bounds__(kThreads) k_sym_inverse(int n, double *A, doub
             }
             __syncwarp();
             invert_pivot(G, lane);
-        } else if (pan_smem) {
+        } else if (PAN) {
 #pragma unroll 8
             for (int t = threadIdx.x - 32; t < b * n; t += kThreads - 32) smem_gj[t] = __ldcg(C + t);
+            for (int t = b * n + threadIdx.x - 32; t < kGJB * n; t += kThreads - 32) smem_gj[t] = 0.0;
         }
         __syncthreads();
-        auto cget = [&](long long idx) -> double { return pan_smem ? smem_gj[idx] : __ldcg(C + idx); };
-        // the warps take the rows' pieces of 32 columns in turn
-        int piece = 0;
-        for (int i = blockIdx.x, ri = 0; i < n; i += gridDim.x, ++ri) {
-            double *row = in_smem ? srow + (long long)ri * n : A + (long long)i * n;
-            const bool inP = i >= k0 && i < k0 + b;
-            const int np = i / 32 + 1;
-            // this warp's pieces of the row: p = warp - piece (mod nw)
-            const int p0 = ((warp - piece) % nw + nw) % nw;
-            piece += np;
-            if (p0 >= np) continue;
-            // B_i = S_iP G (rows outside P) or G's row (inside)
-            if (lane < kGJB) {
+        // rows b .. kGJB - 1 of the last panel count as zero
+        auto cget = [&](int c, int j) -> double {
+            return PAN ? smem_gj[c * n + j] : (c < b ? __ldcg(C + (long long)c * n + j) : 0.0);
+        };
+        for (int i0 = blockIdx.x, r0 = 0; i0 < n; i0 += kRowsMax * gridDim.x, r0 += kRowsMax) {
+            const int rows = min(kRowsMax, (n - i0 + (int)gridDim.x - 1) / (int)gridDim.x);
+            // B_i = S_iP G (rows outside P) or G's row (inside), half a warp a row
+            for (int m = threadIdx.x / kGJB; m < rows; m += kThreads / kGJB) {
+                const int i = i0 + m * gridDim.x, c = threadIdx.x % kGJB;
                 double acc[4] = {0.0, 0.0, 0.0, 0.0};
-                if (inP) {
-                    acc[0] = G[i - k0][lane];
+                if (i >= k0 && i < k0 + b) {
+                    acc[0] = G[i - k0][c];
                 } else {
 #pragma unroll
-                    for (int r = 0; r < kGJB; ++r)
-                        if (r < b) acc[r & 3] += cget((long long)r * n + i) * G[r][lane];
+                    for (int r = 0; r < kGJB; ++r) acc[r & 3] += cget(r, i) * G[r][c];
                 }
-                Brow[warp][lane] = lane < b ? (acc[0] + acc[1]) + (acc[2] + acc[3]) : 0.0;
+                Brow[m][c] = c < b ? (acc[0] + acc[1]) + (acc[2] + acc[3]) : 0.0;
             }
-            __syncwarp();
-            for (int p = p0; p < np; p += nw) {
-                const int j = p * 32 + lane;
-                if (j <= i) {
+            __syncthreads();
+            // the warps take the rows' pieces of 32 columns in turn
+            int next = warp;                                   // this warp's next piece, counted over the rows
+            for (int m = 0; m < rows; ++m) {
+                const int i = i0 + m * gridDim.x, np = i / 32 + 1;
+                double *row = in_smem ? srow + (long long)(r0 + m) * n : A + (long long)i * n;
+                const bool inP = i >= k0 && i < k0 + b;
+                for (; next < np; next += nw) {
+                    const int j = next * 32 + lane;
+                    if (j > i) continue;
                     const bool jP = j >= k0 && j < k0 + b;
                     double v;
                     if (jP) {
-                        v = inP ? -G[i - k0][j - k0] : Brow[warp][j - k0];
+                        v = inP ? -G[i - k0][j - k0] : Brow[m][j - k0];
                     } else {
                         double acc[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-                        for (int c = 0; c < kGJB; ++c)
-                            if (c < b) acc[c & 3] += Brow[warp][c] * cget((long long)c * n + j);
+                        for (int c = 0; c < kGJB; ++c) acc[c & 3] += Brow[m][c] * cget(c, j);
                         const double s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
                         v = inP ? s : row[j] - s;
                     }
@@ -527,8 +528,9 @@ __global__ void __launch_bounds__(kThreads) k_sym_inverse(int n, double *A, doub
                     if (j >= k1 && j < k1 + bn) Cn[(long long)(j - k1) * n + i] = v;
                     if (i >= k1 && i < k1 + bn) Cn[(long long)(i - k1) * n + j] = v;
                 }
+                next -= np;
             }
-            __syncwarp();
+            __syncthreads();
         }
         if (!grid_barrier(bar, nb, phase++, limit)) return;
         cur ^= 1;
@@ -774,23 +776,23 @@ cudaError_t launch_sym_inverse(int n, double *A, double *tmp, unsigned *bar, lon
     if (nblocks > n) nblocks = n;
     // the rows of each block in shared memory when they fit
     const size_t rows_bytes = (size_t)((n + nblocks - 1) / nblocks) * n * sizeof(double);
-    const size_t pivot_bytes = (size_t)kGJB * n * sizeof(double);
-    const bool piv = pivot_bytes <= 160 * 1024;                 // the pivot rows in shared memory
-    const bool rows = (piv ? pivot_bytes : 0) + rows_bytes <= 200 * 1024;
-    int in_smem = (rows ? 1 : 0) | (piv ? 2 : 0);
-    const size_t smem = (piv ? pivot_bytes : 0) + (rows ? rows_bytes : 0);
+    const size_t panel_bytes = (size_t)kGJB * n * sizeof(double);
+    const bool pan = panel_bytes <= 160 * 1024;                 // the panel in shared memory
+    int in_smem = (pan ? panel_bytes : 0) + rows_bytes <= 200 * 1024;
+    const size_t smem = (pan ? panel_bytes : 0) + (in_smem ? rows_bytes : 0);
+    const void *kernel = pan ? (const void *)k_sym_inverse<true> : (const void *)k_sym_inverse<false>;
     if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(k_sym_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sym_inverse, kThreads, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem);
     if (e != cudaSuccess) return e;
     if (!coop || per_sm < 1) return cudaErrorNotSupported;
     e = cudaMemsetAsync(bar, 0, 4 * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     long long limit = spins > 0 ? spins : kGridSpinLimit;
     void *args[] = {&n, &A, &tmp, &bar, &in_smem, &limit};
-    e = cudaLaunchCooperativeKernel((const void *)k_sym_inverse, dim3(nblocks), dim3(kThreads), args, smem, s);
+    e = cudaLaunchCooperativeKernel(kernel, dim3(nblocks), dim3(kThreads), args, smem, s);
     ++g_launches;
     return e;
 }

@@ -70,6 +70,13 @@ __device__ __forceinline__ void block_partial(double ssq, double *out, double *r
     }
 }
 
+// Index of cell (i, j, k) in a.psi.
+template <typename TO>
+__device__ __forceinline__ long long pidx(const SweepArgs<double, TO> &a, int i, int j, int k)
+{
+    return i + (long long)(a.psx ? a.psx : a.g.sx) * j + (a.psx ? a.psy : a.g.sy) * k;
+}
+
 // One tile's share of the grid for this thread.
 struct Tile {
     int x0, y0;            // first owned node
@@ -163,7 +170,7 @@ __device__ __noinline__ double sweep_dp(const SweepArgs<double, TO> &a, long lon
             }
         };
         auto cell_psi = [&](int lz) {
-            return (T.cell_ok && lz <= g.nz - 2) ? a.psi[gidx(g, T.gx - 1, T.gy - 1, lz)] : 0.0;
+            return (T.cell_ok && lz <= g.nz - 2) ? a.psi[pidx(a, T.gx - 1, T.gy - 1, lz)] : 0.0;
         };
         double Tb[3][4], Cf[3][4];
 #pragma unroll
@@ -301,7 +308,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
         su += kend + 1 - kz0;
         const int kfirst = kz0 > 0 ? kz0 - 1 : 0;
         auto cell_psi = [&](int lz) {
-            return (T.cell_ok && lz <= g.nz - 2) ? a.psi[gidx(g, T.gx - 1, T.gy - 1, lz)] : 0.0;
+            return (T.cell_ok && lz <= g.nz - 2) ? a.psi[pidx(a, T.gx - 1, T.gy - 1, lz)] : 0.0;
         };
         const Stage S = make_stage(g, T);
         // planes kfirst, kfirst + 1 as integers, kfirst + 2 with its key, kfirst + 3 on its way
@@ -441,8 +448,6 @@ constexpr int TX2 = 32;
 template <typename TO, int MODE, int TY2>
 __global__ void __launch_bounds__((TX2 + 1) * (TY2 + 1)) k_sweep2_fix(const SweepArgs<double, TO> a, const fix::Consts fc)
 {
-    pdl_begin();
-    if (a.gate && *a.gate) return;
     constexpr int BX2 = TX2 + 1, BY2 = TY2 + 1, NT2 = BX2 * BY2, PX2 = TX2 + 2, PP2 = PX2 * (TY2 + 2);
     __shared__ i64 X[2][4][PP2];                   // corner forces (integers, or doubles where they do not fit)
     __shared__ int Xe[PP2];
@@ -463,6 +468,12 @@ __global__ void __launch_bounds__((TX2 + 1) * (TY2 + 1)) k_sweep2_fix(const Swee
     const bool own = gx < g.nx && gy < g.ny && (tx < TX2 || gx == g.nx - 1) && (ty < TY2 || gy == g.ny - 1);
     const bool cell_ok = gx >= 1 && gx < g.nx && gy >= 1 && gy < g.ny;
     const long long on = gidx(g, gx, gy, 0);
+    // what no kernel of the cycle writes is read before the wait for the predecessor
+    if (a.foreign_psi) pdl_wait();
+    const double psi = cell_ok ? a.psi[pidx(a, gx - 1, gy - 1, 0)] : 0.0;
+    double ip = (MODE == kJacobi && a.dinv && own) ? a.dinv[on] : 0.0;
+    pdl_begin();
+    if (a.gate && *a.gate) return;
     double D[2][4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -472,13 +483,11 @@ __global__ void __launch_bounds__((TX2 + 1) * (TY2 + 1)) k_sweep2_fix(const Swee
 #pragma unroll
         for (int p = 0; p < 2; ++p) D[p][q] = ok ? a.u[p * g.cs + o] : 0.0;
     }
-    const double psi = cell_ok ? a.psi[gidx(g, gx - 1, gy - 1, 0)] : 0.0;
     double fv[2] = {0.0, 0.0};
     if (MODE != kApply && own) {
         fv[0] = a.f[on];
         fv[1] = a.f[g.cs + on];
     }
-    double ip = (MODE == kJacobi && a.dinv && own) ? a.dinv[on] : 0.0;
     const double uv[2] = {D[0][3], D[1][3]};
     const int me = ty * PX2 + tx;
     unsigned key = 0;
@@ -560,19 +569,38 @@ __global__ void __launch_bounds__(kGsThreads) k_gs2_fix(const Geom g, const fix:
                                                         const double *__restrict__ f, const double *__restrict__ uin,
                                                         double *__restrict__ uout, int descending, const int *gate)
 {
-    pdl_begin();
-    if (gate && *gate) return;
     constexpr int H = 4, SN = TILE + 2 * H, SC = SN - 1, SF = SN - 2;
     constexpr int NQ = (TILE + 6) / 2 * ((TILE + 6) / 2);  // nodes of the largest phase
     constexpr int kBad = 1 << 20;                          // exponent of a cell that does not fit
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *su = reinterpret_cast<double *>(smem_raw);   // [2][SN][SN] staged nodes
     double *sf = su + 2 * SN * SN;                        // [2][SF][SF] right-hand side of staged nodes 1 .. SN-2
-    double *sp = sf + 2 * SF * SF;                        // [SC][SC] psi of the staged cells (0 outside the grid)
+    double *sw = sf + 2 * SF * SF;                        // [2][SF][SF] 1 / diagonal and coupling of the node's block
+    double *sp = sw + 2 * SF * SF;                        // [SC][SC] psi of the staged cells (0 outside the grid)
     i64 *X = reinterpret_cast<i64 *>(sp + SC * SC);       // [4][2][NQ] corner forces of a phase
     int *Xe = reinterpret_cast<int *>(X + 8 * NQ);        // [4][NQ] their exponents
     const int tid = threadIdx.x, nt = kGsThreads;
     const int x0 = blockIdx.x * TILE - H, y0 = blockIdx.y * TILE - H;   // global node of staged (0, 0)
+    // psi and the diagonal blocks, which no kernel of the cycle writes, before the wait for
+    // the predecessor: the divisions run while it drains
+    for (int s = tid; s < SC * SC; s += nt) {
+        const int i = x0 + s % SC, j = y0 + s / SC;
+        const bool ok = i >= 0 && i < g.nx - 1 && j >= 0 && j < g.ny - 1;
+        sp[s] = ok ? psi[gidx(g, i, j, 0)] : 0.0;
+    }
+    const double kd = Ke[0], k01 = Ke[1];                 // corner 0: diagonal and coupling
+    __syncthreads();
+    for (int s = tid; s < SF * SF; s += nt) {
+        const int lx = s % SF, ly = s / SF;               // cells below and above staged node (lx + 1, ly + 1)
+        const double p3 = sp[ly * SC + lx], p2 = sp[ly * SC + lx + 1], p1 = sp[(ly + 1) * SC + lx],
+                     p0 = sp[(ly + 1) * SC + lx + 1];
+        const int i = x0 + 1 + lx, j = y0 + 1 + ly;
+        if (i < 0 || i >= g.nx || j < 0 || j >= g.ny) continue;
+        sw[s] = 1.0 / (kd * ((p0 + p1) + (p2 + p3)));
+        sw[SF * SF + s] = k01 * ((p0 + p3) - (p1 + p2));
+    }
+    pdl_begin();
+    if (gate && *gate) return;
     for (int s = tid; s < SN * SN; s += nt) {
         const int i = x0 + s % SN, j = y0 + s / SN;
         const bool ok = i >= 0 && i < g.nx && j >= 0 && j < g.ny;
@@ -587,12 +615,6 @@ __global__ void __launch_bounds__(kGsThreads) k_gs2_fix(const Geom g, const fix:
         sf[s] = ok ? f[o] : 0.0;
         sf[SF * SF + s] = ok ? f[g.cs + o] : 0.0;
     }
-    for (int s = tid; s < SC * SC; s += nt) {
-        const int i = x0 + s % SC, j = y0 + s / SC;
-        const bool ok = i >= 0 && i < g.nx - 1 && j >= 0 && j < g.ny - 1;
-        sp[s] = ok ? psi[gidx(g, i, j, 0)] : 0.0;
-    }
-    const double kd = Ke[0], k01 = Ke[1];                 // corner 0: diagonal and coupling
     __syncthreads();
     for (int q = 0; q < 4; ++q) {
         const int c = descending ? 3 - q : q;
@@ -633,11 +655,10 @@ __global__ void __launch_bounds__(kGsThreads) k_gs2_fix(const Geom g, const fix:
             const int i = x0 + lx, j = y0 + ly;
             if (i < 0 || j < 0 || i >= g.nx || j >= g.ny) continue;
             const int me = ly * SN + lx, mf = (ly - 1) * SF + lx - 1;
-            double pc[4];                                 // cell a: the node is its corner a
+            const double w = sw[mf], s01 = sw[SF * SF + mf];
             int e[4], ee = fix::kNoExp;
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                pc[a] = sp[(ly - (a >> 1)) * SC + lx - (a & 1)];
                 e[a] = Xe[a * NQ + n];
                 ee = max(ee, e[a]);
             }
@@ -657,11 +678,9 @@ __global__ void __launch_bounds__(kGsThreads) k_gs2_fix(const Geom g, const fix:
                             for (int r = 0; r < 2; ++r)
                                 t = madd(Ke[(a * 2 + p) * 8 + b * 2 + r],
                                          su[r * SN * SN + me + ((b >> 1) - (a >> 1)) * SN + (b & 1) - (a & 1)], t);
-                        Ku[p] = madd(pc[a], t, Ku[p]);
+                        Ku[p] = madd(sp[(ly - (a >> 1)) * SC + lx - (a & 1)], t, Ku[p]);
                     }
             }
-            const double w = 1.0 / (kd * ((pc[0] + pc[1]) + (pc[2] + pc[3])));
-            const double s01 = k01 * ((pc[0] + pc[3]) - (pc[1] + pc[2]));
             if (!is_dir(g, 0, i, j, 0)) {
                 const double du = (sf[mf] - Ku[0]) * w;
                 su[me] += du;
@@ -686,7 +705,7 @@ cudaError_t launch_gs2_tile(const Geom &g, const fix::Consts &fc, const double *
                             const double *uin, double *uout, int descending, cudaStream_t s, const int *gate)
 {
     constexpr int SN = TILE + 8, NQ = (TILE + 6) / 2 * ((TILE + 6) / 2);
-    constexpr size_t sm = sizeof(double) * (2 * SN * SN + 2 * (SN - 2) * (SN - 2) + (SN - 1) * (SN - 1) + 8 * NQ) +
+    constexpr size_t sm = sizeof(double) * (2 * SN * SN + 4 * (SN - 2) * (SN - 2) + (SN - 1) * (SN - 1) + 8 * NQ) +
                           sizeof(int) * 4 * NQ;
     static std::atomic<unsigned long long> attr_done{0};
     cudaError_t e = smem_attr_once(reinterpret_cast<const void *>(k_gs2_fix<TILE>), sm, attr_done);

@@ -1875,6 +1875,37 @@ sbm_status sbm_adjoint(sbm_grid G, const double *u, const double *dJdu, double *
 
 // ------------------------------------------------------------------ steps
 
+// FP64 apply / residual of a level on the caller's packed arrays: the sweep takes their
+// strides, so nothing is copied into the level's layout and back (half of the time of a
+// 129^3 residual).  out must not overlap its inputs (packed_apart).
+static cudaError_t sweep_packed(sbm_grid G, int level, int mode, const double *u, const double *f, double *out,
+                                double *part)
+{
+    const Level &L = G->L[level];
+    SweepArgs<double, double> a;
+    a.g = L.g;
+    a.g.sx = L.g.nx;
+    a.g.sy = (long long)L.g.nx * L.g.ny;
+    a.g.cs = nnodes(L.g);
+    a.psx = L.g.sx;
+    a.psy = L.g.sy;
+    a.u = u;
+    a.f = f;
+    a.psi = L.psi64;
+    a.out = out;
+    a.part = part;
+    a.c = L.c64;
+    a.wk[0] = a.wk[1] = a.wk[2] = 0.0;
+    a.kchunk = 0;
+    return launch_sweep<double, double>(mode, a, G->st);
+}
+
+static bool packed_apart(const Level &L, const double *a, const double *b)
+{
+    const long long n = (long long)L.g.dim * nnodes(L.g);
+    return a + n <= b || b + n <= a;
+}
+
 sbm_status sbm_apply(sbm_grid G, int level, int fp32, const double *u, double *Ku)
 {
     sbm_status s = check_level(G, level);
@@ -1887,6 +1918,8 @@ sbm_status sbm_apply(sbm_grid G, int level, int fp32, const double *u, double *K
         CK(launch_pack<double, float>(L.g, L.g.dim, u, L.su[1], G->st));
         CK(sweep<float>(G, level, kApply, L.su[1], nullptr, L.sr, nullptr, 0.0));
         CK(launch_unpack<float, double>(L.g, L.g.dim, L.sr, Ku, G->st));
+    } else if (packed_apart(L, u, Ku)) {
+        CK(sweep_packed(G, level, kApply, u, nullptr, Ku, nullptr));
     } else {
         CK(launch_pack<double, double>(L.g, L.g.dim, u, L.du[1], G->st));
         CK(sweep<double>(G, level, kApply, L.du[1], nullptr, L.dr, nullptr, 0.0));
@@ -1912,6 +1945,8 @@ sbm_status sbm_residual(sbm_grid G, int level, int fp32, const double *f, const 
         CK(launch_pack<double, float>(L.g, L.g.dim, f, L.sf, G->st));
         CK(sweep<float>(G, level, kResidual, L.su[1], L.sf, L.sr, G->part, 0.0));
         CK(launch_unpack<float, double>(L.g, L.g.dim, L.sr, r, G->st));
+    } else if (packed_apart(L, u, r) && packed_apart(L, f, r)) {
+        CK(sweep_packed(G, level, kResidual, u, f, r, G->part));
     } else {
         CK(launch_pack<double, double>(L.g, L.g.dim, u, L.du[1], G->st));
         CK(launch_pack<double, double>(L.g, L.g.dim, f, L.df, G->st));

@@ -64,9 +64,13 @@ __device__ __forceinline__ void row_warp_xy(int tid, int &tx, int &ty)
 // its predecessor drains; each of them first waits for its predecessor to
 // complete (griddepcontrol.wait: memory visible) and then lets its own successor
 // be scheduled.  Launched without the attribute, both are no-ops.
+// What a kernel reads before its wait must have been written by launches before its
+// predecessor: those are complete, since the predecessor passed its own wait.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ void pdl_begin()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
@@ -102,6 +106,12 @@ struct SweepArgs {
     int kchunk;            // node planes per block along z (3D)
     const int *gate = nullptr;   // device flag: when set, the launch does nothing
     const T *dinv = nullptr;     // FP64 Jacobi: 1 / (psi sum of the node's cells), or null (formed in the sweep)
+    // FP64 sweeps: strides of psi where they are not g's (0: they are), and whether the
+    // launch before this one may write psi (a caller's array) - the kernels otherwise read
+    // psi before they wait for their predecessor
+    int psx = 0;
+    long long psy = 0;
+    bool foreign_psi = false;
 };
 
 // Number of z chunks for a z-streaming stencil launch: minimises

@@ -96,6 +96,7 @@ extern "C" sbm_status sbm_residual_noalloc(int dim, const int n[3], double h, co
     a.c = make_coef<double>(dim, h, moduli[0], moduli[1], moduli[2]);
     a.wk[0] = a.wk[1] = a.wk[2] = 0.0;
     a.kchunk = 0;
+    a.foreign_psi = true;
     if ((e = launch_sweep<double, double>(kResidual, a, st)) != cudaSuccess) return fail(SBM_ERR_CUDA, cudaGetErrorString(e));
     double *res = scratch + SBM_NOALLOC_MAX_BLOCKS;
     if ((e = launch_norm_final(scratch, (int)nblocks, res, 0, st)) != cudaSuccess) return fail(SBM_ERR_CUDA, cudaGetErrorString(e));

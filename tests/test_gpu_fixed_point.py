@@ -146,3 +146,22 @@ def test_solve_after_a_new_psi(dim, n):
         u, v = cuda(wk.u0), cuda(wk.u0)
         a, b = g.solve(u, omega=0.5), fresh.solve(v, omega=0.5)
         assert a.cycles == b.cycles and np.array_equal(host(u), host(v))
+
+
+@pytest.mark.parametrize("dim,n", [(2, (41, 33)), (3, (19, 13, 11))])
+def test_steps_on_overlapping_arrays(dim, n):
+    """apply and residual read and write the caller's arrays in place of copies; an output
+    that is one of the inputs gives the same values as one that is not."""
+    import paper_2212_02362_gb300 as sbm
+    wk = random_workload(dim, n, 120)
+    g, P = gpu_grid(wk), oracle_problem(wk)
+    u, f = cuda(W.uniform(121, P.ndofs, -1, 1)), cuda(wk.f)
+    ref, (r, nrm) = g.apply(g.finest, u), g.residual(g.finest, f, u)
+    import ctypes as C
+    v = u.clone()
+    assert sbm.lib().sbm_apply(g._h, g.finest, 0, v.data_ptr(), v.data_ptr()) == 0 and torch.equal(v, ref)
+    for inout in (u.clone(), f.clone()):
+        a, b = (f, inout) if torch.equal(inout, u) else (inout, u)
+        norm = C.c_double()
+        st = sbm.lib().sbm_residual(g._h, g.finest, 0, a.data_ptr(), b.data_ptr(), inout.data_ptr(), C.byref(norm))
+        assert st == 0 and torch.equal(inout, r) and norm.value == nrm
