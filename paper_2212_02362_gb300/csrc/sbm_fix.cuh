@@ -198,17 +198,23 @@ __host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], cons
             mh |= mag_hi(U[p][s + 4]);
         }
     unsigned long long m = (unsigned long long)mh << 32 | 0xffffffffu;
+    bool none = false;
     if (mh == 0u) {                          // all below 2^32: the low words decide
+        i64 any = 0;
         m = 0;
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
-            for (int s = 1; s < 8; ++s) m |= (unsigned long long)(U[p][s] ^ (U[p][s] >> 63));
+            for (int s = 1; s < 8; ++s) {
+                any |= U[p][s];
+                m |= (unsigned long long)(U[p][s] ^ (U[p][s] >> 63));   // 0 for -1 as for 0
+            }
+        none = any == 0;
     }
     int ep;
     const i64 pm = psi_mantissa(psi, ep);
     int sh = norm_shift(m);
-    e = (m == 0ull || pm == 0) ? kNoExp : E - kFixUnit - sh + ep + c.ec;
+    e = (none || pm == 0) ? kNoExp : E - kFixUnit - sh + ep + c.ec;
     if (sh < 0) {                            // sums of opposite corners near the bound
         sh += 3;
 #pragma unroll
@@ -256,19 +262,23 @@ __host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], cons
 }
 
 // The six transformed values of a 2D cell that carry force, in the order U[0][1..3],
-// U[1][1..3] of bfly4, shifted up to 2^61 at most.  Returns the shift; m = 0: all zero.
+// U[1][1..3] of bfly4, shifted up to 2^61 at most.  Returns the shift.
 __host__ __device__ __forceinline__ int transform2(const i64 (&u)[2][4], i64 (&U)[2][4], bool &none)
 {
     unsigned long long m = 0;
+    i64 any = 0;
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) U[p][q] = u[p][q];
         bfly4(U[p]);
 #pragma unroll
-        for (int q = 1; q < 4; ++q) m |= (unsigned long long)(U[p][q] ^ (U[p][q] >> 63));
+        for (int q = 1; q < 4; ++q) {
+            any |= U[p][q];
+            m |= (unsigned long long)(U[p][q] ^ (U[p][q] >> 63));   // 0 for -1 as for 0
+        }
     }
-    none = m == 0ull;
+    none = any == 0;
     const int sh = norm_shift(m);            // |U| <= 4 2^60: at least -2
 #pragma unroll
     for (int p = 0; p < 2; ++p)

@@ -165,3 +165,20 @@ def test_steps_on_overlapping_arrays(dim, n):
         norm = C.c_double()
         st = sbm.lib().sbm_residual(g._h, g.finest, 0, a.data_ptr(), b.data_ptr(), inout.data_ptr(), C.byref(norm))
         assert st == 0 and torch.equal(inout, r) and norm.value == nrm
+
+
+@pytest.mark.parametrize("dim,n", [(2, (65, 33)), (3, (25, 9, 9))])
+def test_decaying_field(dim, n):
+    """A displacement that decays from one node over thirty decades: cells whose values
+    are a unit or two of the integer form, of either sign."""
+    wk = random_workload(dim, n, 130)
+    g, P = gpu_grid(wk), oracle_problem(wk)
+    psi = oracle.floor_psi(wk.psi, wk.psi_min)
+    X = W.node_coords(dim, wk.n, wk.h)
+    r2 = sum((X[a] - c) ** 2 for a, c in zip(range(dim), (0.9, 0.2, 0.2)))
+    for rate in (20.0, 60.0, 85.0):
+        u = np.concatenate([s * np.exp(-rate * r2) for s in (0.0, -1.0, 0.3)[:dim]])
+        assert _rel(host(g.apply(g.finest, cuda(u))), oracle.apply(P, psi, u)) <= 1e-13
+        if dim == 2:
+            ref = oracle.gs_sweep(P, psi, wk.f, u)
+            assert _rel(host(g.smooth(g.finest, cuda(wk.f), cuda(u), "gs")) - u, ref - u) <= 1e-11
