@@ -35,20 +35,28 @@ inline dim3 node_grid(const Geom &g)
     return dim3((g.nx + 31) / 32, (g.ny + 3) / 4, (g.nz + 1) / 2);
 }
 
-// zero_uc (may be null): the coarse correction, zeroed at each coarse node (the
-// start of the coarse level's cycle).
+// zero_uc (may be null): the coarse correction, zeroed at each coarse node (the start of
+// the coarse level's cycle); first: instead, its first Jacobi sweep, which from zero needs
+// no stencil (one launch of five to eight a level and cycle less).  The Jacobi scaling is
+// formed before the wait for the predecessor, which does not write psi.
 template <typename T, int D>
 __global__ void k_restrict(const Geom gf, const Geom gc, const T *__restrict__ rf, T *__restrict__ fc, const int *gate,
-                           T *__restrict__ zero_uc)
+                           T *__restrict__ zero_uc, const FirstSweep<T> first)
 {
-    pdl_begin();
-    if (gate && *gate) return;
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     const int J = blockIdx.y * blockDim.y + threadIdx.y;
     const int K = blockIdx.z * blockDim.z + threadIdx.z;
-    if (I >= gc.nx || J >= gc.ny || K >= gc.nz) return;
-    body::restrict_node<T, D>(gf, gc, rf, fc, I, J, K);
-    if (zero_uc) {
+    const bool in = I < gc.nx && J < gc.ny && K < gc.nz;
+    T ip = T(0);
+    if (first.u && in) ip = first.dinv ? first.dinv[gidx(gc, I, J, K)] : body::inv_psi_sum<T, D>(gc, first.psi, I, J, K);
+    pdl_begin();
+    if (gate && *gate) return;
+    if (!in) return;
+    T f[D];
+    body::restrict_node<T, D>(gf, gc, rf, fc, I, J, K, f);
+    if (first.u) {
+        body::first_sweep<T, D>(first, gc, I, J, K, ip, f);
+    } else if (zero_uc) {
         const long long o = gidx(gc, I, J, K);
         for (int p = 0; p < D; ++p) zero_uc[p * gc.cs + o] = T(0);
     }
@@ -611,18 +619,19 @@ __global__ void k_dJdpsi(const Geom g, const Coef<double> c, const double *__res
 
 template <typename T>
 cudaError_t launch_restrict(const Geom &gf, const Geom &gc, const T *rf, T *fc, cudaStream_t s, const int *gate,
-                            T *zero_uc)
+                            T *zero_uc, const FirstSweep<T> &first)
 {
-    cudaError_t e = gf.dim == 3 ? launch_pdl(k_restrict<T, 3>, node_grid(gc), kNodeBlock, 0, s, gf, gc, rf, fc, gate, zero_uc)
-                                : launch_pdl(k_restrict<T, 2>, node_grid(gc), kNodeBlock, 0, s, gf, gc, rf, fc, gate, zero_uc);
+    cudaError_t e = gf.dim == 3
+                        ? launch_pdl(k_restrict<T, 3>, node_grid(gc), kNodeBlock, 0, s, gf, gc, rf, fc, gate, zero_uc, first)
+                        : launch_pdl(k_restrict<T, 2>, node_grid(gc), kNodeBlock, 0, s, gf, gc, rf, fc, gate, zero_uc, first);
     if (e != cudaSuccess) return e;
     ++g_launches;
     return cudaGetLastError();
 }
 template cudaError_t launch_restrict<double>(const Geom &, const Geom &, const double *, double *, cudaStream_t,
-                                             const int *, double *);
+                                             const int *, double *, const FirstSweep<double> &);
 template cudaError_t launch_restrict<float>(const Geom &, const Geom &, const float *, float *, cudaStream_t, const int *,
-                                            float *);
+                                            float *, const FirstSweep<float> &);
 
 template <typename T>
 cudaError_t launch_prolong_add(const Geom &gf, const Geom &gc, const T *ec, T *uf, cudaStream_t s, const int *gate)

@@ -437,13 +437,42 @@ long long sweep_blocks(const Geom &g, bool fp64)
 // shared memory, no barrier and no z streaming, and each thread's dependent
 // chain is one cell: on coarse levels, whose cost is latency, a launch takes
 // little more than one cell evaluation.
+// The PRO form adds the prolongation of the coarse correction to the values as it reads
+// them (a prolongation launch less), and k_resid_restrict fuses a level's residual with
+// its full weighting and the coarse level's first sweep: a block takes one coarse node,
+// 27 groups of eight threads its fine nodes' residuals (3.4x the arithmetic of the
+// residual alone, which on these levels is nothing beside a launch), a warp the weighted
+// sum.  Measured on one V-cycle of the 129^3 hierarchy with the first sweeps in the
+// restriction: see launch_restrict.
 constexpr int kNodeThreads = 256;
 
-template <int MODE>
-__global__ void __launch_bounds__(kNodeThreads) k_sweep3_node(const SweepArgs<float, float> a)
+// Forces and psi of a node summed over its group of eight lanes; own: the node's values
+// from a lane that has a cell.
+template <bool PRO>
+__device__ __forceinline__ void node_sum(const SweepArgs<float, float> &a, bool valid, int i, int j, int k, int c,
+                                         bool has, const Geom &gc, const float *ec, float (&F)[3], float (&own)[3],
+                                         float &ps)
 {
-    pdl_begin();
-    if (a.gate && *a.gate) return;
+    F[0] = F[1] = F[2] = own[0] = own[1] = own[2] = 0.f;
+    if (valid && has) body::node_cell<PRO>(a, i, j, k, c, ps, gc, ec, F, own);
+    // every lane takes part in the sums; the xor partners stay in the group of eight
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) {
+#pragma unroll
+        for (int p = 0; p < 3; ++p) F[p] += __shfl_xor_sync(0xffffffffu, F[p], off);
+        ps += __shfl_xor_sync(0xffffffffu, ps, off);
+    }
+    const int base = threadIdx.x & 24;
+    const unsigned m = (__ballot_sync(0xffffffffu, has) >> base) & 0xffu;
+    const int src = base + (m ? __ffs(m) - 1 : 0);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) own[p] = __shfl_sync(0xffffffffu, own[p], src);
+}
+
+template <int MODE, bool PRO>
+__global__ void __launch_bounds__(kNodeThreads) k_sweep3_node(const SweepArgs<float, float> a, const Geom gc,
+                                                              const float *__restrict__ ec)
+{
     const Geom &g = a.g;
     const long long n = (long long)g.nx * g.ny * g.nz;
     const long long node = (long long)blockIdx.x * (kNodeThreads / 8) + (threadIdx.x >> 3);
@@ -456,34 +485,93 @@ __global__ void __launch_bounds__(kNodeThreads) k_sweep3_node(const SweepArgs<fl
         j = (int)(t % g.ny);
         k = (int)(t / g.ny);
     }
-    float F[3] = {0.f, 0.f, 0.f}, ps = 0.f;
-    if (valid) body::node_cell(a, i, j, k, c, F, ps);
-    // every lane takes part in the sums; the xor partners stay in the group of eight
-#pragma unroll
-    for (int off = 4; off > 0; off >>= 1) {
-#pragma unroll
-        for (int p = 0; p < 3; ++p) F[p] += __shfl_xor_sync(0xffffffffu, F[p], off);
-        ps += __shfl_xor_sync(0xffffffffu, ps, off);
-    }
+    float F[3], own[3], ps = 0.f;
+    const bool has = valid && body::node_psi(a, i, j, k, c, ps);   // psi before the wait: no kernel of the cycle writes it
+    pdl_begin();
+    if (a.gate && *a.gate) return;
+    node_sum<PRO>(a, valid, i, j, k, c, has, gc, ec, F, own, ps);
     if (valid && c == 0) {
-        const long long o = gidx(g, i, j, k);
-        const float uv[3] = {a.u[o], a.u[g.cs + o], a.u[2 * g.cs + o]};
         double ssq = 0.0;
-        body::finalize<float, float, MODE>(a, i, j, k, F, ps, uv, ssq);
+        body::finalize<float, float, MODE>(a, i, j, k, F, ps, own, ssq);
     }
+}
+
+__global__ void __launch_bounds__(224) k_resid_restrict(const SweepArgs<float, float> a, const Geom gc,
+                                                        float *__restrict__ fc, const FirstSweep<float> first)
+{
+    __shared__ float R[27][3];
+    const Geom &g = a.g;
+    const int I = blockIdx.x, J = blockIdx.y, K = blockIdx.z;
+    const int q = threadIdx.x >> 3, c = threadIdx.x & 7;         // fine node of the 27, corner
+    const int i = 2 * I + q % 3 - 1, j = 2 * J + q / 3 % 3 - 1, k = 2 * K + q / 9 - 1;
+    const bool valid = q < 27 && i >= 0 && j >= 0 && k >= 0 && i < g.nx && j < g.ny && k < g.nz;
+    float F[3], own[3], ps = 0.f;
+    const bool has = valid && body::node_psi(a, i, j, k, c, ps);
+    const float ip = first.u && threadIdx.x < 32 ? body::inv_psi_sum<float, 3>(gc, first.psi, I, J, K) : 0.f;
+    pdl_begin();
+    if (a.gate && *a.gate) return;
+    node_sum<false>(a, valid, i, j, k, c, has, g, nullptr, F, own, ps);
+    if (q < 27 && c == 0) {
+        const long long o = valid ? gidx(g, i, j, k) : 0;
+#pragma unroll
+        for (int p = 0; p < 3; ++p) R[q][p] = (!valid || is_dir(g, p, i, j, k)) ? 0.f : a.f[p * g.cs + o] - F[p];
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int l = threadIdx.x;
+        const float w = l < 27 ? 1.f / (float)(1 << ((l % 3 != 1) + (l / 3 % 3 != 1) + (l / 9 != 1))) : 0.f;
+        float s[3];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+            s[p] = l < 27 ? w * R[l][p] : 0.f;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) s[p] += __shfl_xor_sync(0xffffffffu, s[p], off);
+            s[p] = is_dir(gc, p, I, J, K) ? 0.f : 0.125f * s[p];
+        }
+        if (l == 0) {
+            const long long o = gidx(gc, I, J, K);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) fc[p * gc.cs + o] = s[p];
+            if (first.u) body::first_sweep<float, 3>(first, gc, I, J, K, ip, s);
+        }
+    }
+}
+
+static dim3 node_blocks(const Geom &g)
+{
+    return dim3((unsigned)(((long long)g.nx * g.ny * g.nz + kNodeThreads / 8 - 1) / (kNodeThreads / 8)));
 }
 
 cudaError_t launch_sweep_node(int mode, const SweepArgs<float, float> &a, cudaStream_t s)
 {
-    const long long n = (long long)a.g.nx * a.g.ny * a.g.nz;
-    const dim3 b(kNodeThreads), gr((unsigned)((n + kNodeThreads / 8 - 1) / (kNodeThreads / 8)));
+    const dim3 b(kNodeThreads), gr = node_blocks(a.g);
+    const float *none = nullptr;
     cudaError_t e;
     switch (mode) {
-    case kApply: e = launch_pdl(k_sweep3_node<kApply>, gr, b, 0, s, a); break;
-    case kResidual: e = launch_pdl(k_sweep3_node<kResidual>, gr, b, 0, s, a); break;
-    case kJacobi: e = launch_pdl(k_sweep3_node<kJacobi>, gr, b, 0, s, a); break;
+    case kApply: e = launch_pdl(k_sweep3_node<kApply, false>, gr, b, 0, s, a, a.g, none); break;
+    case kResidual: e = launch_pdl(k_sweep3_node<kResidual, false>, gr, b, 0, s, a, a.g, none); break;
+    case kJacobi: e = launch_pdl(k_sweep3_node<kJacobi, false>, gr, b, 0, s, a, a.g, none); break;
     default: return cudaErrorInvalidValue;
     }
+    if (e != cudaSuccess) return e;
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_prolong_sweep(const SweepArgs<float, float> &a, const Geom &gc, const float *ec, cudaStream_t s)
+{
+    if (a.g.dim != 3 || a.u == a.out) return cudaErrorInvalidValue;
+    cudaError_t e = launch_pdl(k_sweep3_node<kJacobi, true>, node_blocks(a.g), dim3(kNodeThreads), 0, s, a, gc, ec);
+    if (e != cudaSuccess) return e;
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_resid_restrict(const SweepArgs<float, float> &a, const Geom &gc, float *fc,
+                                  const FirstSweep<float> &first, cudaStream_t s)
+{
+    if (a.g.dim != 3) return cudaErrorInvalidValue;
+    cudaError_t e = launch_pdl(k_resid_restrict, dim3(gc.nx, gc.ny, gc.nz), dim3(224), 0, s, a, gc, fc, first);
     if (e != cudaSuccess) return e;
     ++g_launches;
     return cudaGetLastError();

@@ -445,8 +445,12 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
 // spreads the FP64 instructions of the update over twice as many SMs.
 constexpr int TX2 = 32;
 
-template <typename TO, int MODE, int TY2>
-__global__ void __launch_bounds__((TX2 + 1) * (TY2 + 1)) k_sweep2_fix(const SweepArgs<double, TO> a, const fix::Consts fc)
+// PRO: u is taken as u + P ec, ec the correction on the coarse level gc (a prolongation
+// launch less; on large grids its FP64 additions, repeated by the cells around a node, cost
+// more than the launch).
+template <typename TO, int MODE, int TY2, bool PRO>
+__global__ void __launch_bounds__((TX2 + 1) * (TY2 + 1))
+    k_sweep2_fix(const SweepArgs<double, TO> a, const fix::Consts fc, const Geom gc, const double *__restrict__ ec)
 {
     constexpr int BX2 = TX2 + 1, BY2 = TY2 + 1, NT2 = BX2 * BY2, PX2 = TX2 + 2, PP2 = PX2 * (TY2 + 2);
     __shared__ i64 X[2][4][PP2];                   // corner forces (integers, or doubles where they do not fit)
@@ -482,6 +486,38 @@ __global__ void __launch_bounds__((TX2 + 1) * (TY2 + 1)) k_sweep2_fix(const Swee
         const long long o = ok ? gidx(g, i, j, 0) : 0;
 #pragma unroll
         for (int p = 0; p < 2; ++p) D[p][q] = ok ? a.u[p * g.cs + o] : 0.0;
+    }
+    if (PRO) {
+        // the coarse cell around this cell; along an axis an even cell holds its first node
+        // and the midpoint, an odd one the midpoint and its second node
+        const bool ox = ((gx - 1) & 1) != 0, oy = ((gy - 1) & 1) != 0;
+        double C[2][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = ((gx - 1) >> 1) + (q & 1), j = ((gy - 1) >> 1) + (q >> 1);
+            const bool ok = i >= 0 && i < gc.nx && j >= 0 && j < gc.ny;
+            const long long o = ok ? gidx(gc, i, j, 0) : 0;
+#pragma unroll
+            for (int p = 0; p < 2; ++p) C[p][q] = ok ? ec[p * gc.cs + o] : 0.0;
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+#pragma unroll
+            for (int r = 0; r < 4; r += 2) {
+                const double m = 0.5 * (C[p][r] + C[p][r + 1]);
+                C[p][r + (ox ? 0 : 1)] = m;
+            }
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const double m = 0.5 * (C[p][r] + C[p][r + 2]);
+                C[p][r + (oy ? 0 : 2)] = m;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = gx - 1 + (q & 1), j = gy - 1 + (q >> 1);
+                if (i >= 0 && i < g.nx && j >= 0 && j < g.ny) D[p][q] += C[p][q];
+            }
+        }
     }
     double fv[2] = {0.0, 0.0};
     if (MODE != kApply && own) {
@@ -549,6 +585,107 @@ __global__ void __launch_bounds__((TX2 + 1) * (TY2 + 1)) k_sweep2_fix(const Swee
 int rows2(const Geom &g)
 {
     return ((g.nx + 30) / 32) * (long long)((g.ny + 6) / 8) >= 152 ? 8 : 4;
+}
+
+// Small 2D levels: the residual with its full weighting and the coarse level's first sweep
+// in one launch.  A block takes CT x CT coarse nodes: the forces of the (2 CT + 2)^2 cells
+// around them, the residuals of the (2 CT + 1)^2 fine nodes, then the weighted sums.
+constexpr int CT = 4, RC = 2 * CT + 2, RN = 2 * CT + 1, kRrThreads = 128;
+static_assert(RC * RC <= kRrThreads, "one thread a cell");
+
+__global__ void __launch_bounds__(kRrThreads) k_resid_restrict2(const SweepArgs<double, double> a, const fix::Consts fc,
+                                                                const Geom gc, double *__restrict__ rhs,
+                                                                const FirstSweep<double> first)
+{
+    __shared__ i64 X[2][4][RC * RC];
+    __shared__ int Xe[RC * RC];
+    __shared__ double R[2][RN * RN];
+    const Geom &g = a.g;
+    const int tid = threadIdx.x;
+    const int I0 = blockIdx.x * CT, J0 = blockIdx.y * CT;
+    const int lx = tid % RC, ly = tid / RC;
+    const int cx = 2 * I0 - 2 + lx, cy = 2 * J0 - 2 + ly;          // this thread's cell
+    const bool cell = tid < RC * RC;
+    const bool cell_ok = cell && cx >= 0 && cx < g.nx - 1 && cy >= 0 && cy < g.ny - 1;
+    const double psi = cell_ok ? a.psi[gidx(g, cx, cy, 0)] : 0.0;
+    const int I = I0 + tid % CT, J = J0 + tid / CT;                // this thread's coarse node
+    const bool coarse = tid < CT * CT && I < gc.nx && J < gc.ny;
+    double ip = 0.0;
+    if (first.u && coarse) ip = first.dinv ? first.dinv[gidx(gc, I, J, 0)] : body::inv_psi_sum<double, 2>(gc, first.psi, I, J, 0);
+    pdl_begin();
+    if (a.gate && *a.gate) return;
+    double D[2][4];
+    unsigned key = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = cx + (q & 1), j = cy + (q >> 1);
+        const bool ok = cell && i >= 0 && i < g.nx && j >= 0 && j < g.ny;
+        const long long o = ok ? gidx(g, i, j, 0) : 0;
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            D[p][q] = ok ? a.u[p * g.cs + o] : 0.0;
+            key = max(key, fix::exp_key(D[p][q]));
+        }
+    }
+    const int nx = tid % RN, ny = tid / RN;                        // this thread's fine node
+    const int gi = 2 * I0 - 1 + nx, gj = 2 * J0 - 1 + ny;
+    const bool node = tid < RN * RN && gi >= 0 && gi < g.nx && gj >= 0 && gj < g.ny;
+    double fv[2] = {0.0, 0.0};
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+        if (node) fv[p] = a.f[p * g.cs + gidx(g, gi, gj, 0)];
+    const int E = max((int)(key >> 20), fix::kExpLo);
+    i64 U[2][4], F[2][4];
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) U[p][q] = fix::to_fix(D[p][q], E);
+    int e;
+    fix::cell_forces2(U, E, psi, fc, F, e);
+    const bool all = __syncthreads_and(fc.ok && fix::key_ok(key) && fix::psi_ok(psi)) != 0;
+    if (!all) cell_forces2<double>(D, psi, a.c);
+    if (cell) {
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) X[p][q][tid] = all ? F[p][q] : fix::bits_of(D[p][q]);
+        Xe[tid] = e;
+    }
+    __syncthreads();
+    if (tid < RN * RN) {
+        const int c3 = ny * RC + nx, c2 = c3 + 1, c1 = c3 + RC, c0 = c1 + 1;   // the node's corner in its cells
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            double Ku;
+            if (all) {
+                const int ee = max(max(Xe[c0], Xe[c1]), max(Xe[c2], Xe[c3]));
+                Ku = fix::to_double((fix::down(X[p][3][c3], ee - Xe[c3]) + fix::down(X[p][2][c2], ee - Xe[c2])) +
+                                        (fix::down(X[p][1][c1], ee - Xe[c1]) + fix::down(X[p][0][c0], ee - Xe[c0])),
+                                    ee);
+            } else {
+                Ku = fix::of_bits(X[p][3][c3]) + fix::of_bits(X[p][2][c2]) + fix::of_bits(X[p][1][c1]) +
+                     fix::of_bits(X[p][0][c0]);
+            }
+            R[p][tid] = (!node || is_dir(g, p, gi, gj, 0)) ? 0.0 : fv[p] - Ku;
+        }
+    }
+    __syncthreads();
+    if (coarse) {
+        const int m = (2 * (tid / CT) + 1) * RN + 2 * (tid % CT) + 1;   // the coincident fine node
+        double f[2];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            double r[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const double *row = R[p] + m + (d - 1) * RN;
+                r[d] = row[0] + 0.5 * (row[-1] + row[1]);
+            }
+            f[p] = is_dir(gc, p, I, J, 0) ? 0.0 : 0.25 * (r[1] + 0.5 * (r[0] + r[2]));
+            rhs[p * gc.cs + gidx(gc, I, J, 0)] = f[p];
+        }
+        if (first.u) body::first_sweep<double, 2>(first, gc, I, J, 0, ip, f);
+    }
 }
 
 // 2D colour Gauss-Seidel in FP64, one launch per sweep.  A block owns a TILE x TILE tile of
@@ -723,21 +860,8 @@ __global__ void k_inv_psi(const Geom g, const double *__restrict__ psi, double *
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     const int k = blockIdx.z * blockDim.z + threadIdx.z;
     if (i >= g.nx || j >= g.ny || k >= g.nz) return;
-    double c[4];                                          // cells (i-1,j-1), (i,j-1), (i-1,j), (i,j), summed over z
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int ci = i - 1 + (q & 1), cj = j - 1 + (q >> 1);
-        const bool ok = ci >= 0 && cj >= 0 && ci < g.nx - 1 && cj < g.ny - 1;
-        if (g.dim == 3) {
-            const double lo = ok && k > 0 ? psi[gidx(g, ci, cj, k - 1)] : 0.0;
-            const double hi = ok && k < g.nz - 1 ? psi[gidx(g, ci, cj, k)] : 0.0;
-            c[q] = lo + hi;
-        } else {
-            c[q] = ok ? psi[gidx(g, ci, cj, 0)] : 0.0;
-        }
-    }
-    const double s = g.dim == 3 ? (c[0] + c[1]) + (c[2] + c[3]) : c[0] + c[1] + c[2] + c[3];
-    dinv[gidx(g, i, j, k)] = 1.0 / s;
+    dinv[gidx(g, i, j, k)] =
+        g.dim == 3 ? body::inv_psi_sum<double, 3>(g, psi, i, j, k) : body::inv_psi_sum<double, 2>(g, psi, i, j, k);
 }
 
 template <typename TO, int MODE>
@@ -753,8 +877,9 @@ cudaError_t launch_fix_mode(const SweepArgs<double, TO> &a, cudaStream_t s)
     } else {
         const int ty = rows2(a.g);
         const dim3 gr((a.g.nx + 30) / 32, (a.g.ny - 2 + ty) / ty), b(33 * (ty + 1));
-        e = ty == 8 ? launch_pdl(k_sweep2_fix<TO, MODE, 8>, gr, b, 0, s, a, fc)
-                    : launch_pdl(k_sweep2_fix<TO, MODE, 4>, gr, b, 0, s, a, fc);
+        const double *none = nullptr;
+        e = ty == 8 ? launch_pdl(k_sweep2_fix<TO, MODE, 8, false>, gr, b, 0, s, a, fc, a.g, none)
+                    : launch_pdl(k_sweep2_fix<TO, MODE, 4, false>, gr, b, 0, s, a, fc, a.g, none);
     }
     if (e != cudaSuccess) return e;
     ++g_launches;
@@ -772,6 +897,30 @@ long long sweep_blocks_fix(const Geom &g)
     }
     const long long units = (long long)((g.nx - 1 + TX - 1) / TX) * ((g.ny - 1 + TY - 1) / TY) * g.nz;
     return std::min<long long>(152, units);
+}
+
+cudaError_t launch_prolong_sweep(const SweepArgs<double, double> &a, const Geom &gc, const double *ec, cudaStream_t s)
+{
+    if (a.g.dim != 2 || a.u == a.out) return cudaErrorInvalidValue;
+    const fix::Consts fc = fix::make_consts(2, a.c);
+    const int ty = rows2(a.g);
+    const dim3 gr((a.g.nx + 30) / 32, (a.g.ny - 2 + ty) / ty), b(33 * (ty + 1));
+    cudaError_t e = ty == 8 ? launch_pdl(k_sweep2_fix<double, kJacobi, 8, true>, gr, b, 0, s, a, fc, gc, ec)
+                            : launch_pdl(k_sweep2_fix<double, kJacobi, 4, true>, gr, b, 0, s, a, fc, gc, ec);
+    if (e != cudaSuccess) return e;
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_resid_restrict(const SweepArgs<double, double> &a, const Geom &gc, double *fc,
+                                  const FirstSweep<double> &first, cudaStream_t s)
+{
+    if (a.g.dim != 2) return cudaErrorInvalidValue;
+    const dim3 gr((gc.nx + CT - 1) / CT, (gc.ny + CT - 1) / CT);
+    cudaError_t e = launch_pdl(k_resid_restrict2, gr, dim3(kRrThreads), 0, s, a, fix::make_consts(2, a.c), gc, fc, first);
+    if (e != cudaSuccess) return e;
+    ++g_launches;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_inv_psi(const Geom &g, const double *psi, double *dinv, cudaStream_t s)

@@ -213,7 +213,7 @@ struct Opts {
 };
 
 template <typename T>
-cudaError_t sweep(sbm_grid G, int l, int mode, const T *u, const T *f, T *out, double *part, double omega)
+SweepArgs<T, T> sweep_args(sbm_grid G, int l, const T *u, const T *f, T *out, double *part, double omega)
 {
     Level &L = G->L[l];
     SweepArgs<T, T> a;
@@ -228,7 +228,13 @@ cudaError_t sweep(sbm_grid G, int l, int mode, const T *u, const T *f, T *out, d
     a.kchunk = 0;
     a.gate = G->cur_gate;
     if constexpr (std::is_same<T, double>::value) a.dinv = G->dinv_ready ? L.dinv : nullptr;
-    return launch_sweep<T, T>(mode, a, G->st);
+    return a;
+}
+
+template <typename T>
+cudaError_t sweep(sbm_grid G, int l, int mode, const T *u, const T *f, T *out, double *part, double omega)
+{
+    return launch_sweep<T, T>(mode, sweep_args<T>(G, l, u, f, out, part, omega), G->st);
 }
 
 // FP32 3D sweeps: levels of at most kNodeKernelMaxNodes nodes (no norm wanted) use
@@ -240,17 +246,7 @@ cudaError_t sweep<float>(sbm_grid G, int l, int mode, const float *u, const floa
                          double omega)
 {
     Level &L = G->L[l];
-    SweepArgs<float, float> a;
-    a.g = L.g;
-    a.u = u;
-    a.f = f;
-    a.psi = L.psi32;
-    a.out = out;
-    a.part = part;
-    a.c = L.c32;
-    for (int p = 0; p < 3; ++p) a.wk[p] = (L.c64.kdiag[p] != 0.0) ? float(omega / L.c64.kdiag[p]) : 0.f;
-    a.kchunk = 0;
-    a.gate = G->cur_gate;
+    const SweepArgs<float, float> a = sweep_args<float>(G, l, u, f, out, part, omega);
     if (L.g.dim == 3 && part == nullptr && (long long)L.g.nx * L.g.ny * L.g.nz <= kNodeKernelMaxNodes)
         return launch_sweep_node(mode, a, G->st);
     if (L.has_tm && (u == L.su[0] || u == L.su[1]) && (mode == kApply || f == L.sf))
@@ -341,10 +337,37 @@ cudaError_t smooth(sbm_grid G, int l, int &cur, const sbm_opts &o, int nsweeps, 
 
 size_t level_bytes(const Level &L, size_t elem) { return (size_t)L.g.dim * L.g.cs * elem; }
 
-// V(nu1, nu2) on level l: u = P<T>::u(L, cur), right-hand side f.  Coarse levels
-// start from a zero correction; the coarsest is solved with the dense inverse.
+// What the restriction onto level l needs to run that level's first Jacobi sweep.
 template <typename T>
-cudaError_t vcycle(sbm_grid G, int l, int &cur, const sbm_opts &o, const T *f)
+FirstSweep<T> first_sweep_of(sbm_grid G, int l, const sbm_opts &o)
+{
+    Level &C = G->L[l];
+    FirstSweep<T> a;
+    if (l < 1 || o.smoother != SBM_JACOBI || o.nu1 < 1) return a;
+    a.psi = P<T>::psi(C);
+    if constexpr (std::is_same<T, double>::value) a.dinv = G->dinv_ready ? C.dinv : nullptr;
+    a.u = P<T>::u(C, 1);
+    for (int p = 0; p < 3; ++p) a.wk[p] = (C.c64.kdiag[p] != 0.0) ? T(o.omega / C.c64.kdiag[p]) : T(0);
+    return a;
+}
+
+// Levels whose V-cycle steps run fused: small ones, where a launch costs more than its
+// work, with Jacobi smoothing.
+template <typename T>
+bool fused_level(sbm_grid G, int l, const sbm_opts &o)
+{
+    const Geom &g = G->L[l].g;
+    if (o.smoother != SBM_JACOBI) return false;
+    if (std::is_same<T, float>::value) return g.dim == 3 && nnodes(g) <= kNodeKernelMaxNodes;
+    return g.dim == 2 && nnodes(g) <= kFuse2MaxNodes;
+}
+
+// V(nu1, nu2) on level l: u = P<T>::u(L, cur), right-hand side f, of whose pre-smoothing
+// `pre` sweeps have run.  Coarse levels start from a zero correction, or with Jacobi
+// smoothing from the first sweep, which the restriction writes; the coarsest is solved
+// with the dense inverse.
+template <typename T>
+cudaError_t vcycle(sbm_grid G, int l, int &cur, const sbm_opts &o, const T *f, int pre = 0)
 {
     Level &L = G->L[l];
     if (l == 0) {
@@ -358,23 +381,42 @@ cudaError_t vcycle(sbm_grid G, int l, int &cur, const sbm_opts &o, const T *f)
         return cudaSuccess;
     }
     Level &C = G->L[l - 1];
-    CKE(smooth<T>(G, l, cur, o, o.nu1, false, f));
-    if (G->cur_gate && l == G->nl - 1 && std::is_same<T, float>::value) {
+    CKE(smooth<T>(G, l, cur, o, o.nu1 - pre, false, f));
+    // the restriction also starts the coarse correction (the coarsest level's is
+    // overwritten by the dense solve), keeping the cycle a chain of kernels
+    const FirstSweep<T> first = first_sweep_of<T>(G, l - 1, o);
+    const bool gated = G->cur_gate && l == G->nl - 1 && std::is_same<T, float>::value;
+    const bool fused = fused_level<T>(G, l, o);
+    bool restricted = false;
+    if (fused && !gated && (l == 1 || first.u)) {
+        CKE(launch_resid_restrict(sweep_args<T>(G, l, P<T>::u(L, cur), f, nullptr, nullptr, 0.0), C.g, P<T>::f(C), first,
+                                  G->st));
+        restricted = true;
+    }
+    if (gated) {
         // adaptive inner cycles: the norm of this residual decides whether the
         // FP32 V-cycles of the outer iteration go on
         CKE(sweep<T>(G, l, kResidual, P<T>::u(L, cur), f, P<T>::r(L), G->part, 0.0));
         CKE(launch_inner_gate(G->part, (int)sweep_nblocks(G, l, true, P<T>::u(L, cur), f), G->scal, G->gate_rtol,
                               G->gate_tol, G->dgate, G->dgate + 1, G->st));
-    } else {
+    } else if (!restricted) {
         CKE(sweep<T>(G, l, kResidual, P<T>::u(L, cur), f, P<T>::r(L), nullptr, 0.0));
     }
-    // the restriction also zeroes the coarse correction (the coarsest level's is
-    // overwritten by the dense solve), keeping the cycle a chain of kernels
-    CKE(launch_restrict<T>(L.g, C.g, P<T>::r(L), P<T>::f(C), G->st, G->cur_gate, l - 1 > 0 ? P<T>::u(C, 0) : nullptr));
-    int cc = 0;
-    CKE(vcycle<T>(G, l - 1, cc, o, P<T>::f(C)));
-    CKE(launch_prolong_add<T>(L.g, C.g, P<T>::u(C, cc), P<T>::u(L, cur), G->st, G->cur_gate));
-    CKE(smooth<T>(G, l, cur, o, o.nu2, true, f));
+    if (!restricted)
+        CKE(launch_restrict<T>(L.g, C.g, P<T>::r(L), P<T>::f(C), G->st, G->cur_gate, l - 1 > 0 ? P<T>::u(C, 0) : nullptr,
+                               first));
+    int cc = first.u ? 1 : 0;
+    CKE(vcycle<T>(G, l - 1, cc, o, P<T>::f(C), cc));
+    int post = 0;
+    if (fused && o.nu2 > 0) {
+        CKE(launch_prolong_sweep(sweep_args<T>(G, l, P<T>::u(L, cur), f, P<T>::u(L, 1 - cur), nullptr, o.omega), C.g,
+                                 P<T>::u(C, cc), G->st));
+        cur ^= 1;
+        post = 1;
+    } else {
+        CKE(launch_prolong_add<T>(L.g, C.g, P<T>::u(C, cc), P<T>::u(L, cur), G->st, G->cur_gate));
+    }
+    CKE(smooth<T>(G, l, cur, o, o.nu2 - post, true, f));
     return cudaSuccess;
 }
 

@@ -62,23 +62,66 @@ __device__ __forceinline__ void finalize_f(const SweepArgs<T, TO> &a, int gx, in
 // Small 3D levels (FP32), one cell of a node's eight: thread c of the node's group
 // of eight evaluates the cell of which node (i, j, k) is corner c (bit m = the
 // node's offset along axis m within the cell) and returns the force on that
-// corner and the cell's psi; cells outside the grid give zeros.
-__device__ __forceinline__ void node_cell(const SweepArgs<float, float> &a, int i, int j, int k, int c,
-                                          float (&F)[3], float &ps)
+// corner, the cell's psi (given: ps, read by node_psi) and the node's own values; cells
+// outside the grid give zeros.  ec (may be null): u is taken as u + P ec, ec the
+// correction on the coarse level gc.
+__device__ __forceinline__ bool node_psi(const SweepArgs<float, float> &a, int i, int j, int k, int c, float &ps)
 {
     const Geom &g = a.g;
-    const int cx = c & 1, cy = (c >> 1) & 1, cz = (c >> 2) & 1;
-    const int ci = i - cx, cj = j - cy, ck = k - cz;
-    F[0] = F[1] = F[2] = 0.f;
+    const int ci = i - (c & 1), cj = j - ((c >> 1) & 1), ck = k - ((c >> 2) & 1);
     ps = 0.f;
-    if (ci < 0 || cj < 0 || ck < 0 || ci >= g.nx - 1 || cj >= g.ny - 1 || ck >= g.nz - 1) return;
+    if (ci < 0 || cj < 0 || ck < 0 || ci >= g.nx - 1 || cj >= g.ny - 1 || ck >= g.nz - 1) return false;
     ps = a.psi[gidx(g, ci, cj, ck)];
+    return true;
+}
+
+template <bool PRO>
+__device__ __forceinline__ void node_cell(const SweepArgs<float, float> &a, int i, int j, int k, int c, float ps,
+                                          const Geom &gc, const float *__restrict__ ec, float (&F)[3], float (&own)[3])
+{
+    const Geom &g = a.g;
+    const int ci = i - (c & 1), cj = j - ((c >> 1) & 1), ck = k - ((c >> 2) & 1);
     float U[3][8];
 #pragma unroll
     for (int b = 0; b < 8; ++b) {
         const long long o = gidx(g, ci + (b & 1), cj + ((b >> 1) & 1), ck + (b >> 2));
 #pragma unroll
         for (int p = 0; p < 3; ++p) U[p][b] = a.u[p * g.cs + o];
+    }
+    if (PRO) {
+        // the coarse cell around this cell; along an axis an even cell holds its first node
+        // and the midpoint, an odd one the midpoint and its second node
+        float E[3][8];
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const long long o = gidx(gc, (ci >> 1) + (b & 1), (cj >> 1) + ((b >> 1) & 1), (ck >> 1) + (b >> 2));
+#pragma unroll
+            for (int p = 0; p < 3; ++p) E[p][b] = ec[p * gc.cs + o];
+        }
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) {
+                const bool odd = ((ax == 0 ? ci : ax == 1 ? cj : ck) & 1) != 0;
+#pragma unroll
+                for (int b = 0; b < 8; ++b) {
+                    if ((b >> ax) & 1) continue;
+                    const float m = 0.5f * (E[p][b] + E[p][b | (1 << ax)]);
+                    if (odd) E[p][b] = m;
+                    else E[p][b | (1 << ax)] = m;
+                }
+            }
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int b = 0; b < 8; ++b) U[p][b] += E[p][b];
+    }
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        float v = U[p][0];
+#pragma unroll
+        for (int b = 1; b < 8; ++b) v = (c == b) ? U[p][b] : v;
+        own[p] = v;
     }
     cell_forces3<float>(U, ps, a.c);
 #pragma unroll
@@ -121,7 +164,7 @@ __device__ __forceinline__ T fw_row(const T *__restrict__ row, int I, int nx)
 // outside the grid) so they are all in flight together.
 template <typename T, int D>
 __device__ __forceinline__ void restrict_node(const Geom &gf, const Geom &gc, const T *__restrict__ rf,
-                                              T *__restrict__ fc, int I, int J, int K)
+                                              T *__restrict__ fc, int I, int J, int K, T (&out)[D])
 {
     constexpr bool d3 = D == 3;
     const T scale = d3 ? T(0.125) : T(0.25);
@@ -151,7 +194,38 @@ __device__ __forceinline__ void restrict_node(const Geom &gf, const Geom &gc, co
             s *= scale;
         }
         fc[p * gc.cs + oc] = s;
+        out[p] = s;
     }
+}
+
+// 1 / (sum of psi over the node's cells), in the order of the sweeps.
+template <typename T, int D>
+__device__ __forceinline__ T inv_psi_sum(const Geom &g, const T *__restrict__ psi, int i, int j, int k)
+{
+    T c[4];                                       // cells (i-1,j-1), (i,j-1), (i-1,j), (i,j), summed over z
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int ci = i - 1 + (q & 1), cj = j - 1 + (q >> 1);
+        const bool ok = ci >= 0 && cj >= 0 && ci < g.nx - 1 && cj < g.ny - 1;
+        if (D == 3) {
+            const T lo = ok && k > 0 ? psi[gidx(g, ci, cj, k - 1)] : T(0);
+            const T hi = ok && k < g.nz - 1 ? psi[gidx(g, ci, cj, k)] : T(0);
+            c[q] = lo + hi;
+        } else {
+            c[q] = ok ? psi[gidx(g, ci, cj, 0)] : T(0);
+        }
+    }
+    return T(1) / (D == 3 ? (c[0] + c[1]) + (c[2] + c[3]) : c[0] + c[1] + c[2] + c[3]);
+}
+
+// The sweep of FirstSweep at one coarse node, f its right-hand side (0 on Dirichlet dofs).
+template <typename T, int D>
+__device__ __forceinline__ void first_sweep(const FirstSweep<T> &a, const Geom &g, int i, int j, int k, T ip,
+                                            const T (&f)[D])
+{
+    const long long o = gidx(g, i, j, k);
+#pragma unroll
+    for (int p = 0; p < D; ++p) a.u[p * g.cs + o] = f[p] * ip * a.wk[p];
 }
 
 // u_f += P e_c on free fine dofs.  One thread per coarse node (I,J,K) writes the

@@ -114,6 +114,16 @@ struct SweepArgs {
     bool foreign_psi = false;
 };
 
+// First pre-smoothing sweep of a coarse level, from a zero correction: u = omega D^-1 f on
+// free dofs, written by the restriction that forms f.  psi, dinv as in SweepArgs (the
+// coarse level's); u null: no sweep.
+template <typename T>
+struct FirstSweep {
+    const T *psi = nullptr;
+    const T *dinv = nullptr;
+    T *u = nullptr;
+    T wk[3] = {T(0), T(0), T(0)};
+};
 // Number of z chunks for a z-streaming stencil launch: minimises
 // waves x (layers per block), where a wave is `slots` resident blocks (the
 // kernel's blocks per SM x 152 SMs), a block streams ceil(nzc/nc) layers plus one
@@ -220,7 +230,7 @@ cudaError_t launch_gs2_sweep(const Geom &g, const Coef<T> &c, const T *psi, cons
 
 template <typename T>
 cudaError_t launch_restrict(const Geom &gf, const Geom &gc, const T *rf, T *fc, cudaStream_t s,
-                            const int *gate = nullptr, T *zero_uc = nullptr);
+                            const int *gate = nullptr, T *zero_uc = nullptr, const FirstSweep<T> &first = FirstSweep<T>());
 
 template <typename T>
 cudaError_t launch_prolong_add(const Geom &gf, const Geom &gc, const T *ec, T *uf, cudaStream_t s,
@@ -261,6 +271,18 @@ cudaError_t launch_bottom_dirichlet(const Geom &g, double *A, cudaStream_t s);
 cudaError_t launch_sweep_node(int mode, const SweepArgs<float, float> &a, cudaStream_t s);
 // Levels with at most this many nodes use the cell-parallel per-node FP32 kernel.
 constexpr long long kNodeKernelMaxNodes = 20000;
+// Fused steps of small levels, whose launches cost more than their work: the residual
+// with its full weighting and the coarse level's first sweep, and a prolongation with the
+// Jacobi sweep after it (a.out gets the sweep of a.u + P ec; a.u is not changed).
+// FP32 3D (k_stencil.cu) and FP64 2D (k_stencil_fix.cu).
+cudaError_t launch_resid_restrict(const SweepArgs<float, float> &a, const Geom &gc, float *fc,
+                                  const FirstSweep<float> &first, cudaStream_t s);
+cudaError_t launch_resid_restrict(const SweepArgs<double, double> &a, const Geom &gc, double *fc,
+                                  const FirstSweep<double> &first, cudaStream_t s);
+cudaError_t launch_prolong_sweep(const SweepArgs<float, float> &a, const Geom &gc, const float *ec, cudaStream_t s);
+cudaError_t launch_prolong_sweep(const SweepArgs<double, double> &a, const Geom &gc, const double *ec, cudaStream_t s);
+// 2D FP64 levels with at most this many nodes take the fused steps.
+constexpr long long kFuse2MaxNodes = 20000;
 
 // Inverse of the coarsest-level matrix in place (one cooperative launch);
 // bar: 4 device words, bar[2] != 0 afterwards if a grid barrier timed out.
