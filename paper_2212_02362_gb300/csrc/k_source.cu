@@ -14,7 +14,14 @@
 // forms each cell's eigenstrain stress once, then one thread per node gathers from
 // its cells (no atomics).  This is setup work, run once per load: not part of the
 // V-cycle.
+//
+// Bound by FP64 issue (about two lanes per SM and clock): the gather's 72 + 32 additions a
+// node run on 64-bit integers instead, the node's values turned into them on their
+// largest exponent (53 bits kept down to 2^-5 of it); 16 FP64 instructions a node are
+// left, and the square root where psi is not constant around the node.  Values that do
+// not fit (infinities, NaN, extreme exponents) are added in FP64.
 #include "sbm_common.cuh"
+#include "sbm_fix.cuh"
 
 namespace sbm {
 
@@ -52,12 +59,12 @@ __global__ void __launch_bounds__(kThr) k_cell_stress(const SourceArgs A, const 
     double tr = 0.0;
 #pragma unroll
     for (int a = 0; a < D; ++a) tr += e[a];
-    const double pc = psi[c];
-    // cubic C: sigma_pp = c11 e_pp + c12 (tr - e_pp), sigma_pq = 2 c44 e_pq (tensor shear)
+    // cubic C: sigma_pp = (c11 - c12) e_pp + c12 tr, sigma_pq = 2 c44 e_pq (tensor shear)
+    const double pc = psi[c], l = A.c12 * tr, sh = pc * (2.0 * A.c44);
 #pragma unroll
-    for (int a = 0; a < D; ++a) sig[a * NC + c] = pc * (A.c11 * e[a] + A.c12 * (tr - e[a]));
+    for (int a = 0; a < D; ++a) sig[a * NC + c] = pc * madd(A.c11 - A.c12, e[a], l);
 #pragma unroll
-    for (int v = D; v < (D == 3 ? 6 : 3); ++v) sig[v * NC + c] = pc * (2.0 * A.c44 * e[v]);
+    for (int v = D; v < (D == 3 ? 6 : 3); ++v) sig[v * NC + c] = sh * e[v];
 }
 
 // Pass 2 (or the only pass without eigenstrain): one thread per node gathering its
@@ -76,11 +83,12 @@ __global__ void __launch_bounds__(kThr) k_source_terms(const SourceArgs A, const
     const int nd[3] = {n % A.nx, (n % nxy) / A.nx, n / nxy};
     const int mc[3] = {A.nx - 1, A.ny - 1, D == 3 ? A.nz - 1 : 1};
     const int NC = mc[0] * mc[1] * mc[2];
-    double acc[3] = {0.0, 0.0, 0.0};
-    double ps = 0.0, g[3] = {0.0, 0.0, 0.0};
+    constexpr int NV = D == 3 ? 6 : 3, NK = 1 << D;
+    double sv[NK][NV], pv[NK];                    // the cells' stresses (0 outside the grid) and psi (mirrored)
+    unsigned ks = 0, kp = 0;
     int inside = 0;
 #pragma unroll
-    for (int c = 0; c < (1 << D); ++c) {
+    for (int c = 0; c < NK; ++c) {
         int cc[3] = {0, 0, 0};
         bool in = true;
 #pragma unroll
@@ -90,29 +98,88 @@ __global__ void __launch_bounds__(kThr) k_source_terms(const SourceArgs A, const
             cc[a] = min(max(v, 0), mc[a] - 1);
         }
         const int cid = cc[0] + mc[0] * (cc[1] + mc[1] * cc[2]);
-        const double pc = psi[cid];
-        ps += pc;
+        pv[c] = psi[cid];
+        kp = max(kp, fix::exp_key(pv[c]));
+        inside += in ? 1 : 0;
 #pragma unroll
-        for (int a = 0; a < D; ++a) g[a] += ((c >> a) & 1) ? pc : -pc;
-        if (!in) continue;
-        ++inside;
-        if (sig) {
-            // s_q = +1 when the cell lies below the node along q (bit clear), -1 above
+        for (int v = 0; v < NV; ++v) {
+            sv[c][v] = (in && sig) ? sig[v * NC + cid] : 0.0;
+            ks = max(ks, fix::exp_key(sv[c][v]));
+        }
+    }
+    double acc[D], ps, g[D];
+    bool flat;                                    // no gradient of psi
+    if (fix::key_ok(kp)) {
+        const int E = max((int)(kp >> 20), fix::kExpLo);
+        fix::i64 s = 0, d[D];
+#pragma unroll
+        for (int a = 0; a < D; ++a) d[a] = 0;
+#pragma unroll
+        for (int c = 0; c < NK; ++c) {
+            const fix::i64 v = fix::to_fix(pv[c], E);
+            s += v;
+#pragma unroll
+            for (int a = 0; a < D; ++a) d[a] += ((c >> a) & 1) ? v : -v;
+        }
+        ps = fix::to_double(s, E - fix::kFixUnit);
+        fix::i64 any = 0;
+#pragma unroll
+        for (int a = 0; a < D; ++a) any |= d[a];
+        flat = any == 0;
+#pragma unroll
+        for (int a = 0; a < D; ++a) g[a] = flat ? 0.0 : fix::to_double(d[a], E - fix::kFixUnit);
+    } else {
+        ps = 0.0;
+        flat = false;
+#pragma unroll
+        for (int a = 0; a < D; ++a) g[a] = 0.0;
+#pragma unroll
+        for (int c = 0; c < NK; ++c) {
+            ps += pv[c];
+#pragma unroll
+            for (int a = 0; a < D; ++a) g[a] += ((c >> a) & 1) ? pv[c] : -pv[c];
+        }
+    }
+    // s_q = +1 when the cell lies below the node along q (bit clear), -1 above
+    if (fix::key_ok(ks)) {
+        const int E = max((int)(ks >> 20), fix::kExpLo);
+        fix::i64 s[D];
+#pragma unroll
+        for (int p = 0; p < D; ++p) s[p] = 0;
+#pragma unroll
+        for (int c = 0; c < NK; ++c) {
+            fix::i64 v[NV];
+#pragma unroll
+            for (int m = 0; m < NV; ++m) v[m] = fix::to_fix<5>(sv[c][m], E);     // 24 terms at most
 #pragma unroll
             for (int p = 0; p < D; ++p)
 #pragma unroll
+                for (int q = 0; q < D; ++q) s[p] += ((c >> q) & 1) ? -v[vslot<D>(p, q)] : v[vslot<D>(p, q)];
+        }
+#pragma unroll
+        for (int p = 0; p < D; ++p) acc[p] = fix::to_double(s[p], E - fix::kFixUnit + 2);
+    } else {
+#pragma unroll
+        for (int p = 0; p < D; ++p) {
+            acc[p] = 0.0;
+#pragma unroll
+            for (int c = 0; c < NK; ++c)
+#pragma unroll
                 for (int q = 0; q < D; ++q) {
-                    const double v = sig[vslot<D>(p, q) * NC + cid];
+                    const double v = sv[c][vslot<D>(p, q)];
                     acc[p] += ((c >> q) & 1) ? -v : v;
                 }
         }
     }
     const double inv = A.inv;
     const double pn = ps * (1.0 / (1 << D));
-    double gg = 0.0;
+    double gn = 0.0;
+    if (!flat) {
+        double gg = 0.0;
 #pragma unroll
-    for (int a = 0; a < D; ++a) gg += (g[a] * inv) * (g[a] * inv);
-    const double gn = sqrt(gg);
+        for (int a = 0; a < D; ++a) gg += (g[a] * inv) * (g[a] * inv);
+        gn = sqrt(gg);
+    }
     const double w = (double)inside * (1.0 / (1 << D));
 #pragma unroll
     for (int p = 0; p < D; ++p) {

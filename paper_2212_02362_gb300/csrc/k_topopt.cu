@@ -11,12 +11,14 @@
 // own value), V = h^d sum_c eta_c.
 //
 // One thread per cell: eta and its 2d face neighbours, u at the 2^d corner nodes
-// (d components, packed), the cell's force vector S_c u_c from the sum-factorised
-// cell routine of the operator, and the update.  The kernel also writes the next
+// (d components, packed), the cell's strain energy, and the update.  In 3D the energy is
+// formed in integers (sbm_fix.cuh): in FP64 the kernel is bound by FP64 issue, and the
+// energy was four fifths of it.  The kernel also writes the next
 // stiffness (eta' + zeta)^2 and per-block partial sums of eta' (the next volume)
 // and of psi_c e_c (the compliance u^T K u h^d of the solve that produced u), each
 // summed in a fixed order so that results do not depend on scheduling.  FP64.
 #include "sbm_common.cuh"
+#include "sbm_fix.cuh"
 
 namespace sbm {
 
@@ -25,7 +27,7 @@ namespace {
 constexpr int kThr = 256;
 
 template <int D>
-__global__ void __launch_bounds__(kThr) k_topopt_step(const TopoptArgs A, const Coef<double> c,
+__global__ void __launch_bounds__(kThr) k_topopt_step(const TopoptArgs A, const Coef<double> c, const fix::Consts fc,
                                                       const double *__restrict__ eta, const double *__restrict__ u,
                                                       const double *__restrict__ psi_solve,
                                                       const double *__restrict__ eta_sum, double *__restrict__ eta_out,
@@ -54,18 +56,30 @@ __global__ void __launch_bounds__(kThr) k_topopt_step(const TopoptArgs A, const 
         const int N = A.nx * A.ny * (D == 3 ? A.nz : 1);
         double e = 0.0;
         if (D == 3) {
-            double U[3][8], U0[3][8];
+            double U[3][8];
 #pragma unroll
             for (int a = 0; a < 8; ++a) {
                 const int o = (ci + (a & 1)) + A.nx * ((cj + ((a >> 1) & 1)) + A.ny * (ck + ((a >> 2) & 1)));
 #pragma unroll
-                for (int p = 0; p < 3; ++p) U0[p][a] = U[p][a] = u[p * N + o];
+                for (int p = 0; p < 3; ++p) U[p][a] = u[p * N + o];
             }
-            cell_forces3<double>(U, 1.0, c);
+            fix::i64 I[3][8];
+            bool none;
+            int eu;
+            if (fc.ok && fix::transform_cell3(U, I, none, eu)) {
+                e = none ? 0.0 : fix::cell_work3(I, eu, I, eu, fc);
+            } else {
+                double U0[3][8];
 #pragma unroll
-            for (int a = 0; a < 8; ++a)
+                for (int a = 0; a < 8; ++a)
 #pragma unroll
-                for (int p = 0; p < 3; ++p) e += U0[p][a] * U[p][a];
+                    for (int p = 0; p < 3; ++p) U0[p][a] = U[p][a];
+                cell_forces3<double>(U, 1.0, c);
+#pragma unroll
+                for (int a = 0; a < 8; ++a)
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) e += U0[p][a] * U[p][a];
+            }
         } else {
             double U[2][4], U0[2][4];
 #pragma unroll
@@ -138,9 +152,9 @@ cudaError_t launch_topopt_step(int dim, const TopoptArgs &A, const Coef<double> 
     if (NN * dim >= (1ll << 31)) return cudaErrorInvalidValue;               // 32-bit indexing
     const dim3 grid((unsigned)topopt_blocks(NC));
     if (dim == 3)
-        k_topopt_step<3><<<grid, kThr, 0, s>>>(A, c, eta, u, psi_solve, eta_sum, eta_out, psi_next, part);
+        k_topopt_step<3><<<grid, kThr, 0, s>>>(A, c, fix::make_consts(dim, c), eta, u, psi_solve, eta_sum, eta_out, psi_next, part);
     else
-        k_topopt_step<2><<<grid, kThr, 0, s>>>(A, c, eta, u, psi_solve, eta_sum, eta_out, psi_next, part);
+        k_topopt_step<2><<<grid, kThr, 0, s>>>(A, c, fix::make_consts(dim, c), eta, u, psi_solve, eta_sum, eta_out, psi_next, part);
     ++g_launches;
     return cudaGetLastError();
 }

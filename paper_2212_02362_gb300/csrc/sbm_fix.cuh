@@ -67,17 +67,19 @@ __host__ __device__ __forceinline__ bool key_ok(unsigned key)
     return key == 0u || (key >= ((unsigned)kExpLo << 20) && key < ((unsigned)kExpHi << 20));
 }
 
-// v as an integer on the unit 2^(E - 1023 - 59), E >= the biased exponent of v.
+// v as an integer on the unit 2^(E - 1023 - 52 - UP), E >= the biased exponent of v: below
+// 2^(53 + UP).  UP = 7 unless sums of more than eight values follow.
+template <int UP = 7>
 __host__ __device__ __forceinline__ i64 to_fix(double v, int E)
 {
     const i64 b = bits_of(v);
     const int ex = (int)((unsigned)(b >> 52) & 0x7ffu);
     const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
     const int sh = E - ex;
-    const i64 a = sh > 63 ? 0 : (i64)((m << 7) >> sh);
+    const i64 a = sh > 63 ? 0 : (i64)((m << UP) >> sh);
     return b < 0 ? -a : a;
 }
-constexpr int kFixUnit = 1023 + 59;     // to_fix's unit is 2^(E - kFixUnit)
+constexpr int kFixUnit = 1023 + 59;     // to_fix<7>'s unit is 2^(E - kFixUnit)
 
 // a * 2^e as a double (e such that the result is normal; a may be zero).
 __host__ __device__ __forceinline__ double to_double(i64 a, int e)
@@ -98,7 +100,7 @@ __host__ __device__ __forceinline__ Frac split(i64 k)
     return f;
 }
 
-// (a k) / 2^64 to within two units: the parts a_lo k_lo and the low halves of the cross
+// (a k) / 2^64 to within two units, k >= 0: the parts a_lo k_lo and the low halves of the cross
 // products are dropped.
 __host__ __device__ __forceinline__ i64 mul(i64 a, Frac k)
 {
@@ -180,25 +182,17 @@ __host__ __device__ __forceinline__ int norm_shift(unsigned long long m) { retur
 
 __host__ __device__ __forceinline__ i64 down(i64 v, int s) { return v >> (s > 63 ? 63 : s); }
 
-// One 3D cell: in-plane transforms (bfly4xy of the integers) of its bottom and top faces
-// on the unit 2^(E - kFixUnit), its psi.  Returns the transformed face forces, the
-// unit of which is 2^e (e = kNoExp: no force, Fb = Ft = 0).
-__host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], const i64 (&Tt)[3][4], int E, double psi,
-                                                     const Consts &c, i64 (&Fb)[3][4], i64 (&Ft)[3][4], int &e)
+// The 21 transformed values of a 3D cell that carry force (U[p][1..7] of bfly8), shifted up
+// to 2^61 at most.  Returns the shift (-3 at least); none: all are zero.
+__host__ __device__ __forceinline__ int normalize3(i64 (&U)[3][8], bool &none)
 {
-    i64 U[3][8];
     unsigned mh = 0;
 #pragma unroll
     for (int p = 0; p < 3; ++p)
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            U[p][s] = Tb[p][s] + Tt[p][s];
-            U[p][s + 4] = Tt[p][s] - Tb[p][s];
-            if (s > 0) mh |= mag_hi(U[p][s]);
-            mh |= mag_hi(U[p][s + 4]);
-        }
+        for (int s = 1; s < 8; ++s) mh |= mag_hi(U[p][s]);
     unsigned long long m = (unsigned long long)mh << 32 | 0xffffffffu;
-    bool none = false;
+    none = false;
     if (mh == 0u) {                          // all below 2^32: the low words decide
         i64 any = 0;
         m = 0;
@@ -211,12 +205,10 @@ __host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], cons
             }
         none = any == 0;
     }
-    int ep;
-    const i64 pm = psi_mantissa(psi, ep);
-    int sh = norm_shift(m);
-    e = (none || pm == 0) ? kNoExp : E - kFixUnit - sh + ep + c.ec;
+    const int sh = norm_shift(m);
+    int up = sh;
     if (sh < 0) {                            // sums of opposite corners near the bound
-        sh += 3;
+        up += 3;
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
@@ -225,12 +217,16 @@ __host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], cons
 #pragma unroll
     for (int p = 0; p < 3; ++p)
 #pragma unroll
-        for (int s = 1; s < 8; ++s) U[p][s] = (i64)((unsigned long long)U[p][s] << (sh & 63));
-    Frac k[7];
-#pragma unroll
-    for (int i = 0; i < 7; ++i) k[i] = split(mul(pm, c.c[i]));
+        for (int s = 1; s < 8; ++s) U[p][s] = (i64)((unsigned long long)U[p][s] << (up & 63));
+    return sh;
+}
+
+// The stress map of a 3D cell on normalised values, constants k (Consts times psi's
+// mantissa, or psi's 1): dU[p][s], dU[p][0] = 0, below 2^57 in magnitude for k below 2^60.
+__host__ __device__ __forceinline__ void stress3(const i64 (&U)[3][8], const Frac (&k)[7], int neg12, i64 (&dU)[3][8])
+{
     i64 ltr = mul(U[0][1] + U[1][2] + U[2][4], k[1]);
-    ltr = c.neg12 ? -ltr : ltr;
+    ltr = neg12 ? -ltr : ltr;
     const i64 sxx = mul(U[0][1], k[0]) + ltr, syy = mul(U[1][2], k[0]) + ltr, szz = mul(U[2][4], k[0]) + ltr;
     const i64 sxy = mul(U[1][1] + U[0][2], k[2]);
     const i64 sxz = mul(U[2][1] + U[0][4], k[2]);
@@ -246,9 +242,38 @@ __host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], cons
     const i64 d05 = a + d, d16 = a - d;
     const i64 d23 = mul(S + U[2][3], k[5]), d15 = mul(S + U[1][5], k[5]), d06 = mul(S + U[0][6], k[5]);
     const i64 d07 = mul(U[0][7], k[6]), d17 = mul(U[1][7], k[6]), d27 = mul(U[2][7], k[6]);
-    const i64 dU[3][8] = {{0, sxx, sxy, d03, sxz, d05, d06, d07},
-                          {0, sxy, syy, d13, syz, d15, d16, d17},
-                          {0, sxz, syz, d23, szz, d25, d26, d27}};
+    const i64 r[3][8] = {{0, sxx, sxy, d03, sxz, d05, d06, d07},
+                         {0, sxy, syy, d13, syz, d15, d16, d17},
+                         {0, sxz, syz, d23, szz, d25, d26, d27}};
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int s = 0; s < 8; ++s) dU[p][s] = r[p][s];
+}
+
+// One 3D cell: in-plane transforms (bfly4xy of the integers) of its bottom and top faces
+// on the unit 2^(E - kFixUnit), its psi.  Returns the transformed face forces, the
+// unit of which is 2^e (e = kNoExp: no force, Fb = Ft = 0).
+__host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], const i64 (&Tt)[3][4], int E, double psi,
+                                                     const Consts &c, i64 (&Fb)[3][4], i64 (&Ft)[3][4], int &e)
+{
+    i64 U[3][8], dU[3][8];
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            U[p][s] = Tb[p][s] + Tt[p][s];
+            U[p][s + 4] = Tt[p][s] - Tb[p][s];
+        }
+    bool none;
+    const int sh = normalize3(U, none);
+    int ep;
+    const i64 pm = psi_mantissa(psi, ep);
+    e = (none || pm == 0) ? kNoExp : E - kFixUnit - sh + ep + c.ec;
+    Frac k[7];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) k[i] = split(mul(pm, c.c[i]));
+    stress3(U, k, c.neg12, dU);
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
         Fb[p][0] = -dU[p][4];
@@ -259,6 +284,55 @@ __host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], cons
             Ft[p][s] = dU[p][s] + dU[p][s + 4];
         }
     }
+}
+
+// Nodal values of a 3D cell as transformed, normalised integers: v = U 2^(e), e returned.
+// False when a value does not fit.
+__host__ __device__ __forceinline__ bool transform_cell3(const double (&v)[3][8], i64 (&U)[3][8], bool &none, int &e)
+{
+    unsigned key = 0;
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int a = 0; a < 8; ++a) {
+            const unsigned q = exp_key(v[p][a]);
+            key = q > key ? q : key;
+        }
+    if (!key_ok(key)) return false;
+    const int E = (int)(key >> 20) > kExpLo ? (int)(key >> 20) : kExpLo;
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+#pragma unroll
+        for (int a = 0; a < 8; ++a) U[p][a] = to_fix(v[p][a], E);
+        bfly8(U[p]);
+    }
+    e = E - kFixUnit - normalize3(U, none);
+    return true;
+}
+
+// v^T S u of a 3D cell (S the unit-psi cell matrix of the constants c), u and v given as
+// transform_cell3 leaves them: the sum, in 128 bits, of 21 products of the stress of u with
+// the transform of v, in the basis where the cell's rigid motion has dropped out.
+__host__ __device__ __forceinline__ double cell_work3(const i64 (&U)[3][8], int eu, const i64 (&V)[3][8], int ev,
+                                                      const Consts &c)
+{
+    i64 dU[3][8];
+    Frac k[7];                               // twice the constants: no sum over cells follows
+#pragma unroll
+    for (int i = 0; i < 7; ++i) k[i] = split((((i64)c.c[i].hi << 32) + c.c[i].lo) * 2);
+    stress3(U, k, c.neg12, dU);
+    __int128 s = 0;                          // 21 x 2^59 x 2^61 at most
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int q = 1; q < 8; ++q) s += (__int128)dU[p][q] * V[p][q];
+    const i64 hi = (i64)(s >> 64);
+    const unsigned long long lo = (unsigned long long)s;
+    if (s == 0) return 0.0;
+    // dU = U c / 2^63 with c in units of 2^(ec - 65)
+    const double d = (double)hi * 18446744073709551616.0 + (double)lo;
+    const int e = eu + ev + c.ec - 2, f = (int)((unsigned)(bits_of(d) >> 52) & 0x7ffu) + e;
+    return f > 0 && f < 2047 ? of_bits(bits_of(d) + ((i64)e << 52)) : ldexp(d, e);
 }
 
 // The six transformed values of a 2D cell that carry force, in the order U[0][1..3],
