@@ -31,9 +31,17 @@ __device__ __forceinline__ void node_of(const Geom &g, long long t, int &i, int 
 // Launch geometry of the node-wise kernels: a 3D grid of (32, 4, 2) blocks covers
 // (nx, ny, nz) directly, so no index decoding by division is needed.
 const dim3 kNodeBlock(32, 4, 2);
-inline dim3 node_grid(const Geom &g)
+inline dim3 node_grid(const Geom &g, const dim3 b = kNodeBlock)
 {
-    return dim3((g.nx + 31) / 32, (g.ny + 3) / 4, (g.nz + 1) / 2);
+    return dim3((g.nx + b.x - 1) / b.x, (g.ny + b.y - 1) / b.y, (g.nz + b.z - 1) / b.z);
+}
+
+// The 3D transfers: in FP64 some 120 instructions a node, whose issue on one SM is what a
+// block of eight warps costs on a small level (13 us); single warps spread over all SMs.
+template <typename T>
+inline dim3 transfer_block(const Geom &g)
+{
+    return sizeof(T) == 8 && g.dim == 3 ? dim3(32, 1, 1) : kNodeBlock;
 }
 
 // zero_uc (may be null): the coarse correction, zeroed at each coarse node (the start of
@@ -310,8 +318,8 @@ __global__ void k_copy_gated(long long n, const T *__restrict__ src, T *__restri
 
 // -------------------------------------------------------------- bottom solve
 
-// Dense K of the coarsest level over packed dofs (p*N + node).  One thread per column
-// (q, node m) and neighbour of m: it sums psi_c K_e over the cells that hold both nodes
+// Dense K of the coarsest level over the dofs node * d + p, an order in which K is banded.
+// One thread per column (node m, q) and neighbour of m: it sums psi_c K_e over the cells that hold both nodes
 // (K_e the unit-psi cell matrix, row = corner * d + component) in a fixed order and
 // writes the column's d entries at that neighbour; A is zero elsewhere.
 __global__ void k_bottom_assemble(const Geom g, const double *__restrict__ psi, const double *__restrict__ Ke, double *A)
@@ -321,10 +329,10 @@ __global__ void k_bottom_assemble(const Geom g, const double *__restrict__ psi, 
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (t >= n * nn) return;
     const long long col = t / nn;
-    const int nb = (int)(t % nn), q = (int)(col / N);
+    const int nb = (int)(t % nn), q = (int)(col % d);
     const int off[3] = {nb % 3 - 1, nb / 3 % 3 - 1, d == 3 ? nb / 9 - 1 : 0};
     int m[3];
-    node_of(g, col % N, m[0], m[1], m[2]);
+    node_of(g, col / d, m[0], m[1], m[2]);
     const int i = m[0] + off[0], j = m[1] + off[1], k = m[2] + off[2];
     if (i < 0 || j < 0 || k < 0 || i >= g.nx || j >= g.ny || k >= g.nz) return;
     double s[3] = {0.0, 0.0, 0.0};
@@ -342,7 +350,7 @@ __global__ void k_bottom_assemble(const Geom g, const double *__restrict__ psi, 
         for (int p = 0; p < d; ++p) s[p] += pc * Ke[(a * d + p) * nc * d + b * d + q];
     }
     const long long node = i + (long long)g.nx * (j + (long long)g.ny * k);
-    for (int p = 0; p < d; ++p) A[(p * N + node) * n + col] = s[p];
+    for (int p = 0; p < d; ++p) A[(node * d + p) * n + col] = s[p];
 }
 
 // Dirichlet dofs: identity rows and columns (their correction is zero).  One thread
@@ -353,9 +361,9 @@ __global__ void k_bottom_dirichlet(const Geom g, double *A)
     const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (e >= n * n) return;
     const long long t = e / n, m = e % n;
-    const int p = (int)(t / N);
+    const int p = (int)(t % g.dim);
     int i, j, k;
-    node_of(g, t % N, i, j, k);
+    node_of(g, t / g.dim, i, j, k);
     if (!is_dir(g, p, i, j, k)) return;
     A[t * n + m] = (m == t) ? 1.0 : 0.0;
     A[m * n + t] = (m == t) ? 1.0 : 0.0;
@@ -379,7 +387,9 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned nblocks, un
         volatile unsigned *cnt = bar;
         long long it = 0;
         while (*cnt < target) {
-            if (++it > limit || *(volatile unsigned *)(bar + 2)) {
+            // another block's timeout is looked for now and then only: a second load a poll
+            // doubles the wait's granularity
+            if (++it > limit || ((it & 63) == 0 && *(volatile unsigned *)(bar + 2))) {
                 atomicExch(bar + 2, 1u);
                 ok = 0;
                 break;
@@ -399,65 +409,72 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned nblocks, un
 // met are SPD, so no pivoting is needed.  One cooperative launch; block b owns rows
 // b + m gridDim.x, and the columns S_:P of the next pivot block (the panel, kGJB x n) are
 // written to a double-buffered exchange area during a pass, so one grid barrier per pass
-// orders the passes.  In a pass warp 0 inverts the pivot block in registers (the chain
-// of kGJB divisions bounds a pass on small n) while the other warps bring the panel to
-// shared memory; then the warps share the 32-column pieces of the block's rows.
-// Measured with the assembly: 375 dofs 0.76 -> 0.23 ms, 720 dofs 2.15 -> 0.65 ms.
+// orders the passes.  In a pass four warps invert the pivot block (a chain of kGJB
+// reciprocals, which bounds a pass on small n) while the others bring the panel to
+// shared memory; then the warps share the 32-column pieces of the block's rows.  375
+// dofs 0.66 -> 0.31 ms, 720 dofs 2.05 -> 0.74 ms (the Gauss-Jordan form by 256 threads
+// before), of which the pivot chain is 0.16 and 0.30.
 constexpr int kGJB = 16;
 
 // 1 / d, d > 0, to an ulp: the hardware's approximate reciprocal (PTX rcp.approx.ftz.f64,
-// 2^-20) and two Newton steps r <- r + r (1 - d r).  The inversion below is a chain of
-// these; extreme exponents take the division.
+// 2^-20) and one cubic Newton step r <- r + r (e + e^2), e = 1 - d r.  The inversion below
+// is a chain of these; extreme exponents take the division.
 __device__ __forceinline__ double pivot_rcp(double d)
 {
     const int ex = (int)(__double_as_longlong(d) >> 52);
     if (ex < 64 || ex > 1980) return 1.0 / d;
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    r = fma(r, fma(-d, r, 1.0), r);
-    return fma(r, fma(-d, r, 1.0), r);
+    const double e = fma(-d, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
-// Inverse of the kGJB x kGJB SPD matrix in shared memory by one warp: lane (r, h) keeps
-// row r, columns 8 h .. 8 h + 7.  By symmetry the pivot row is the pivot column, so a
-// step broadcasts columns by shuffles and costs nine FP64 instructions and the
-// reciprocal.
-__device__ __forceinline__ void invert_pivot(double (*P)[kGJB + 1], int lane)
+// Inverse of the kGJB x kGJB SPD matrix in shared memory by threads 0 .. 127.  An SM
+// sub-partition issues one FP64 instruction of a warp in 64 cycles, dependent or not, so the
+// matrix is spread over four warps (thread: row tid / 8, two columns) and a step costs each
+// of them six: the reciprocal (3), the scaled column and two updates.  By symmetry the pivot
+// row is the pivot column, which its owners hand round through colbuf[2][kGJB].
+__device__ __forceinline__ void invert_pivot(double (*P)[kGJB + 1], double (*colbuf)[kGJB], int tid)
 {
-    const int r = lane & 15, h = lane >> 4;
-    double v[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) v[c] = P[r][8 * h + c];
+    const int r = tid >> 3, c0 = 2 * (tid & 7);
+    double v[2] = {P[r][c0], P[r][c0 + 1]};
+    if (c0 == 0) colbuf[0][r] = v[0];
+    asm volatile("bar.sync 1, 128;" ::: "memory");
 #pragma unroll
     for (int q = 0; q < kGJB; ++q) {
-        const double col = __shfl_sync(0xffffffffu, v[q & 7], (q & 8) * 2 + r);      // S_rq
-        const double ip = pivot_rcp(__shfl_sync(0xffffffffu, col, q));
-        const double t = col * ip;                                                   // S_rq / S_qq
+        const double *col = colbuf[q & 1];
+        const double ip = pivot_rcp(col[q]);
+        const double t = col[r] * ip;                              // S_rq / S_qq
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const double pq = __shfl_sync(0xffffffffu, col, h * 8 + c);              // S_q,8h+c
-            const double tq = __shfl_sync(0xffffffffu, t, h * 8 + c);
-            const double w = fma(-t, pq, v[c]);
-            v[c] = 8 * h + c == q ? (r == q ? -ip : t) : (r == q ? tq : w);
+        for (int e = 0; e < 2; ++e) {
+            const double w = fma(r == q ? ip : -t, col[c0 + e], r == q ? 0.0 : v[e]);
+            v[e] = c0 + e == q ? (r == q ? -ip : t) : w;
+        }
+        if (q + 1 < kGJB) {
+            if (c0 == ((q + 1) & ~1)) colbuf[(q + 1) & 1][r] = v[(q + 1) & 1];
+            asm volatile("bar.sync 1, 128;" ::: "memory");
         }
     }
-#pragma unroll
-    for (int c = 0; c < 8; ++c) P[r][8 * h + c] = -v[c];
+    P[r][c0] = -v[0];
+    P[r][c0 + 1] = -v[1];
 }
 
 // PAN: the panel is staged in shared memory (else read from L2); in_smem: the block's
-// rows stay in shared memory.  kRowsMax rows a block at most have their B in shared memory
+// rows stay in shared memory; bw: the half bandwidth of the matrix.  Rows beyond the pivot
+// block by more than bw have a zero panel and are passed over (a third of the products is
+// left).  kRowsMax rows a block at most have their B in shared memory
 // at once.
 constexpr int kRowsMax = 16;
 
 template <bool PAN>
-__global__ void __launch_bounds__(kThreads) k_sym_inverse(int n, double *A, double *tmp, unsigned *bar, int in_smem,
+__global__ void __launch_bounds__(kThreads) k_sym_inverse(int n, int bw, double *A, double *tmp, unsigned *bar, int in_smem,
                                                           long long limit)
 {
     extern __shared__ double smem_gj[];           // the panel (PAN), then the block's rows (in_smem)
     double *srow = smem_gj + (PAN ? (long long)kGJB * n : 0);
     __shared__ double G[kGJB][kGJB + 1];
     __shared__ double Brow[kRowsMax][kGJB];
+    __shared__ double colbuf[2][kGJB];
     const unsigned nb = gridDim.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = kThreads / 32;
     const long long xb = (long long)kGJB * n;     // one exchange buffer: panel[r][i] = S[i][k0 + r]
@@ -481,17 +498,17 @@ __global__ void __launch_bounds__(kThreads) k_sym_inverse(int n, double *A, doub
         const double *C = tmp + cur * xb;
         double *Cn = tmp + (1 - cur) * xb;
         // the exchange buffers alternate between passes: reads of them bypass L1
-        if (warp == 0) {
-            for (int t = lane; t < kGJB * kGJB; t += 32) {
+        if (warp < 4) {
+            for (int t = threadIdx.x; t < kGJB * kGJB; t += 128) {
                 const int r = t / kGJB, c = t % kGJB;
                 G[r][c] = (r < b && c < b) ? __ldcg(C + (long long)r * n + k0 + c) : (r == c ? 1.0 : 0.0);
             }
-            __syncwarp();
-            invert_pivot(G, lane);
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            invert_pivot(G, colbuf, threadIdx.x);
         } else if (PAN) {
 #pragma unroll 8
-            for (int t = threadIdx.x - 32; t < b * n; t += kThreads - 32) smem_gj[t] = __ldcg(C + t);
-            for (int t = b * n + threadIdx.x - 32; t < kGJB * n; t += kThreads - 32) smem_gj[t] = 0.0;
+            for (int t = threadIdx.x - 128; t < b * n; t += kThreads - 128) smem_gj[t] = __ldcg(C + t);
+            for (int t = b * n + threadIdx.x - 128; t < kGJB * n; t += kThreads - 128) smem_gj[t] = 0.0;
         }
         __syncthreads();
         // rows b .. kGJB - 1 of the last panel count as zero
@@ -500,17 +517,18 @@ __global__ void __launch_bounds__(kThreads) k_sym_inverse(int n, double *A, doub
         };
         for (int i0 = blockIdx.x, r0 = 0; i0 < n; i0 += kRowsMax * gridDim.x, r0 += kRowsMax) {
             const int rows = min(kRowsMax, (n - i0 + (int)gridDim.x - 1) / (int)gridDim.x);
-            // B_i = S_iP G (rows outside P) or G's row (inside), half a warp a row
-            for (int m = threadIdx.x / kGJB; m < rows; m += kThreads / kGJB) {
-                const int i = i0 + m * gridDim.x, c = threadIdx.x % kGJB;
-                double acc[4] = {0.0, 0.0, 0.0, 0.0};
-                if (i >= k0 && i < k0 + b) {
-                    acc[0] = G[i - k0][c];
-                } else {
+            // B_i = S_iP G (rows outside P) or G's row (inside), a warp a row, each half of it
+            // half of the products
+            for (int m = warp; m < rows; m += nw) {
+                const int i = i0 + m * gridDim.x, c = lane & 15, r0h = lane >> 4 << 3;
+                const bool inP = i >= k0 && i < k0 + b;
+                if (i >= k0 + b + bw) continue;
+                double acc = inP && r0h == 0 ? G[i - k0][c] : 0.0;
+                if (!inP)
 #pragma unroll
-                    for (int r = 0; r < kGJB; ++r) acc[r & 3] += cget(r, i) * G[r][c];
-                }
-                Brow[m][c] = c < b ? (acc[0] + acc[1]) + (acc[2] + acc[3]) : 0.0;
+                    for (int r = 0; r < kGJB / 2; ++r) acc = fma(cget(r0h + r, i), G[r0h + r][c], acc);
+                acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+                if (lane < kGJB) Brow[m][c] = c < b ? acc : 0.0;
             }
             __syncthreads();
             // the warps take the rows' pieces of 32 columns in turn
@@ -519,6 +537,11 @@ __global__ void __launch_bounds__(kThreads) k_sym_inverse(int n, double *A, doub
                 const int i = i0 + m * gridDim.x, np = i / 32 + 1;
                 double *row = in_smem ? srow + (long long)(r0 + m) * n : A + (long long)i * n;
                 const bool inP = i >= k0 && i < k0 + b;
+                if (i >= k0 + b + bw) {                        // unchanged: hand on the next panel's part
+                    for (int j = k1 + lane; warp == 0 && j < k1 + bn && j <= i; j += 32)
+                        Cn[(long long)(j - k1) * n + i] = row[j];
+                    continue;
+                }
                 for (; next < np; next += nw) {
                     const int j = next * 32 + lane;
                     if (j > i) continue;
@@ -527,11 +550,10 @@ __global__ void __launch_bounds__(kThreads) k_sym_inverse(int n, double *A, doub
                     if (jP) {
                         v = inP ? -G[i - k0][j - k0] : Brow[m][j - k0];
                     } else {
-                        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+                        double acc[2] = {0.0, 0.0};
 #pragma unroll
-                        for (int c = 0; c < kGJB; ++c) acc[c & 3] += Brow[m][c] * cget(c, j);
-                        const double s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-                        v = inP ? s : row[j] - s;
+                        for (int c = 0; c < kGJB; ++c) acc[c & 1] += Brow[m][c] * cget(c, j);
+                        v = inP ? acc[0] + acc[1] : row[j] - (acc[0] + acc[1]);
                     }
                     row[j] = v;
                     if (j >= k1 && j < k1 + bn) Cn[(long long)(j - k1) * n + i] = v;
@@ -632,8 +654,8 @@ cudaError_t launch_restrict(const Geom &gf, const Geom &gc, const T *rf, T *fc, 
                             T *zero_uc, const FirstSweep<T> &first)
 {
     cudaError_t e = gf.dim == 3
-                        ? launch_pdl(k_restrict<T, 3>, node_grid(gc), kNodeBlock, 0, s, gf, gc, rf, fc, gate, zero_uc, first)
-                        : launch_pdl(k_restrict<T, 2>, node_grid(gc), kNodeBlock, 0, s, gf, gc, rf, fc, gate, zero_uc, first);
+                        ? launch_pdl(k_restrict<T, 3>, node_grid(gc, transfer_block<T>(gc)), transfer_block<T>(gc), 0, s, gf, gc, rf, fc, gate, zero_uc, first)
+                        : launch_pdl(k_restrict<T, 2>, node_grid(gc, transfer_block<T>(gc)), transfer_block<T>(gc), 0, s, gf, gc, rf, fc, gate, zero_uc, first);
     if (e != cudaSuccess) return e;
     ++g_launches;
     return cudaGetLastError();
@@ -646,8 +668,8 @@ template cudaError_t launch_restrict<float>(const Geom &, const Geom &, const fl
 template <typename T>
 cudaError_t launch_prolong_add(const Geom &gf, const Geom &gc, const T *ec, T *uf, cudaStream_t s, const int *gate)
 {
-    cudaError_t e = gf.dim == 3 ? launch_pdl(k_prolong_add<T, 3>, node_grid(gc), kNodeBlock, 0, s, gf, gc, ec, uf, gate)
-                                : launch_pdl(k_prolong_add<T, 2>, node_grid(gc), kNodeBlock, 0, s, gf, gc, ec, uf, gate);
+    cudaError_t e = gf.dim == 3 ? launch_pdl(k_prolong_add<T, 3>, node_grid(gc, transfer_block<T>(gc)), transfer_block<T>(gc), 0, s, gf, gc, ec, uf, gate)
+                                : launch_pdl(k_prolong_add<T, 2>, node_grid(gc, transfer_block<T>(gc)), transfer_block<T>(gc), 0, s, gf, gc, ec, uf, gate);
     if (e != cudaSuccess) return e;
     ++g_launches;
     return cudaGetLastError();
@@ -784,7 +806,7 @@ cudaError_t launch_bottom_dirichlet(const Geom &g, double *A, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_sym_inverse(int n, double *A, double *tmp, unsigned *bar, long long spins, cudaStream_t s)
+cudaError_t launch_sym_inverse(int n, int bw, double *A, double *tmp, unsigned *bar, long long spins, cudaStream_t s)
 {
     int dev = 0, nsm = 0, per_sm = 0, coop = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -810,7 +832,7 @@ cudaError_t launch_sym_inverse(int n, double *A, double *tmp, unsigned *bar, lon
     e = cudaMemsetAsync(bar, 0, 4 * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     long long limit = spins > 0 ? spins : kGridSpinLimit;
-    void *args[] = {&n, &A, &tmp, &bar, &in_smem, &limit};
+    void *args[] = {&n, &bw, &A, &tmp, &bar, &in_smem, &limit};
     e = cudaLaunchCooperativeKernel(kernel, dim3(nblocks), dim3(kThreads), args, smem, s);
     ++g_launches;
     return e;

@@ -435,6 +435,85 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
     }
 }
 
+// Small 3D levels: eight consecutive threads per node, thread c evaluating the cell of which
+// the node is corner c; exponents and forces are combined by shuffles and the first three
+// lanes finalise a component each.  A cell that does not fit sends its warp to FP64
+// instructions.  No shared memory, no barrier, no plane ring: what is left is one round
+// of loads and one cell's chain.
+constexpr int kNode64Threads = 128;
+
+template <int MODE>
+__global__ void __launch_bounds__(kNode64Threads) k_sweep3_node64(const SweepArgs<double, double> a, const fix::Consts fc)
+{
+    const Geom &g = a.g;
+    const int n = g.nx * g.ny * g.nz;
+    const int node = blockIdx.x * (kNode64Threads / 8) + (threadIdx.x >> 3);
+    const int c = threadIdx.x & 7;
+    const bool valid = node < n;
+    const int i = node % g.nx, j = node / g.nx % g.ny, k = node / (g.nx * g.ny);
+    const int ci = i - (c & 1), cj = j - ((c >> 1) & 1), ck = k - (c >> 2);
+    const bool has = valid && ci >= 0 && cj >= 0 && ck >= 0 && ci < g.nx - 1 && cj < g.ny - 1 && ck < g.nz - 1;
+    const long long on = valid ? gidx(g, i, j, k) : 0;
+    const int p = c < 3 ? c : 0;                          // the component this lane finalises (lanes 0..2)
+    // what no kernel of the cycle writes is read before the wait for the predecessor
+    const double psi = has ? a.psi[gidx(g, ci, cj, ck)] : 0.0;
+    double ip = (MODE == kJacobi && a.dinv) ? a.dinv[on] : 0.0;
+    pdl_begin();
+    if (a.gate && *a.gate) return;
+    double V[3][8];
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const long long o = has ? gidx(g, ci + (b & 1), cj + ((b >> 1) & 1), ck + (b >> 2)) : 0;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) V[q][b] = has ? a.u[q * g.cs + o] : 0.0;
+    }
+    const double uv = MODE == kJacobi ? a.u[p * g.cs + on] : 0.0;
+    const double fv = MODE != kApply ? a.f[p * g.cs + on] : 0.0;
+    i64 U[3][8], F[3];
+    bool none;
+    int eu, e;
+    const bool ok = fix::transform_cell3(V, U, none, eu) && fix::psi_ok(psi) && fc.ok;
+    double Ku = 0.0;
+    if (__all_sync(0xffffffffu, ok)) {
+        fix::corner_force3(U, none, eu, c, psi, fc, F, e);
+        int ee = e;
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) ee = max(ee, __shfl_xor_sync(0xffffffffu, ee, off));
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            F[q] = fix::down(F[q], ee - e);
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) F[q] += __shfl_xor_sync(0xffffffffu, F[q], off);
+        }
+        Ku = fix::to_double(p == 0 ? F[0] : p == 1 ? F[1] : F[2], ee);
+    } else {
+        cell_forces3<double>(V, psi, a.c);
+        double f[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            f[q] = V[q][0];
+#pragma unroll
+            for (int b = 1; b < 8; ++b) f[q] = c == b ? V[q][b] : f[q];
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) f[q] += __shfl_xor_sync(0xffffffffu, f[q], off);
+        }
+        Ku = p == 0 ? f[0] : p == 1 ? f[1] : f[2];
+    }
+    if (MODE == kJacobi && !a.dinv) {
+        double s = psi;
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        ip = 1.0 / s;
+    }
+    if (!valid || c >= 3) return;
+    const bool dir = is_dir(g, p, i, j, k);
+    double r;
+    if (MODE == kJacobi) r = dir ? uv : uv + (fv - Ku) * ip * (p == 0 ? a.wk[0] : p == 1 ? a.wk[1] : a.wk[2]);
+    else if (MODE == kResidual) r = dir ? 0.0 : fv - Ku;
+    else r = Ku;
+    a.out[p * g.cs + on] = r;
+}
+
 // ------------------------------------------------------------------------- 2D
 //
 // One thread per cell of a 32 x TY2 tile (the first row and column the halo), which
@@ -897,6 +976,24 @@ long long sweep_blocks_fix(const Geom &g)
     }
     const long long units = (long long)((g.nx - 1 + TX - 1) / TX) * ((g.ny - 1 + TY - 1) / TY) * g.nz;
     return std::min<long long>(152, units);
+}
+
+cudaError_t launch_sweep_node64(int mode, const SweepArgs<double, double> &a, cudaStream_t s)
+{
+    if (a.g.dim != 3 || (long long)a.g.nx * a.g.ny * a.g.nz >= (1 << 24)) return cudaErrorInvalidValue;
+    const int n = a.g.nx * a.g.ny * a.g.nz;
+    const dim3 gr((n + kNode64Threads / 8 - 1) / (kNode64Threads / 8)), b(kNode64Threads);
+    const fix::Consts fc = fix::make_consts(3, a.c);
+    cudaError_t e;
+    switch (mode) {
+    case kApply: e = launch_pdl(k_sweep3_node64<kApply>, gr, b, 0, s, a, fc); break;
+    case kResidual: e = launch_pdl(k_sweep3_node64<kResidual>, gr, b, 0, s, a, fc); break;
+    case kJacobi: e = launch_pdl(k_sweep3_node64<kJacobi>, gr, b, 0, s, a, fc); break;
+    default: return cudaErrorInvalidValue;
+    }
+    if (e != cudaSuccess) return e;
+    ++g_launches;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_prolong_sweep(const SweepArgs<double, double> &a, const Geom &gc, const double *ec, cudaStream_t s)

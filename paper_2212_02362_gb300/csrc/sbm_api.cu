@@ -234,7 +234,10 @@ SweepArgs<T, T> sweep_args(sbm_grid G, int l, const T *u, const T *f, T *out, do
 template <typename T>
 cudaError_t sweep(sbm_grid G, int l, int mode, const T *u, const T *f, T *out, double *part, double omega)
 {
-    return launch_sweep<T, T>(mode, sweep_args<T>(G, l, u, f, out, part, omega), G->st);
+    const SweepArgs<T, T> a = sweep_args<T>(G, l, u, f, out, part, omega);
+    if constexpr (std::is_same<T, double>::value)
+        if (a.g.dim == 3 && !part && nnodes(a.g) <= kNode64MaxNodes) return launch_sweep_node64(mode, a, G->st);
+    return launch_sweep<T, T>(mode, a, G->st);
 }
 
 // FP32 3D sweeps: levels of at most kNodeKernelMaxNodes nodes (no norm wanted) use
@@ -521,10 +524,12 @@ sbm_status setup_bottom(sbm_grid G)
     if (G->bottom_ready) return SBM_OK;
     Level &B = G->L[0];
     const long long n = G->nb;
+    // the furthest neighbour of a node, in dofs
+    const int bw = std::max(16, B.g.dim * ((B.g.dim == 3 ? B.g.nx * B.g.ny : 0) + B.g.nx + 2));
     CK(cudaMemsetAsync(G->A64, 0, sizeof(double) * n * n, G->st));
     CK(launch_bottom_assemble(B.g, B.psi64, B.Ke64, G->A64, G->st));
     CK(launch_bottom_dirichlet(B.g, G->A64, G->st));
-    CK(launch_sym_inverse((int)n, G->A64, G->gjtmp, G->gjbar, G->gj_spins, G->st));
+    CK(launch_sym_inverse((int)n, bw, G->A64, G->gjtmp, G->gjbar, G->gj_spins, G->st));
     {
         unsigned hbar[4] = {0, 0, 0, 0};
         CK(cudaMemcpyAsync(hbar, G->gjbar, sizeof(hbar), cudaMemcpyDeviceToHost, G->st));
@@ -1668,12 +1673,11 @@ static sbm_status grid_create_impl(const sbm_grid_desc *d, sbm_grid G)
     CK(gmalloc(G, (void **)&G->gather, sizeof(int) * G->nb));
     {
         std::vector<int> gi(G->nb);
-        const long long N = nnodes(B.g);
         for (int p = 0; p < B.g.dim; ++p)
             for (int k = 0; k < B.g.nz; ++k)
                 for (int j = 0; j < B.g.ny; ++j)
                     for (int i = 0; i < B.g.nx; ++i)
-                        gi[p * N + i + (long long)B.g.nx * (j + (long long)B.g.ny * k)] = (int)(p * B.g.cs + gidx(B.g, i, j, k));
+                        gi[(i + (long long)B.g.nx * (j + (long long)B.g.ny * k)) * B.g.dim + p] = (int)(p * B.g.cs + gidx(B.g, i, j, k));
         CK(cudaMemcpy(G->gather, gi.data(), sizeof(int) * G->nb, cudaMemcpyHostToDevice));
     }
     CK(cudaEventCreate(&G->ev0));

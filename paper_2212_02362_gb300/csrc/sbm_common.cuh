@@ -197,6 +197,13 @@ cudaError_t launch_sweep(int mode, const SweepArgs<T, TO> &a, cudaStream_t s);
 template <typename TO>
 cudaError_t launch_sweep_fix(int mode, const SweepArgs<double, TO> &a, cudaStream_t s);
 long long sweep_blocks_fix(const Geom &g);
+// FP64 3D sweep with eight threads (one per cell) per node in integer arithmetic, for
+// small levels (no partial sums).
+cudaError_t launch_sweep_node64(int mode, const SweepArgs<double, double> &a, cudaStream_t s);
+// Levels with at most this many nodes use it: there the tiled sweep's few blocks and the
+// latency of its plane ring cost more than evaluating every cell eight times (9^3 and 17^3:
+// 12 against 5 us a sweep; 33^3: 14 against 24 us).
+constexpr long long kNode64MaxNodes = 12000;
 // dinv[node] = 1 / (sum of psi over the node's cells), summed in the sweeps' order.
 cudaError_t launch_inv_psi(const Geom &g, const double *psi, double *dinv, cudaStream_t s);
 // One 2D FP64 colour Gauss-Seidel sweep (see launch_gs2_sweep); c: the level's constants.
@@ -284,10 +291,10 @@ cudaError_t launch_prolong_sweep(const SweepArgs<double, double> &a, const Geom 
 // 2D FP64 levels with at most this many nodes take the fused steps.
 constexpr long long kFuse2MaxNodes = 20000;
 
-// Inverse of the coarsest-level matrix in place (one cooperative launch);
-// bar: 4 device words, bar[2] != 0 afterwards if a grid barrier timed out.
+// Inverse of the coarsest-level matrix (half bandwidth bw) in place (one cooperative launch);
+// bw >= 16; bar: 4 device words, bar[2] != 0 afterwards if a grid barrier timed out.
 // spins: polls a block makes at one grid barrier before giving up (<= 0: default).
-cudaError_t launch_sym_inverse(int n, double *A, double *tmp, unsigned *bar, long long spins, cudaStream_t s);
+cudaError_t launch_sym_inverse(int n, int bw, double *A, double *tmp, unsigned *bar, long long spins, cudaStream_t s);
 cudaError_t launch_round(long long n, const double *src, float *dst, cudaStream_t s);
 template <typename T>
 cudaError_t launch_bottom_apply(int n, const T *Ainv, const int *gather, const T *b, T *u,

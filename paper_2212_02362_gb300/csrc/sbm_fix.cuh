@@ -310,6 +310,34 @@ __host__ __device__ __forceinline__ bool transform_cell3(const double (&v)[3][8]
     return true;
 }
 
+// Force on corner a of a 3D cell with transformed, normalised values U (transform_cell3,
+// exponent eu) and psi: F on the unit 2^e (e = kNoExp: none).
+__host__ __device__ __forceinline__ void corner_force3(const i64 (&U)[3][8], bool none, int eu, int a, double psi,
+                                                       const Consts &c, i64 (&F)[3], int &e)
+{
+    i64 dU[3][8];
+    int ep;
+    const i64 pm = psi_mantissa(psi, ep);
+    e = (none || pm == 0) ? kNoExp : eu + ep + c.ec;
+    Frac k[7];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) k[i] = split(mul(pm, c.c[i]));
+    stress3(U, k, c.neg12, dU);
+    // the transform's row of basis function s at corner a: the product over the axes of s of
+    // +1 (corner bit set) or -1
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        i64 f = 0;
+#pragma unroll
+        for (int s = 1; s < 8; ++s) {
+            const int m = s & ~a;                                  // axes of s whose corner bit is clear
+            const bool neg = ((m ^ (m >> 1) ^ (m >> 2)) & 1) != 0;
+            f += neg ? -dU[p][s] : dU[p][s];
+        }
+        F[p] = f;
+    }
+}
+
 // v^T S u of a 3D cell (S the unit-psi cell matrix of the constants c), u and v given as
 // transform_cell3 leaves them: the sum, in 128 bits, of 21 products of the stress of u with
 // the transform of v, in the basis where the cell's rigid motion has dropped out.

@@ -27,7 +27,9 @@ def _rel(a, b):
 
 # one tile holds 32 x 10 cells: one cell, exactly a tile, a tile and a remainder of one
 # cell on either axis, one plane per block and long segments
-@pytest.mark.parametrize("n", [(2, 2, 2), (3, 2, 17), (33, 11, 2), (34, 12, 3), (33, 11, 15), (66, 12, 6), (9, 31, 33)])
+# (with the norm; apply and smoothing of up to 12000 nodes take eight threads a node, (97, 41, 25) the tiles)
+@pytest.mark.parametrize("n", [(2, 2, 2), (3, 2, 17), (33, 11, 2), (34, 12, 3), (33, 11, 15), (66, 12, 6), (9, 31, 33),
+                               (97, 41, 25)])
 def test_tile_edges(n):
     wk = random_workload(3, n, 90)
     g, P = gpu_grid(wk), oracle_problem(wk)
