@@ -72,6 +72,29 @@ __global__ void k_restrict(const Geom gf, const Geom gc, const T *__restrict__ r
 }
 
 template <typename T, int D>
+__global__ void k_first_sweep(const Geom st, const Geom v, int off, const T *__restrict__ f, const FirstSweep<T> first,
+                              T *__restrict__ zero)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    const int k = blockIdx.z * blockDim.z + threadIdx.z;
+    const bool in = i < st.nx && j < st.ny && k < st.nz;
+    const int vi = i - off, vj = j - off, vk = D == 3 ? k - off : 0;
+    const bool view = vi >= 0 && vj >= 0 && vk >= 0 && vi < v.nx && vj < v.ny && vk < v.nz;
+    T ip = T(0);
+    if (in && view) ip = first.dinv ? first.dinv[gidx(v, vi, vj, vk)] : body::inv_psi_sum<T, D>(v, first.psi, vi, vj, vk);
+    pdl_begin();
+    if (!in) return;
+    const long long o = gidx(st, i, j, k);
+#pragma unroll
+    for (int p = 0; p < D; ++p) {
+        first.u[p * st.cs + o] =
+            (view && !is_dir(v, p, vi, vj, vk)) ? f[p * st.cs + o] * ip * first.wk[p] : T(0);
+        if (zero && !view) zero[p * st.cs + o] = T(0);
+    }
+}
+
+template <typename T, int D>
 __global__ void k_prolong_add(const Geom gf, const Geom gc, const T *__restrict__ ec, T *__restrict__ uf,
                               const int *gate)
 {
@@ -664,6 +687,21 @@ template cudaError_t launch_restrict<double>(const Geom &, const Geom &, const d
                                              const int *, double *, const FirstSweep<double> &);
 template cudaError_t launch_restrict<float>(const Geom &, const Geom &, const float *, float *, cudaStream_t, const int *,
                                             float *, const FirstSweep<float> &);
+
+template <typename T>
+cudaError_t launch_first_sweep(const Geom &st, const Geom &v, int off, const T *f, const FirstSweep<T> &first, T *zero,
+                               cudaStream_t s)
+{
+    cudaError_t e = st.dim == 3 ? launch_pdl(k_first_sweep<T, 3>, node_grid(st), kNodeBlock, 0, s, st, v, off, f, first, zero)
+                                : launch_pdl(k_first_sweep<T, 2>, node_grid(st), kNodeBlock, 0, s, st, v, off, f, first, zero);
+    if (e != cudaSuccess) return e;
+    ++g_launches;
+    return cudaGetLastError();
+}
+template cudaError_t launch_first_sweep<double>(const Geom &, const Geom &, int, const double *, const FirstSweep<double> &,
+                                                double *, cudaStream_t);
+template cudaError_t launch_first_sweep<float>(const Geom &, const Geom &, int, const float *, const FirstSweep<float> &,
+                                               float *, cudaStream_t);
 
 template <typename T>
 cudaError_t launch_prolong_add(const Geom &gf, const Geom &gc, const T *ec, T *uf, cudaStream_t s, const int *gate)

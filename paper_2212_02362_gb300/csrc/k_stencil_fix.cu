@@ -952,7 +952,8 @@ cudaError_t launch_fix_mode(const SweepArgs<double, TO> &a, cudaStream_t s)
         static std::atomic<unsigned long long> attr_done{0};
         e = smem_attr_once(reinterpret_cast<const void *>(k_sweep3_fix<TO, MODE>), kSmem, attr_done);
         if (e != cudaSuccess) return e;
-        e = launch_pdl(k_sweep3_fix<TO, MODE>, dim3((unsigned)sweep_blocks_fix(a.g)), dim3(NT), kSmem, s, a, fc);
+        e = launch_pdl(k_sweep3_fix<TO, MODE>, dim3((unsigned)(a.max_ctas ? std::min<long long>(sweep_blocks_fix(a.g), a.max_ctas) : sweep_blocks_fix(a.g))),
+                       dim3(NT), kSmem, s, a, fc);
     } else {
         const int ty = rows2(a.g);
         const dim3 gr((a.g.nx + 30) / 32, (a.g.ny - 2 + ty) / ty), b(33 * (ty + 1));

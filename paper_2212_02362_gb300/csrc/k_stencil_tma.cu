@@ -566,7 +566,7 @@ static cudaError_t launch_f2_mode(const SweepArgs<float, float> &a, const CUtens
     static std::atomic<unsigned long long> attr_done{0};
     cudaError_t ea = smem_attr_once(reinterpret_cast<const void *>(k_sweep3_f2<MODE>), kSmemBytes, attr_done);
     if (ea != cudaSuccess) return ea;
-    cudaError_t e = launch_pdl(k_sweep3_f2<MODE>, dim3(ctas_f2(a.g)), dim3(BXP, BYP), kSmemBytes, s, tmap[0], tmap[1],
+    cudaError_t e = launch_pdl(k_sweep3_f2<MODE>, dim3(a.max_ctas ? std::min(ctas_f2(a.g), a.max_ctas) : ctas_f2(a.g)), dim3(BXP, BYP), kSmemBytes, s, tmap[0], tmap[1],
                                tmap[2], a, org, err);
     if (e != cudaSuccess) return e;
     ++g_launches;

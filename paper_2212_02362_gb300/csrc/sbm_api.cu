@@ -82,6 +82,10 @@ struct Patch {
 };
 
 constexpr int kBranches = 8;   // side streams for concurrent patches
+// CTAs handed out to the patches in flight: two per SM's worth, since a sweep's CTAs finish at
+// different times (refined 3D voids: 29.0 ms without shares, 30.1 with 152, 28.1 with 228,
+// 27.7 with 304).
+constexpr double kShareCtas = 304;
 
 struct GraphSlot {
     bool valid = false;
@@ -116,6 +120,7 @@ struct sbm_grid_s {
     int *derr = nullptr;        // device error flag of the TMA kernels
     int *dgate = nullptr;       // adaptive inner cycles: [0] gate flag, [1] FP32 V-cycles run
     const int *cur_gate = nullptr;   // gate applied to the launches being enqueued (or null)
+    int cur_ctas = 0;           // CTAs of the persistent sweeps being enqueued (0: one per SM)
     double gate_rtol = 0, gate_tol = 0;
     double *scal = nullptr;     // device scalars, see k_norm_final
     double *hscal = nullptr;    // pinned host copy
@@ -227,6 +232,7 @@ SweepArgs<T, T> sweep_args(sbm_grid G, int l, const T *u, const T *f, T *out, do
     for (int p = 0; p < 3; ++p) a.wk[p] = (L.c64.kdiag[p] != 0.0) ? T(omega / L.c64.kdiag[p]) : T(0);
     a.kchunk = 0;
     a.gate = G->cur_gate;
+    a.max_ctas = part ? 0 : G->cur_ctas;
     if constexpr (std::is_same<T, double>::value) a.dinv = G->dinv_ready ? L.dinv : nullptr;
     return a;
 }
@@ -354,6 +360,18 @@ FirstSweep<T> first_sweep_of(sbm_grid G, int l, const sbm_opts &o)
     return a;
 }
 
+// A zero correction on level l, with Jacobi smoothing right away its first sweep (cur = 1
+// then: one pre-smoothing sweep done).
+template <typename T>
+cudaError_t zero_start(sbm_grid G, int l, int &cur, const sbm_opts &o, const T *f)
+{
+    Level &L = G->L[l];
+    const FirstSweep<T> first = first_sweep_of<T>(G, l, o);
+    cur = first.u ? 1 : 0;
+    if (!first.u) return cudaMemsetAsync(P<T>::u(L, 0), 0, (size_t)L.g.dim * L.g.cs * sizeof(T), G->st);
+    return launch_first_sweep<T>(L.g, L.g, 0, f, first, nullptr, G->st);
+}
+
 // Levels whose V-cycle steps run fused: small ones, where a launch costs more than its
 // work, with Jacobi smoothing.
 template <typename T>
@@ -454,8 +472,9 @@ cudaError_t enqueue_body(sbm_grid G, const sbm_opts &o, const double *rhs)
     const int fine = G->nl - 1;
     Level &L = G->L[fine];
     if (G->desc.precision == SBM_MIXED) {
-        CKE(cudaMemsetAsync(L.su[0], 0, level_bytes(L, sizeof(float)), G->st));
         int cur = 0;
+        CKE(zero_start<float>(G, fine, cur, o, L.sf));
+        const int pre = cur;
         if (o.inner_rtol > 0.0) {
             CKE(cudaMemsetAsync(G->dgate, 0, sizeof(int), G->st));
             G->cur_gate = G->dgate;
@@ -463,7 +482,8 @@ cudaError_t enqueue_body(sbm_grid G, const sbm_opts &o, const double *rhs)
             G->gate_tol = 0.5 * o.tol;      // margin: the FP32 residual may underestimate the FP64 one
         }
         cudaError_t e = cudaSuccess;
-        for (int it = 0; it < o.inner_cycles && e == cudaSuccess; ++it) e = vcycle<float>(G, fine, cur, o, L.sf);
+        for (int it = 0; it < o.inner_cycles && e == cudaSuccess; ++it)
+            e = vcycle<float>(G, fine, cur, o, L.sf, it == 0 ? pre : 0);
         G->cur_gate = nullptr;
         CKE(e);
         CKE(launch_add<float>((long long)L.g.dim * L.g.cs, L.su[cur], L.du[0], G->st));
@@ -852,11 +872,19 @@ cudaError_t amr_branches(sbm_grid G, const std::vector<int> &list, F &&work)
     CKE(cudaEventRecord(G->fork_ev, main));
     for (int b = 0; b < nb; ++b) CKE(cudaStreamWaitEvent(G->side[b], G->fork_ev, 0));
     cudaError_t err = cudaSuccess;
+    // The persistent 3D sweeps run one CTA per SM, so sweeps of several patches would queue
+    // for the SMs, each in more and shorter z segments than it needs: a patch gets the
+    // share of the SMs that its nodes have among the patches in flight.
+    double total = 0.0;
+    for (int a : list) total += (double)nnodes(amr_geom(G, a));
+    total *= (double)nb / (double)list.size();
     for (size_t i = 0; i < list.size() && err == cudaSuccess; ++i) {
         G->st = G->side[i % nb];
+        G->cur_ctas = std::max(2, (int)std::ceil(kShareCtas * (double)nnodes(amr_geom(G, list[i])) / total));
         err = work(list[i]);
     }
     G->st = main;
+    G->cur_ctas = 0;
     for (int b = 0; b < nb; ++b) {
         cudaError_t e = cudaEventRecord(G->join_ev[b], G->side[b]);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(main, G->join_ev[b], 0);
@@ -914,6 +942,7 @@ cudaError_t sweep_view(sbm_grid G, Patch &Pt, int mode, const T *u, const T *f, 
             a.c = Pt.c32;
             for (int p = 0; p < 3; ++p) a.wk[p] = (Pt.c64.kdiag[p] != 0.0) ? float(omega / Pt.c64.kdiag[p]) : 0.f;
             a.kchunk = 0;
+            a.max_ctas = G->cur_ctas;
             return launch_sweep_f2(mode, a, Pt.tm32[u == Pt.se[0] ? 0 : 1], G->derr, G->st, make_int3(1, 1, 1));
         }
     }
@@ -927,7 +956,21 @@ cudaError_t sweep_view(sbm_grid G, Patch &Pt, int mode, const T *u, const T *f, 
     a.c = PP<T>::c(Pt);
     for (int p = 0; p < 3; ++p) a.wk[p] = (Pt.c64.kdiag[p] != 0.0) ? T(omega / Pt.c64.kdiag[p]) : T(0);
     a.kchunk = 0;
+    a.max_ctas = G->cur_ctas;
     return launch_sweep<T, T>(mode, a, G->st);
+}
+
+// The first Jacobi sweep of a patch from a zero correction into e(1), both corrections zero
+// on the padding (no memset, no stencil); cur and the sweeps done follow.
+template <typename T>
+cudaError_t patch_first(sbm_grid G, Patch &Pt, int &cur, const sbm_opts &o)
+{
+    FirstSweep<T> a;
+    a.psi = PP<T>::psi(Pt) + Pt.voff;
+    a.u = PP<T>::e(Pt, 1);
+    for (int p = 0; p < 3; ++p) a.wk[p] = (Pt.c64.kdiag[p] != 0.0) ? T(o.omega / Pt.c64.kdiag[p]) : T(0);
+    cur = 1;
+    return launch_first_sweep<T>(Pt.s, Pt.v, 1, PP<T>::rhs(Pt), a, PP<T>::e(Pt, 0), G->st);
 }
 
 template <typename T>
@@ -1022,19 +1065,23 @@ cudaError_t amr_cycle(sbm_grid G, const sbm_opts &o, double *const *target = nul
     for (int L = (int)lev.size() - 1; L >= 1; --L)
         CKE(amr_branches(G, lev[L], [&](int a) -> cudaError_t {
             Patch &Pt = G->P[a - 1];
-            CKE(cudaMemsetAsync(PP<T>::e(Pt, 0), 0, patch_bytes(Pt, sizeof(T)), G->st));
-            CKE(cudaMemsetAsync(PP<T>::e(Pt, 1), 0, patch_bytes(Pt, sizeof(T)), G->st));
             cur[a] = 0;
-            CKE(patch_smooth<T>(G, Pt, cur[a], o, o.nu1, false));
+            if (o.smoother == SBM_JACOBI && o.nu1 > 0) {
+                CKE(patch_first<T>(G, Pt, cur[a], o));
+            } else {
+                CKE(cudaMemsetAsync(PP<T>::e(Pt, 0), 0, patch_bytes(Pt, sizeof(T)), G->st));
+                CKE(cudaMemsetAsync(PP<T>::e(Pt, 1), 0, patch_bytes(Pt, sizeof(T)), G->st));
+            }
+            CKE(patch_smooth<T>(G, Pt, cur[a], o, o.nu1 - cur[a], false));
             CKE(sweep_view<T>(G, Pt, kResidual, PP<T>::e(Pt, cur[a]), PP<T>::rhs(Pt), PP<T>::res(Pt), 0.0));
             const int pa = Pt.parent;
             return launch_amr_restrict<T>(Pt.s, Pt.info, amr_geom(G, pa), amr_info(G, pa), PP<T>::res(Pt),
                                           amr_rhs<T>(G, pa), G->st);
         }));
     T *base_rhs = std::is_same<T, double>::value ? (T *)B.df : (T *)B.sf;
-    CKE(cudaMemsetAsync(P<T>::u(B, 0), 0, level_bytes(B, sizeof(T)), G->st));
     int cb = 0;
-    CKE(vcycle<T>(G, G->nl - 1, cb, o, base_rhs));
+    CKE(zero_start<T>(G, G->nl - 1, cb, o, base_rhs));
+    CKE(vcycle<T>(G, G->nl - 1, cb, o, base_rhs, cb));
     // coarsest level first (every parent's final correction before its children)
     for (int L = 1; L < (int)lev.size(); ++L)
         CKE(amr_branches(G, lev[L], [&](int a) -> cudaError_t {

@@ -112,6 +112,7 @@ struct SweepArgs {
     int psx = 0;
     long long psy = 0;
     bool foreign_psi = false;
+    int max_ctas = 0;            // persistent 3D sweeps without norm: at most this many CTAs (0: one per SM)
 };
 
 // First pre-smoothing sweep of a coarse level, from a zero correction: u = omega D^-1 f on
@@ -238,6 +239,13 @@ cudaError_t launch_gs2_sweep(const Geom &g, const Coef<T> &c, const T *psi, cons
 template <typename T>
 cudaError_t launch_restrict(const Geom &gf, const Geom &gc, const T *rf, T *fc, cudaStream_t s,
                             const int *gate = nullptr, T *zero_uc = nullptr, const FirstSweep<T> &first = FirstSweep<T>());
+
+// The sweep of FirstSweep on its own: on the view v that starts at storage node (off, ..) of
+// s (off = 0: the whole level), f and first.u in the storage's layout, first.psi at the
+// view's origin; first.u and zero (may be null) get 0 on the storage nodes off the view.
+template <typename T>
+cudaError_t launch_first_sweep(const Geom &st, const Geom &v, int off, const T *f, const FirstSweep<T> &first, T *zero,
+                               cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_prolong_add(const Geom &gf, const Geom &gc, const T *ec, T *uf, cudaStream_t s,
