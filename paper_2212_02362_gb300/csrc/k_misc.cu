@@ -31,17 +31,42 @@ __device__ __forceinline__ void node_of(const Geom &g, long long t, int &i, int 
 // Launch geometry of the node-wise kernels: a 3D grid of (32, 4, 2) blocks covers
 // (nx, ny, nz) directly, so no index decoding by division is needed.
 const dim3 kNodeBlock(32, 4, 2);
-inline dim3 node_grid(const Geom &g, const dim3 b = kNodeBlock)
+inline dim3 node_grid(const Geom &g)
 {
-    return dim3((g.nx + b.x - 1) / b.x, (g.ny + b.y - 1) / b.y, (g.nz + b.z - 1) / b.z);
+    return dim3((g.nx + 31) / 32, (g.ny + 3) / 4, (g.nz + 1) / 2);
 }
 
-// The 3D transfers: in FP64 some 120 instructions a node, whose issue on one SM is what a
-// block of eight warps costs on a small level (13 us); single warps spread over all SMs.
-template <typename T>
-inline dim3 transfer_block(const Geom &g)
+// The 3D transfers in FP64 cost some 100 FP64 instructions a node, each of which occupies a
+// sub-partition for 64 cycles whether 1 or 32 lanes take part: they number the nodes
+// linearly (no empty lanes at the ends of short rows) in blocks of two warps, which
+// spread small levels over all SMs.
+template <typename T, int D>
+constexpr bool kLinear = sizeof(T) == 8 && D == 3;
+
+template <typename T, int D>
+inline void transfer_shape(const Geom &g, dim3 &grid, dim3 &block)
 {
-    return sizeof(T) == 8 && g.dim == 3 ? dim3(32, 1, 1) : kNodeBlock;
+    if (kLinear<T, D>) {
+        grid = dim3((unsigned)(((long long)g.nx * g.ny * g.nz + 63) / 64));
+        block = dim3(64);
+    } else {
+        grid = node_grid(g);
+        block = kNodeBlock;
+    }
+}
+
+template <typename T, int D>
+__device__ __forceinline__ bool transfer_node(const Geom &g, int &i, int &j, int &k)
+{
+    if (kLinear<T, D>) {
+        const long long t = blockIdx.x * 64ll + threadIdx.x;
+        node_of(g, t, i, j, k);
+        return k < g.nz;
+    }
+    i = blockIdx.x * blockDim.x + threadIdx.x;
+    j = blockIdx.y * blockDim.y + threadIdx.y;
+    k = blockIdx.z * blockDim.z + threadIdx.z;
+    return i < g.nx && j < g.ny && k < g.nz;
 }
 
 // zero_uc (may be null): the coarse correction, zeroed at each coarse node (the start of
@@ -52,10 +77,8 @@ template <typename T, int D>
 __global__ void k_restrict(const Geom gf, const Geom gc, const T *__restrict__ rf, T *__restrict__ fc, const int *gate,
                            T *__restrict__ zero_uc, const FirstSweep<T> first)
 {
-    const int I = blockIdx.x * blockDim.x + threadIdx.x;
-    const int J = blockIdx.y * blockDim.y + threadIdx.y;
-    const int K = blockIdx.z * blockDim.z + threadIdx.z;
-    const bool in = I < gc.nx && J < gc.ny && K < gc.nz;
+    int I, J, K;
+    const bool in = transfer_node<T, D>(gc, I, J, K);
     T ip = T(0);
     if (first.u && in) ip = first.dinv ? first.dinv[gidx(gc, I, J, K)] : body::inv_psi_sum<T, D>(gc, first.psi, I, J, K);
     pdl_begin();
@@ -100,10 +123,8 @@ __global__ void k_prolong_add(const Geom gf, const Geom gc, const T *__restrict_
 {
     pdl_begin();
     if (gate && *gate) return;
-    const int I = blockIdx.x * blockDim.x + threadIdx.x;
-    const int J = blockIdx.y * blockDim.y + threadIdx.y;
-    const int K = blockIdx.z * blockDim.z + threadIdx.z;
-    if (I >= gc.nx || J >= gc.ny || K >= gc.nz) return;
+    int I, J, K;
+    if (!transfer_node<T, D>(gc, I, J, K)) return;
     body::prolong_node<T, D>(gf, gc, ec, uf, I, J, K);
 }
 
@@ -676,9 +697,11 @@ template <typename T>
 cudaError_t launch_restrict(const Geom &gf, const Geom &gc, const T *rf, T *fc, cudaStream_t s, const int *gate,
                             T *zero_uc, const FirstSweep<T> &first)
 {
-    cudaError_t e = gf.dim == 3
-                        ? launch_pdl(k_restrict<T, 3>, node_grid(gc, transfer_block<T>(gc)), transfer_block<T>(gc), 0, s, gf, gc, rf, fc, gate, zero_uc, first)
-                        : launch_pdl(k_restrict<T, 2>, node_grid(gc, transfer_block<T>(gc)), transfer_block<T>(gc), 0, s, gf, gc, rf, fc, gate, zero_uc, first);
+    dim3 gr, b;
+    if (gf.dim == 3) transfer_shape<T, 3>(gc, gr, b);
+    else transfer_shape<T, 2>(gc, gr, b);
+    cudaError_t e = gf.dim == 3 ? launch_pdl(k_restrict<T, 3>, gr, b, 0, s, gf, gc, rf, fc, gate, zero_uc, first)
+                                : launch_pdl(k_restrict<T, 2>, gr, b, 0, s, gf, gc, rf, fc, gate, zero_uc, first);
     if (e != cudaSuccess) return e;
     ++g_launches;
     return cudaGetLastError();
@@ -706,8 +729,11 @@ template cudaError_t launch_first_sweep<float>(const Geom &, const Geom &, int, 
 template <typename T>
 cudaError_t launch_prolong_add(const Geom &gf, const Geom &gc, const T *ec, T *uf, cudaStream_t s, const int *gate)
 {
-    cudaError_t e = gf.dim == 3 ? launch_pdl(k_prolong_add<T, 3>, node_grid(gc, transfer_block<T>(gc)), transfer_block<T>(gc), 0, s, gf, gc, ec, uf, gate)
-                                : launch_pdl(k_prolong_add<T, 2>, node_grid(gc, transfer_block<T>(gc)), transfer_block<T>(gc), 0, s, gf, gc, ec, uf, gate);
+    dim3 gr, b;
+    if (gf.dim == 3) transfer_shape<T, 3>(gc, gr, b);
+    else transfer_shape<T, 2>(gc, gr, b);
+    cudaError_t e = gf.dim == 3 ? launch_pdl(k_prolong_add<T, 3>, gr, b, 0, s, gf, gc, ec, uf, gate)
+                                : launch_pdl(k_prolong_add<T, 2>, gr, b, 0, s, gf, gc, ec, uf, gate);
     if (e != cudaSuccess) return e;
     ++g_launches;
     return cudaGetLastError();

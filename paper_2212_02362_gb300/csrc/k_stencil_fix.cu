@@ -307,9 +307,10 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
         const Tile T = make_tile(g, t, ntx, tx, ty);
         su += kend + 1 - kz0;
         const int kfirst = kz0 > 0 ? kz0 - 1 : 0;
-        auto cell_psi = [&](int lz) {
-            return (T.cell_ok && lz <= g.nz - 2) ? a.psi[pidx(a, T.gx - 1, T.gy - 1, lz)] : 0.0;
-        };
+        // the cell column's psi from here on (advanced a layer at a time)
+        const double *pp = a.psi + (T.cell_ok ? pidx(a, T.gx - 1, T.gy - 1, kfirst) : 0);
+        const long long psy = a.psx ? a.psy : g.sy;
+        auto cell_psi = [&](int lz) { return (T.cell_ok && lz <= g.nz - 2) ? *pp : 0.0; };
         const Stage S = make_stage(g, T);
         // planes kfirst, kfirst + 1 as integers, kfirst + 2 with its key, kfirst + 3 on its way
         for (int k = kfirst; k < kfirst + 3; ++k) load_plane(a.u, g, S, k, slot(k));
@@ -349,6 +350,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
             i64 *X = X2 + buf * 9 * PP;
             int *Xe = Xe2 + buf * PP;
             double *ps = ps2 + buf * PP;
+            pp += psy;
             const double psi_next = cell_psi(lz + 1);
             const bool fin = T.own && lz >= kz0;
             double fv[3], uv[3];
@@ -456,7 +458,7 @@ __global__ void __launch_bounds__(kNode64Threads) k_sweep3_node64(const SweepArg
     const long long on = valid ? gidx(g, i, j, k) : 0;
     const int p = c < 3 ? c : 0;                          // the component this lane finalises (lanes 0..2)
     // what no kernel of the cycle writes is read before the wait for the predecessor
-    const double psi = has ? a.psi[gidx(g, ci, cj, ck)] : 0.0;
+    const double psi = has ? a.psi[pidx(a, ci, cj, ck)] : 0.0;
     double ip = (MODE == kJacobi && a.dinv) ? a.dinv[on] : 0.0;
     pdl_begin();
     if (a.gate && *a.gate) return;

@@ -237,13 +237,17 @@ SweepArgs<T, T> sweep_args(sbm_grid G, int l, const T *u, const T *f, T *out, do
     return a;
 }
 
+// FP64 sweeps: small 3D levels (no norm wanted) by the per-node kernel, the rest tiled.
+cudaError_t launch_sweep64(int mode, const SweepArgs<double, double> &a, cudaStream_t s)
+{
+    if (a.g.dim == 3 && !a.part && nnodes(a.g) <= kNode64MaxNodes) return launch_sweep_node64(mode, a, s);
+    return launch_sweep<double, double>(mode, a, s);
+}
+
 template <typename T>
 cudaError_t sweep(sbm_grid G, int l, int mode, const T *u, const T *f, T *out, double *part, double omega)
 {
-    const SweepArgs<T, T> a = sweep_args<T>(G, l, u, f, out, part, omega);
-    if constexpr (std::is_same<T, double>::value)
-        if (a.g.dim == 3 && !part && nnodes(a.g) <= kNode64MaxNodes) return launch_sweep_node64(mode, a, G->st);
-    return launch_sweep<T, T>(mode, a, G->st);
+    return launch_sweep64(mode, sweep_args<T>(G, l, u, f, out, part, omega), G->st);   // FP32: specialised below
 }
 
 // FP32 3D sweeps: levels of at most kNodeKernelMaxNodes nodes (no norm wanted) use
@@ -1990,7 +1994,7 @@ static cudaError_t sweep_packed(sbm_grid G, int level, int mode, const double *u
     a.c = L.c64;
     a.wk[0] = a.wk[1] = a.wk[2] = 0.0;
     a.kchunk = 0;
-    return launch_sweep<double, double>(mode, a, G->st);
+    return launch_sweep64(mode, a, G->st);
 }
 
 static bool packed_apart(const Level &L, const double *a, const double *b)

@@ -184,27 +184,18 @@ __host__ __device__ __forceinline__ i64 down(i64 v, int s) { return v >> (s > 63
 
 // The 21 transformed values of a 3D cell that carry force (U[p][1..7] of bfly8), shifted up
 // to 2^61 at most.  Returns the shift (-3 at least); none: all are zero.
-__host__ __device__ __forceinline__ int normalize3(i64 (&U)[3][8], bool &none)
+// mh: the OR of their mag_hi.
+__host__ __device__ __forceinline__ int normalize3(i64 (&U)[3][8], unsigned mh, bool &none)
 {
-    unsigned mh = 0;
-#pragma unroll
-    for (int p = 0; p < 3; ++p)
-#pragma unroll
-        for (int s = 1; s < 8; ++s) mh |= mag_hi(U[p][s]);
     unsigned long long m = (unsigned long long)mh << 32 | 0xffffffffu;
-    none = false;
-    if (mh == 0u) {                          // all below 2^32: the low words decide
-        i64 any = 0;
+    if (mh == 0u) {                          // all below 2^32: the magnitudes themselves decide
         m = 0;
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
-            for (int s = 1; s < 8; ++s) {
-                any |= U[p][s];
-                m |= (unsigned long long)(U[p][s] ^ (U[p][s] >> 63));   // 0 for -1 as for 0
-            }
-        none = any == 0;
+            for (int s = 1; s < 8; ++s) m |= (unsigned long long)(U[p][s] < 0 ? -U[p][s] : U[p][s]);
     }
+    none = m == 0ull;
     const int sh = norm_shift(m);
     int up = sh;
     if (sh < 0) {                            // sums of opposite corners near the bound
@@ -258,15 +249,18 @@ __host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], cons
                                                      const Consts &c, i64 (&Fb)[3][4], i64 (&Ft)[3][4], int &e)
 {
     i64 U[3][8], dU[3][8];
+    unsigned mh = 0;
 #pragma unroll
     for (int p = 0; p < 3; ++p)
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
             U[p][s] = Tb[p][s] + Tt[p][s];
             U[p][s + 4] = Tt[p][s] - Tb[p][s];
+            if (s > 0) mh |= mag_hi(U[p][s]);
+            mh |= mag_hi(U[p][s + 4]);
         }
     bool none;
-    const int sh = normalize3(U, none);
+    const int sh = normalize3(U, mh, none);
     int ep;
     const i64 pm = psi_mantissa(psi, ep);
     e = (none || pm == 0) ? kNoExp : E - kFixUnit - sh + ep + c.ec;
@@ -306,7 +300,12 @@ __host__ __device__ __forceinline__ bool transform_cell3(const double (&v)[3][8]
         for (int a = 0; a < 8; ++a) U[p][a] = to_fix(v[p][a], E);
         bfly8(U[p]);
     }
-    e = E - kFixUnit - normalize3(U, none);
+    unsigned mh = 0;
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int s = 1; s < 8; ++s) mh |= mag_hi(U[p][s]);
+    e = E - kFixUnit - normalize3(U, mh, none);
     return true;
 }
 
