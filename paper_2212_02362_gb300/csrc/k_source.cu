@@ -70,7 +70,9 @@ __global__ void __launch_bounds__(kThr) k_cell_stress(const SourceArgs A, const 
 // Pass 2 (or the only pass without eigenstrain): one thread per node gathering its
 // 2^d cells: the eigenstrain load sum_c sum_q s_q sig_pq(c) / (2^(d-1) h) from the
 // cell stresses, psi_n, |grad psi|_n and the volume share for the body force and
-// the traction.
+// the traction.  The sums over the cells run on 64-bit integers (sbm_fix.cuh): with FP64
+// instructions their issue bound the kernel.  All three terms at 129^3: 0.66 -> 0.33 ms, the
+// node's own FP64 instructions (|grad psi|, the products with b and t) being most of it.
 template <int D>
 __global__ void __launch_bounds__(kThr) k_source_terms(const SourceArgs A, const double *__restrict__ psi,
                                                        const double *__restrict__ sig, const double *__restrict__ b,

@@ -442,8 +442,8 @@ long long sweep_blocks(const Geom &g, bool fp64)
 // its full weighting and the coarse level's first sweep: a block takes one coarse node,
 // 27 groups of eight threads its fine nodes' residuals (3.4x the arithmetic of the
 // residual alone, which on these levels is nothing beside a launch), a warp the weighted
-// sum.  Measured on one V-cycle of the 129^3 hierarchy with the first sweeps in the
-// restriction: see launch_restrict.
+// sum.  On the 129^3 hierarchy it takes 5.6 us from 17^3 to 9^3 and 4.3 us from 9^3 to
+// 5^3, where a sweep alone takes 4.1 us and a restriction alone 5.
 constexpr int kNodeThreads = 256;
 
 // Forces and psi of a node summed over its group of eight lanes; own: the node's values

@@ -13,7 +13,7 @@
 // One thread per cell: eta and its 2d face neighbours, u at the 2^d corner nodes
 // (d components, packed), the cell's strain energy, and the update.  In 3D the energy is
 // formed in integers (sbm_fix.cuh): in FP64 the kernel is bound by FP64 issue, and the
-// energy was four fifths of it.  The kernel also writes the next
+// energy was four fifths of it (524k cells: 246 -> 68 us).  The kernel also writes the next
 // stiffness (eta' + zeta)^2 and per-block partial sums of eta' (the next volume)
 // and of psi_c e_c (the compliance u^T K u h^d of the solve that produced u), each
 // summed in a fixed order so that results do not depend on scheduling.  FP64.
