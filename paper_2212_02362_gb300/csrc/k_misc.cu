@@ -39,16 +39,18 @@ inline dim3 node_grid(const Geom &g)
 // The 3D transfers in FP64 cost some 100 FP64 instructions a node, each of which occupies a
 // sub-partition for 64 cycles whether 1 or 32 lanes take part: they number the nodes
 // linearly (no empty lanes at the ends of short rows) in blocks of two warps, which
-// spread small levels over all SMs.
+// spread small levels over all SMs (65^3 FP64 solve 10.1 -> 9.4 ms).  In
+// FP32 the decoding costs more than the lanes save (129^3 solve 12.39 -> 12.53 ms).
 template <typename T, int D>
 constexpr bool kLinear = sizeof(T) == 8 && D == 3;
+constexpr int kTransferThreads = 64;
 
 template <typename T, int D>
 inline void transfer_shape(const Geom &g, dim3 &grid, dim3 &block)
 {
     if (kLinear<T, D>) {
-        grid = dim3((unsigned)(((long long)g.nx * g.ny * g.nz + 63) / 64));
-        block = dim3(64);
+        grid = dim3((unsigned)nblk((long long)g.nx * g.ny * g.nz, kTransferThreads));
+        block = dim3(kTransferThreads);
     } else {
         grid = node_grid(g);
         block = kNodeBlock;
@@ -59,8 +61,15 @@ template <typename T, int D>
 __device__ __forceinline__ bool transfer_node(const Geom &g, int &i, int &j, int &k)
 {
     if (kLinear<T, D>) {
-        const long long t = blockIdx.x * 64ll + threadIdx.x;
-        node_of(g, t, i, j, k);
+        const long long t = (long long)blockIdx.x * kTransferThreads + threadIdx.x;
+        if (t >> 32) {
+            node_of(g, t, i, j, k);
+        } else {
+            const unsigned r = (unsigned)t / g.nx, z = r / g.ny;
+            i = (unsigned)t - r * g.nx;
+            j = r - z * g.ny;
+            k = z;
+        }
         return k < g.nz;
     }
     i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -638,7 +647,7 @@ __global__ void k_bottom_apply(int n, const T *__restrict__ Ainv, const int *__r
 // density != 0: dJ/drho = dJ/dpsi (1 - psi_min) q rho^(q-1);  density == 0 and
 // grho != null: dJ/dpsi_raw = dJ/dpsi where psi_raw > psi_min, else 0.  The 3D product is
 // formed in integers (sbm_fix.cuh): in FP64 its 220 instructions a cell took 1.58 ms on
-// 4.2 M cells, bound by their issue.
+// 4.2 M cells, bound by their issue; 0.60 ms in integers.
 __global__ void k_dJdpsi(const Geom g, const Coef<double> c, const fix::Consts fc, const double *__restrict__ u,
                          const double *__restrict__ lam, double *__restrict__ gout, double *__restrict__ grho,
                          const double *__restrict__ rho, const double *__restrict__ praw, double psi_min,
