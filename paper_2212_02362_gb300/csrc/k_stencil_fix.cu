@@ -316,6 +316,9 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
         const long long psy = a.psx ? a.psy : g.sy;
         auto cell_psi = [&](int lz) { return (T.cell_ok && lz <= g.nz - 2) ? *pp : 0.0; };
         const Stage S = make_stage(g, T);
+        // the last step of a segment leaves a copy (plane kend + 4) in flight; copies are not
+        // ordered among each other, so it has to land before its slot is loaded again
+        cp_async_wait_all();
         // planes kfirst, kfirst + 1 as integers, kfirst + 2 with its key, kfirst + 3 on its way
         for (int k = kfirst; k < kfirst + 3; ++k) load_plane(a.u, g, S, k, slot(k));
         if (tid < 4) keys[tid] = 0u;

@@ -184,3 +184,18 @@ def test_decaying_field(dim, n):
         if dim == 2:
             ref = oracle.gs_sweep(P, psi, wk.f, u)
             assert _rel(host(g.smooth(g.finest, cuda(wk.f), cuda(u), "gs")) - u, ref - u) <= 1e-11
+
+
+@pytest.mark.parametrize("n", [(321, 101, 5), (257, 91, 6), (193, 121, 7), (161, 111, 3)])
+def test_blocks_of_several_tiles(n):
+    """Shallow grids with more tiles than SMs: a block goes from the top of one tile to the
+    bottom of the next, whose planes go into ring slots that the last step's copy (a plane
+    above the grid: zeros) was issued for."""
+    wk = random_workload(3, n, 140)
+    g, P = gpu_grid(wk), oracle_problem(wk)
+    u = W.uniform(141, P.ndofs, -1, 1)
+    psi = oracle.floor_psi(wk.psi, wk.psi_min)
+    ref = oracle.residual(P, psi, wk.f, u)
+    for _ in range(5):
+        r, nrm = g.residual(g.finest, cuda(wk.f), cuda(u))
+        assert _rel(host(r), ref) <= 1e-13 and np.isclose(nrm, oracle.norm_free(P, ref), rtol=1e-13)
