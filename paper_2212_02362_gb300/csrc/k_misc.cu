@@ -997,7 +997,7 @@ cudaError_t launch_dJdpsi(const Geom &g, const Coef<double> &c, const double *u,
                           double *grho_out, const double *rho, const double *psi_raw, double psi_min, double q,
                           int density, cudaStream_t s)
 {
-    k_dJdpsi<<<nblk(ncells(g), 128), 128, 0, s>>>(g, c, fix::make_consts(g.dim, c), u, lam, g_out, grho_out, rho, psi_raw, psi_min, q, density);
+    k_dJdpsi<<<nblk(ncells(g), 128), 128, 0, s>>>(g, c, fix::level_consts(g.dim, c), u, lam, g_out, grho_out, rho, psi_raw, psi_min, q, density);
     ++g_launches;
     return cudaGetLastError();
 }

@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
             buf ^= 1;
             if (fin) {
                 const int e1 = Xe[me + 1], e2 = Xe[me + PX], e3 = Xe[me + PX + 1];
-                const int ee = max(max(en, e1), max(e2, e3));
+                const int ee = max(max(en, e1), max(e2, e3)) + fix::kNodeBits3;
                 const int d0 = ee - en, d1 = ee - e1, d2 = ee - e2, d3 = ee - e3;
                 double Ku[3];
 #pragma unroll
@@ -489,6 +489,7 @@ __global__ void __launch_bounds__(kNode64Threads) k_sweep3_node64(const SweepArg
         int ee = e;
 #pragma unroll
         for (int off = 4; off > 0; off >>= 1) ee = max(ee, __shfl_xor_sync(0xffffffffu, ee, off));
+        ee += fix::kNodeBits3;
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             F[q] = fix::down(F[q], ee - e);
@@ -641,7 +642,7 @@ __global__ void __launch_bounds__((TX2 + 1) * (TY2 + 1))
     if (all) {
         if (own) {
             const int e1 = Xe[me + 1], e2 = Xe[me + PX2], e3 = Xe[me + PX2 + 1];
-            const int ee = max(max(e, e1), max(e2, e3));
+            const int ee = max(max(e, e1), max(e2, e3)) + fix::kNodeBits2;
 #pragma unroll
             for (int p = 0; p < 2; ++p)
                 Ku[p] = fix::to_double((fix::down(F[p][3], ee - e) + fix::down(X[p][2][me + 1], ee - e1)) +
@@ -748,7 +749,7 @@ __global__ void __launch_bounds__(kRrThreads) k_resid_restrict2(const SweepArgs<
         for (int p = 0; p < 2; ++p) {
             double Ku;
             if (all) {
-                const int ee = max(max(Xe[c0], Xe[c1]), max(Xe[c2], Xe[c3]));
+                const int ee = max(max(Xe[c0], Xe[c1]), max(Xe[c2], Xe[c3])) + fix::kNodeBits2;
                 Ku = fix::to_double((fix::down(X[p][3][c3], ee - Xe[c3]) + fix::down(X[p][2][c2], ee - Xe[c2])) +
                                         (fix::down(X[p][1][c1], ee - Xe[c1]) + fix::down(X[p][0][c0], ee - Xe[c0])),
                                     ee);
@@ -959,7 +960,7 @@ __global__ void k_inv_psi(const Geom g, const double *__restrict__ psi, double *
 template <typename TO, int MODE>
 cudaError_t launch_fix_mode(const SweepArgs<double, TO> &a, cudaStream_t s)
 {
-    const fix::Consts fc = fix::make_consts(a.g.dim, a.c);
+    const fix::Consts fc = fix::level_consts(a.g.dim, a.c);
     cudaError_t e;
     if (a.g.dim == 3) {
         static std::atomic<unsigned long long> attr_done{0};
@@ -997,7 +998,7 @@ cudaError_t launch_sweep_node64(int mode, const SweepArgs<double, double> &a, cu
     if (a.g.dim != 3 || (long long)a.g.nx * a.g.ny * a.g.nz >= (1 << 24)) return cudaErrorInvalidValue;
     const int n = a.g.nx * a.g.ny * a.g.nz;
     const dim3 gr((n + kNode64Threads / 8 - 1) / (kNode64Threads / 8)), b(kNode64Threads);
-    const fix::Consts fc = fix::make_consts(3, a.c);
+    const fix::Consts fc = fix::level_consts(3, a.c);
     cudaError_t e;
     switch (mode) {
     case kApply: e = launch_pdl(k_sweep3_node64<kApply>, gr, b, 0, s, a, fc); break;
@@ -1013,7 +1014,7 @@ cudaError_t launch_sweep_node64(int mode, const SweepArgs<double, double> &a, cu
 cudaError_t launch_prolong_sweep(const SweepArgs<double, double> &a, const Geom &gc, const double *ec, cudaStream_t s)
 {
     if (a.g.dim != 2 || a.u == a.out) return cudaErrorInvalidValue;
-    const fix::Consts fc = fix::make_consts(2, a.c);
+    const fix::Consts fc = fix::level_consts(2, a.c);
     const int ty = rows2(a.g);
     const dim3 gr((a.g.nx + 30) / 32, (a.g.ny - 2 + ty) / ty), b(33 * (ty + 1));
     cudaError_t e = ty == 8 ? launch_pdl(k_sweep2_fix<double, kJacobi, 8, true>, gr, b, 0, s, a, fc, gc, ec)
@@ -1028,7 +1029,7 @@ cudaError_t launch_resid_restrict(const SweepArgs<double, double> &a, const Geom
 {
     if (a.g.dim != 2) return cudaErrorInvalidValue;
     const dim3 gr((gc.nx + CT - 1) / CT, (gc.ny + CT - 1) / CT);
-    cudaError_t e = launch_pdl(k_resid_restrict2, gr, dim3(kRrThreads), 0, s, a, fix::make_consts(2, a.c), gc, fc, first);
+    cudaError_t e = launch_pdl(k_resid_restrict2, gr, dim3(kRrThreads), 0, s, a, fix::level_consts(2, a.c), gc, fc, first);
     if (e != cudaSuccess) return e;
     ++g_launches;
     return cudaGetLastError();
@@ -1045,7 +1046,7 @@ cudaError_t launch_inv_psi(const Geom &g, const double *psi, double *dinv, cudaS
 cudaError_t launch_gs2_fix(const Geom &g, const Coef<double> &c, const double *psi, const double *Ke, const double *f,
                            const double *uin, double *uout, int descending, cudaStream_t s, const int *gate)
 {
-    const fix::Consts fc = fix::make_consts(2, c);
+    const fix::Consts fc = fix::level_consts(2, c);
     const long long b32 = ((g.nx + 31) / 32) * (long long)((g.ny + 31) / 32);
     if (b32 >= 304) return launch_gs2_tile<32>(g, fc, psi, Ke, f, uin, uout, descending, s, gate);
     return launch_gs2_tile<16>(g, fc, psi, Ke, f, uin, uout, descending, s, gate);

@@ -152,9 +152,9 @@ cudaError_t launch_topopt_step(int dim, const TopoptArgs &A, const Coef<double> 
     if (NN * dim >= (1ll << 31)) return cudaErrorInvalidValue;               // 32-bit indexing
     const dim3 grid((unsigned)topopt_blocks(NC));
     if (dim == 3)
-        k_topopt_step<3><<<grid, kThr, 0, s>>>(A, c, fix::make_consts(dim, c), eta, u, psi_solve, eta_sum, eta_out, psi_next, part);
+        k_topopt_step<3><<<grid, kThr, 0, s>>>(A, c, fix::level_consts(dim, c), eta, u, psi_solve, eta_sum, eta_out, psi_next, part);
     else
-        k_topopt_step<2><<<grid, kThr, 0, s>>>(A, c, fix::make_consts(dim, c), eta, u, psi_solve, eta_sum, eta_out, psi_next, part);
+        k_topopt_step<2><<<grid, kThr, 0, s>>>(A, c, fix::level_consts(dim, c), eta, u, psi_solve, eta_sum, eta_out, psi_next, part);
     ++g_launches;
     return cudaGetLastError();
 }
