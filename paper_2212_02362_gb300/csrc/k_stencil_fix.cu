@@ -10,25 +10,29 @@
 // Work split.  A block owns a tile of 32 x 10 cells in x/y (33 x 11 threads, one per cell
 // column with the halo column and row; 12 warps, so 168 registers a thread) and a
 // contiguous range of (tile, node plane) units, which it streams along z, one cell layer
-// a step.  Node planes pass through a four-slot shared-memory ring in four stages, so
-// that nothing inside a step waits for global memory and one barrier a step suffices.  In
-// step lz
+// a step.  Node planes pass through a four-slot shared-memory ring, so that nothing
+// inside a step waits for global memory and one barrier a step suffices.  In step lz
 //   plane lz+4  is copied by cp.async (into the slot that plane lz left in step lz - 1)
-//   plane lz+3  has arrived: each thread takes the largest exponent of the values it
-//               copied into the plane's key
-//   plane lz+2  is turned into integers in place, each thread the values it copied
-//   plane lz+1  is read by the cells of layer lz
+//   plane lz+3  has arrived: each thread takes the largest exponent of each node it copied
+//   plane lz+1  is read by the cells of layer lz, each turning its face's values into
+//               integers on a unit of its own (the exponents of its four nodes), kept
+//               for the layer above; where a cell's two faces differ, both are shifted to
+//               the larger of their units
 // The forces a layer sends to its top plane are carried in registers in the transformed
 // basis with their exponent; those of the four columns around a node are exchanged
 // through a double-buffered shared array with the exponents beside them.
 //
-// A plane or a psi that the integer form does not take (sbm_fix.cuh) ends the integer
+// A cell or a psi that the integer form does not take (sbm_fix.cuh) ends the integer
 // loop before any node that depends on it; the block finishes its range with the FP64
 // body below, which also runs when the level's constants do not fit.
 //
+// A unit per staged plane and tile instead (values converted once, in place, instead of by
+// the four cells around a column) took 200 us for the 129^3 residual, but lost the digits
+// of cells far below the tile's largest value.
+//
 // Measured (kernel time, FP64 instructions -> this form): residual with norm at 129^3
-// 812 -> 187 us (0.8 TB/s), Jacobi sweep at 65^3 155 -> 34 us, at 33^3 46 -> 12 us; the ALU
-// pipe about 55% busy with one block of 12 warps per SM (registers).
+// 812 -> 212 us (0.76 TB/s), Jacobi sweep at 65^3 155 -> 40 us, at 33^3 46 -> 12.5 us; issue
+// and latency of one block of 12 warps per SM (registers).
 #include <algorithm>
 
 #include "sbm_common.cuh"
@@ -45,8 +49,8 @@ constexpr int TX = 32, TY = 10;                   // cells of a tile
 constexpr int BX = TX + 1, BY = TY + 1, NT = BX * BY;
 constexpr int PX = TX + 2, PY = TY + 2, PP = PX * PY;
 // ring of node planes (4 x 3 components); two buffers of 9 exchanged forces, psi of the
-// cells below + above and the exponent (the FP64 body: 12 forces and psi)
-constexpr size_t kSmem = sizeof(double) * (12 + 2 * (9 + 1)) * PP + 2 * sizeof(int) * PP;
+// cells below + above and the exponent (the FP64 body: 12 forces and psi); the ring's node keys
+constexpr size_t kSmem = sizeof(double) * (12 + 2 * (9 + 1)) * PP + (2 + 4) * sizeof(int) * PP;
 
 // 8-byte global -> shared copy; ok = false fills zeros (src must still be valid).
 __device__ __forceinline__ void cp_async8(void *sdst, const void *gsrc, bool ok)
@@ -240,12 +244,12 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
     pdl_begin();
     if (a.gate && *a.gate) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *up = reinterpret_cast<double *>(smem_raw);        // [4][3][PP]: doubles, then integers
+    double *up = reinterpret_cast<double *>(smem_raw);        // [4][3][PP] ring of node planes
     i64 *X2 = reinterpret_cast<i64 *>(up + 12 * PP);           // [2][9][PP]: corner forces 0..2 of a plane
     double *ps2 = up + 30 * PP;                                // [2][PP]
     int *Xe2 = reinterpret_cast<int *>(ps2 + 2 * PP);          // [2][PP]: exponents of the forces
+    unsigned *node_keys = reinterpret_cast<unsigned *>(Xe2 + 2 * PP);   // [4][PP]: of the ring's nodes
     __shared__ double red[((NT + 31) / 32) * 32];
-    __shared__ unsigned keys[4];
 
     const Geom &g = a.g;
     const int tid = threadIdx.x;
@@ -268,38 +272,30 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
     long long rest = fc.ok ? ue : ub;          // units from here on are left to the FP64 body
 
     auto slot = [&](int k) { return up + (k & 3) * 3 * PP; };
-    // the largest exponent key of the values this thread copied, into the plane's key
+    // the largest exponent key of each node this thread copied
     auto take_key = [&](int k) {
         const double *pl = slot(k);
-        unsigned m = 0;
-#pragma unroll
-        for (int p = 0; p < 3; ++p) m = max(m, fix::exp_key(pl[p * PP + tid]));
-        if (tid + NT < PP)
-#pragma unroll
-            for (int p = 0; p < 3; ++p) m = max(m, fix::exp_key(pl[p * PP + tid + NT]));
-        const unsigned w = (tid | 31) < NT ? 0xffffffffu : (1u << (NT & 31)) - 1u;   // the last warp is partial
-        m = __reduce_max_sync(w, m);
-        if ((tid & 31) == 0) atomicMax(&keys[k & 3], m);
+        unsigned *nk = node_keys + (k & 3) * PP;
+        auto node = [&](int s) {
+            nk[s] = max(max(fix::exp_key(pl[s]), fix::exp_key(pl[PP + s])), fix::exp_key(pl[2 * PP + s]));
+        };
+        node(tid);
+        if (tid + NT < PP) node(tid + NT);
     };
-    auto exp_of = [&](int k) { return max((int)(keys[k & 3] >> 20), fix::kExpLo); };
-    auto to_ints = [&](int k) {
-        double *pl = slot(k);
-        const int E = exp_of(k);
-#pragma unroll
-        for (int p = 0; p < 3; ++p) pl[p * PP + tid] = fix::of_bits(fix::to_fix(pl[p * PP + tid], E));
-        if (tid + NT < PP)
-#pragma unroll
-            for (int p = 0; p < 3; ++p)
-                pl[p * PP + tid + NT] = fix::of_bits(fix::to_fix(pl[p * PP + tid + NT], E));
+    // and of the four nodes of this thread's face
+    auto face_key = [&](int k) {
+        const unsigned *nk = node_keys + (k & 3) * PP;
+        return max(max(nk[me], nk[me + 1]), max(nk[me + PX], nk[me + PX + 1]));
     };
-    auto corners = [&](int k, i64 (&C)[3][4]) {
-        const i64 *pl = reinterpret_cast<const i64 *>(slot(k));
+    // the face's values as integers on E, transformed
+    auto corners = [&](int k, int E, i64 (&C)[3][4]) {
+        const double *pl = slot(k);
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
-            C[p][0] = pl[p * PP + me];
-            C[p][1] = pl[p * PP + me + 1];
-            C[p][2] = pl[p * PP + me + PX];
-            C[p][3] = pl[p * PP + me + PX + 1];
+            C[p][0] = fix::to_fix(pl[p * PP + me], E);
+            C[p][1] = fix::to_fix(pl[p * PP + me + 1], E);
+            C[p][2] = fix::to_fix(pl[p * PP + me + PX], E);
+            C[p][3] = fix::to_fix(pl[p * PP + me + PX + 1], E);
             bfly4xy(C[p]);
         }
     };
@@ -319,26 +315,21 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
         // the last step of a segment leaves a copy (plane kend + 4) in flight; copies are not
         // ordered among each other, so it has to land before its slot is loaded again
         cp_async_wait_all();
-        // planes kfirst, kfirst + 1 as integers, kfirst + 2 with its key, kfirst + 3 on its way
+        // planes kfirst to kfirst + 2 with their keys, kfirst + 3 on its way
         for (int k = kfirst; k < kfirst + 3; ++k) load_plane(a.u, g, S, k, slot(k));
-        if (tid < 4) keys[tid] = 0u;
         double psi = cell_psi(kfirst), psi_prev = 0.0;
         cp_async_wait_all();
         __syncthreads();
         load_plane(a.u, g, S, kfirst + 3, slot(kfirst + 3));
         for (int k = kfirst; k < kfirst + 3; ++k) take_key(k);
-        bool bad = __syncthreads_or(!fix::psi_ok(psi));
-        for (int k = kfirst; k < kfirst + 3; ++k) bad = bad || !fix::key_ok(keys[k & 3]);
-        if (bad) {
+        if (__syncthreads_or(!fix::psi_ok(psi))) {
             rest = seg + kz0;
             break;
         }
-        to_ints(kfirst);
-        to_ints(kfirst + 1);
-        __syncthreads();
         i64 Tb[3][4], Cf[3][4];
-        int Eb = exp_of(kfirst), ecf = fix::kNoExp;
-        corners(kfirst, Tb);
+        unsigned kb = face_key(kfirst);                        // the bottom face: its key, its unit
+        int Eb = fix::face_exp(kb), ecf = fix::kNoExp;
+        corners(kfirst, Eb, Tb);
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
@@ -346,14 +337,9 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
         __syncthreads();                                       // plane kfirst's slot is free
 #pragma unroll 1
         for (int lz = kfirst; lz <= kend; ++lz) {
-            if (!fix::key_ok(keys[(lz + 2) & 3])) {            // the same for the whole block
-                rest = seg + max(lz, kz0);
-                break;
-            }
             cp_async_wait_all();                               // plane lz + 3 in this thread's copies
             take_key(lz + 3);
             load_plane(a.u, g, S, lz + 4, slot(lz + 4));
-            if (tid == 0) keys[lz & 3] = 0u;                   // for plane lz + 4
             i64 *X = X2 + buf * 9 * PP;
             int *Xe = Xe2 + buf * PP;
             double *ps = ps2 + buf * PP;
@@ -368,31 +354,19 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
                 uv[p] = (MODE == kJacobi && fin) ? a.u[p * g.cs + on] : 0.0;
             }
             double ip = (MODE == kJacobi && a.dinv && fin) ? a.dinv[on] : 0.0;
-            to_ints(lz + 2);
-            // the cell of layer lz, both faces on the larger of their planes' units
-            const int Et = exp_of(lz + 1);
-            const int E = max(Eb, Et);
+            // the cell of layer lz
+            const unsigned kt = face_key(lz + 1);
+            const bool fits = fix::key_ok(max(kb, kt));
+            const int Et = fix::face_exp(kt);
             i64 Tt[3][4], Fb[3][4], Ft[3][4];
-            corners(lz + 1, Tt);
-            if (Eb != Et) {
-#pragma unroll
-                for (int p = 0; p < 3; ++p)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        Tb[p][q] = fix::down(Tb[p][q], E - Eb);
-                        Tt[p][q] = fix::down(Tt[p][q], E - Et);
-                    }
-            }
+            corners(lz + 1, Et, Tt);
             int e;
-            fix::cell_faces3(Tb, Tt, E, psi, fc, Fb, Ft, e);
-            if (E != Et) {
-                corners(lz + 1, Tb);
-            } else {
+            fix::cell_faces3(Tb, Eb, Tt, Et, psi, fc, Fb, Ft, e);
 #pragma unroll
-                for (int p = 0; p < 3; ++p)
+            for (int p = 0; p < 3; ++p)
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) Tb[p][q] = Tt[p][q];
-            }
+                for (int q = 0; q < 4; ++q) Tb[p][q] = Tt[p][q];
+            kb = kt;
             Eb = Et;
             // plane lz: top face of layer lz - 1 + bottom face of layer lz
             const int en = max(e, ecf), s0 = en - ecf, s1 = en - e;
@@ -413,7 +387,10 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
             if (MODE == kJacobi && !a.dinv) ps[me] = psi_prev + psi;
             psi_prev = psi;
             psi = psi_next;
-            const int bad_next = __syncthreads_or(!fix::psi_ok(psi));
+            if (__syncthreads_or(!fits || (!fix::psi_ok(psi) && lz < kend))) {
+                rest = seg + max(lz, kz0);                     // this plane's cells, or the next psi
+                break;
+            }
             buf ^= 1;
             if (fin) {
                 const int e1 = Xe[me + 1], e2 = Xe[me + PX], e3 = Xe[me + PX + 1];
@@ -430,10 +407,6 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
                 if (MODE == kJacobi && !a.dinv)
                     ip = 1.0 / ((ps[me] + ps[me + 1]) + (ps[me + PX] + ps[me + PX + 1]));
                 body::finalize_f<double, TO, MODE>(a, T.gx, T.gy, lz, Ku, ip, uv, fv, ssq);
-            }
-            if (bad_next && lz < kend) {
-                rest = seg + max(lz + 1, kz0);
-                break;
             }
         }
     }

@@ -6,8 +6,8 @@
 // per value and one power of two per cell.
 //
 //   1. The nodal values around a cell become integers |u| < 2^60 on a common power of
-//      two, the largest one in the staged node plane: a double keeps all of its 53 bits
-//      down to 2^-7 of that largest value.
+//      two, which follows the largest of the cell's own values: a double keeps all of its
+//      53 bits down to 2^-7 (in the tiled 3D sweep 2^-6, see face_exp) of that value.
 //   2. The mean/difference transform is exact (additions of integers).
 //   3. The cell's 21 transformed values are shifted left until the largest reaches
 //      2^60, so the products below keep the cell's own leading digits, however small
@@ -25,8 +25,8 @@
 // cells each, rms of a cell's largest corner error over its largest |K||u| (the formula in
 // FP64 with FMAs in brackets), moduli (1, 0.6, 0.5): random values 3.5e-17 (8.5e-17),
 // hourglass patterns 2.3e-17 (4.6e-17), components decades apart 4.3e-17 (1.0e-16),
-// smooth displacements 1.2e-18 (4.1e-17).  Step 1 adds 2^-60 of the unit's value for every
-// nodal value that has more digits than fit.  Values that do not fit the scheme
+// smooth displacements 1.2e-18 (4.1e-17).  Step 1 truncates values below 2^-7 of the largest.
+// Values that do not fit the scheme
 // (infinities, NaN, exponents beyond the range below, negative psi) are recognised while
 // they are staged, and the caller evaluates those planes with FP64 instructions.
 #pragma once
@@ -69,6 +69,17 @@ __host__ __device__ __forceinline__ bool key_ok(unsigned key)
     return key == 0u || (key >= ((unsigned)kExpLo << 20) && key < ((unsigned)kExpHi << 20));
 }
 
+// The exponent that a face's values are staged on, from the key of the largest: rounded up to
+// an odd one, so that the two faces of a cell mostly share it (a 129^3 residual of values all
+// of one size 236 us, as with steps of four; 249 us without).  The values then keep 59 or 60
+// bits of the largest: the residual of a solved displacement (45 x 37 x 41) is 5.0e-17 off against
+// long double, 4.3e-17 of that the rounding of the result; 1.1e-16 with steps of four.
+__host__ __device__ __forceinline__ int face_exp(unsigned key)
+{
+    const int e = (int)(key >> 20);
+    return (e > kExpLo ? e : kExpLo) | 1;
+}
+
 // v as an integer on the unit 2^(E - 1023 - 52 - UP), E >= the biased exponent of v: below
 // 2^(53 + UP).  UP = 7 unless sums of more than eight values follow.
 template <int UP = 7>
@@ -77,8 +88,8 @@ __host__ __device__ __forceinline__ i64 to_fix(double v, int E)
     const i64 b = bits_of(v);
     const int ex = (int)((unsigned)(b >> 52) & 0x7ffu);
     const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
-    const int sh = E - ex;
-    const i64 a = sh > 63 ? 0 : (i64)((m << UP) >> sh);
+    const unsigned sh = (unsigned)(E - ex);
+    const i64 a = (i64)((m << UP) >> (sh < 63u ? sh : 63u));
     return b < 0 ? -a : a;
 }
 constexpr int kFixUnit = 1023 + 59;     // to_fix<7>'s unit is 2^(E - kFixUnit)
@@ -283,19 +294,36 @@ __host__ __device__ __forceinline__ void stress3(const i64 (&U)[3][8], const Fra
 }
 
 // One 3D cell: in-plane transforms (bfly4xy of the integers) of its bottom and top faces
-// on the unit 2^(E - kFixUnit), its psi.  Returns the transformed face forces, the
-// unit of which is 2^e (e = kNoExp: no force, Fb = Ft = 0).
-__host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], const i64 (&Tt)[3][4], int E, double psi,
-                                                     const Consts &c, i64 (&Fb)[3][4], i64 (&Ft)[3][4], int &e)
+// on the units 2^(Eb - kFixUnit) and 2^(Et - kFixUnit), its psi.  Returns the transformed
+// face forces, the unit of which is 2^e (e = kNoExp: no force, Fb = Ft = 0).
+__host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], int Eb, const i64 (&Tt)[3][4], int Et,
+                                                     double psi, const Consts &c, i64 (&Fb)[3][4], i64 (&Ft)[3][4], int &e)
 {
     i64 U[3][8], dU[3][8];
+    const int E = Eb > Et ? Eb : Et;
+    if (Eb == Et) {
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                U[p][s] = Tb[p][s] + Tt[p][s];
+                U[p][s + 4] = Tt[p][s] - Tb[p][s];
+            }
+    } else {
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const i64 b = down(Tb[p][s], E - Eb), t = down(Tt[p][s], E - Et);
+                U[p][s] = b + t;
+                U[p][s + 4] = t - b;
+            }
+    }
     unsigned mh = 0;
 #pragma unroll
     for (int p = 0; p < 3; ++p)
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-            U[p][s] = Tb[p][s] + Tt[p][s];
-            U[p][s + 4] = Tt[p][s] - Tb[p][s];
             if (s > 0) mh |= mag_hi(U[p][s]);
             mh |= mag_hi(U[p][s + 4]);
         }
@@ -317,6 +345,12 @@ __host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], cons
             Ft[p][s] = dU[p][s] + dU[p][s + 4];
         }
     }
+}
+
+__host__ __device__ __forceinline__ void cell_faces3(const i64 (&Tb)[3][4], const i64 (&Tt)[3][4], int E, double psi,
+                                                     const Consts &c, i64 (&Fb)[3][4], i64 (&Ft)[3][4], int &e)
+{
+    cell_faces3(Tb, E, Tt, E, psi, c, Fb, Ft, e);
 }
 
 // Nodal values of a 3D cell as transformed, normalised integers: v = U 2^(e), e returned.

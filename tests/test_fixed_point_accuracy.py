@@ -118,6 +118,40 @@ extern "C" void errors2(const double *m, const double *uu, double psi, double *e
     }
 }
 
+// The 3D forces by faces, each on its own unit as the tiled sweep stages it
+extern "C" void errors_staged(const double *m, const double *uu, double psi, double *err)
+{
+    const Coef<double> c = coef(3, m);
+    double u[3][8];
+    Q q[3][8];
+    memcpy(u, uu, sizeof(u));
+    for (int i = 0; i < 24; ++i) q[i / 8][i % 8] = u[i / 8][i % 8];
+    cell_forces3<Q>(q, (Q)psi, wide(c));
+    fix::i64 T[2][3][4], Fb[3][4], Ft[3][4];
+    int E[2], e;
+    for (int z = 0; z < 2; ++z) {
+        unsigned key = 0;
+        for (int i = 0; i < 12; ++i) {
+            const unsigned k = fix::exp_key(u[i / 4][4 * z + i % 4]);
+            key = k > key ? k : key;
+        }
+        E[z] = fix::face_exp(key);
+        for (int p = 0; p < 3; ++p) {
+            for (int k = 0; k < 4; ++k) T[z][p][k] = fix::to_fix(u[p][4 * z + k], E[z]);
+            bfly4xy(T[z][p]);
+        }
+    }
+    fix::cell_faces3(T[0], E[0], T[1], E[1], psi, fix::make_consts(3, c), Fb, Ft, e);
+    for (int p = 0; p < 3; ++p) {
+        bfly4xyT(Fb[p]);
+        bfly4xyT(Ft[p]);
+        for (int a = 0; a < 4; ++a) {
+            err[p * 8 + a] = (double)fabsl(fix::to_double(Fb[p][a], e) - q[p][a]);
+            err[p * 8 + a + 4] = (double)fabsl(fix::to_double(Ft[p][a], e) - q[p][a + 4]);
+        }
+    }
+}
+
 // v^T S u: the errors of the integer form and of FP64, and |v|^T |S| |u|
 extern "C" void errors_work(const double *m, const double *uu, const double *vv, double *err)
 {
@@ -211,6 +245,28 @@ def test_forces_are_no_further_off_than_in_fp64(lib, dim, mod, kind):
     for e in (whole, own):
         rms = np.sqrt((e ** 2).mean(axis=1))
         assert rms[0] <= rms[2] and rms[1] <= rms[2], rms
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_faces_on_units_of_their_own(lib, kind):
+    """Cells staged face by face, every scale modulo the units' steps, the faces up to 2^70 apart."""
+    count = 400
+    mod = np.array(MODULI[0], float)
+    psi = 10.0 ** W.uniform(341, count, -4, 0)
+    for scale in (1.0, 2.0, 4.0, 8.0):
+        for above in (0, 1, 2, 3, 4, 5, 7, 10, 30, 59, 60, 61, 70):
+            for face in (0, 1):
+                whole, own = np.zeros((2, count)), np.zeros((2, count))
+                for i, u in enumerate(_cells(kind, 3, count, 342)):
+                    u, err = scale * u, np.zeros(24)
+                    u[:, 4 * face:4 * face + 4] *= 2.0 ** -above
+                    lib.errors_staged(_p(mod), _p(u), C.c_double(psi[i]), _p(err))
+                    ref, k, _ = _errors(lib, 3, mod, u, psi[i])
+                    for j, e in enumerate((err, ref[2])):
+                        whole[j, i], own[j, i] = e.max() / k.max(), (e / k).max()
+                for e in (whole, own):
+                    rms = np.sqrt((e ** 2).mean(axis=1))
+                    assert rms[0] <= rms[1], (scale, above, face, rms)
 
 
 @pytest.mark.parametrize("kind", KINDS)

@@ -215,3 +215,45 @@ def test_blocks_of_several_tiles(n):
     for _ in range(5):
         r, nrm = _residual(wk, wk.psi, u)
         assert _rel(r, ref) <= 1e-13 and np.isclose(nrm, oracle.norm_free(P, ref), rtol=1e-13)
+
+
+def _scale(P, psi, u, n):
+    """(|K| |u|) of every dof: the sum over its cells of |psi K_e| |u|."""
+    nx, ny, nz = n
+    Ke = np.abs(oracle.element_matrix(P))
+    v, out = np.abs(u).reshape(3, nz, ny, nx), np.zeros((3, nz, ny, nx))
+    at = lambda a: (slice(a >> 2, nz - 1 + (a >> 2)), slice((a >> 1) & 1, ny - 1 + ((a >> 1) & 1)),
+                    slice(a & 1, nx - 1 + (a & 1)))
+    U = np.stack([v[(p,) + at(a)] for a in range(8) for p in range(3)])
+    F = np.tensordot(Ke, U, axes=([1], [0])) * psi.reshape(nz - 1, ny - 1, nx - 1)
+    for a in range(8):
+        for p in range(3):
+            out[(p,) + at(a)] += F[a * 3 + p]
+    return out.reshape(-1)
+
+
+# FP64 forms of the operator differ in a dof by their rounding: 24 terms a cell and 8 cells, each
+# off by 2^-53 of its share of |K||u|, in either of the two
+LOCAL = 2 * 32 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("field", ["x2", "x3", "x4", "x8", "decay", "spot", "checker", "halves", "tiny"])
+def test_fields_of_many_sizes_in_a_tile(field):
+    """Displacements that vary by many powers of two within a tile of the 3D sweep: every
+    dof's error against its own |K||u|, and the same values wherever the tiles lie."""
+    n = (75, 27, 23)
+    wk = random_workload(3, n, 150, bits=(0, 0, 0))
+    P = oracle_problem(wk)
+    wk.f = np.zeros(P.ndofs)
+    X = W.node_coords(3, wk.n, wk.h)
+    x, y, z = (c / wk.h for c in X)
+    w = {"x2": ((1 + x) / 75) ** 2, "x3": ((1 + x) / 75) ** 3, "x4": ((1 + x) / 75) ** 4, "x8": ((1 + x) / 75) ** 8,
+         "decay": np.exp(-0.5 * x - 0.3 * y), "spot": np.exp(-0.1 * ((x - 40) ** 2 + (y - 13) ** 2 + (z - 11) ** 2)),
+         "checker": np.where((x + y + z) % 2 > 0, 1.0, 1e-9), "halves": np.where(x > 20, 1.0, 1e-12),
+         "tiny": np.where(y > 13, 1.0, 1e-140)}[field]
+    u = np.tile(w, 3) * W.uniform(151, P.ndofs, 0.5, 1) * np.sign(W.uniform(152, P.ndofs, -1, 1))
+    r, _ = _residual(wk, wk.psi, u)
+    ref, scale = oracle.residual(P, wk.psi, wk.f, u), _scale(P, wk.psi, u, n)
+    free = ~oracle.dirichlet_mask(P)
+    assert free.sum() == P.ndofs
+    assert (np.abs(r - ref) / scale).max() <= LOCAL
