@@ -16,8 +16,8 @@
 // V-cycle.
 //
 // Bound by FP64 issue (about two lanes per SM and clock): the gather's 72 + 32 additions a
-// node run on 64-bit integers instead, the node's values turned into them on their
-// largest exponent (53 bits kept down to 2^-5 of it); 16 FP64 instructions a node are
+// node run on 64-bit integers instead, the node's values turned into them on the
+// largest exponent of the stress rows (53 bits kept down to 2^-5 of it); 16 FP64 instructions a node are
 // left, and the square root where psi is not constant around the node.  Values that do
 // not fit (infinities, NaN, extreme exponents) are added in FP64.
 #include "sbm_common.cuh"
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(kThr) k_cell_stress(const SourceArgs A, const 
 // 2^d cells: the eigenstrain load sum_c sum_q s_q sig_pq(c) / (2^(d-1) h) from the
 // cell stresses, psi_n, |grad psi|_n and the volume share for the body force and
 // the traction.  The sums over the cells run on 64-bit integers (sbm_fix.cuh): with FP64
-// instructions their issue bound the kernel.  All three terms at 129^3: 0.66 -> 0.33 ms, the
+// instructions their issue bound the kernel.  All three terms at 129^3: 0.66 -> 0.30 ms, the
 // node's own FP64 instructions (|grad psi|, the products with b and t) being most of it.
 template <int D>
 __global__ void __launch_bounds__(kThr) k_source_terms(const SourceArgs A, const double *__restrict__ psi,
@@ -87,7 +87,9 @@ __global__ void __launch_bounds__(kThr) k_source_terms(const SourceArgs A, const
     const int NC = mc[0] * mc[1] * mc[2];
     constexpr int NV = D == 3 ? 6 : 3, NK = 1 << D;
     double sv[NK][NV], pv[NK];                    // the cells' stresses (0 outside the grid) and psi (mirrored)
-    unsigned ks = 0, kp = 0;
+    unsigned kv[NV], kp = 0;                      // largest exponents: of each stress component, of psi
+#pragma unroll
+    for (int v = 0; v < NV; ++v) kv[v] = 0;
     int inside = 0;
 #pragma unroll
     for (int c = 0; c < NK; ++c) {
@@ -106,7 +108,7 @@ __global__ void __launch_bounds__(kThr) k_source_terms(const SourceArgs A, const
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             sv[c][v] = (in && sig) ? sig[v * NC + cid] : 0.0;
-            ks = max(ks, fix::exp_key(sv[c][v]));
+            kv[v] = max(kv[v], fix::exp_key(sv[c][v]));
         }
     }
     double acc[D], ps, g[D];
@@ -142,8 +144,24 @@ __global__ void __launch_bounds__(kThr) k_source_terms(const SourceArgs A, const
             for (int a = 0; a < D; ++a) g[a] += ((c >> a) & 1) ? pv[c] : -pv[c];
         }
     }
-    // s_q = +1 when the cell lies below the node along q (bit clear), -1 above
-    if (fix::key_ok(ks)) {
+    // s_q = +1 when the cell lies below the node along q (bit clear), -1 above.  A component of the
+    // force sums a row of the stress; rows within 2^2 of each other share a unit (their own
+    // largest values then keep 56 bits), others take one each.
+    unsigned kr[D], ks = 0;
+#pragma unroll
+    for (int p = 0; p < D; ++p) {
+        kr[p] = 0;
+#pragma unroll
+        for (int q = 0; q < D; ++q) kr[p] = max(kr[p], kv[vslot<D>(p, q)]);
+        ks = max(ks, kr[p]);
+    }
+    bool shared = fix::key_ok(ks), each = true;
+#pragma unroll
+    for (int p = 0; p < D; ++p) {
+        each = each && fix::key_ok(kr[p]);
+        shared = shared && (kr[p] == 0u || (kr[p] >> 20) + 2u >= (ks >> 20));
+    }
+    if (shared) {
         const int E = max((int)(ks >> 20), fix::kExpLo);
         fix::i64 s[D];
 #pragma unroll
@@ -160,6 +178,20 @@ __global__ void __launch_bounds__(kThr) k_source_terms(const SourceArgs A, const
         }
 #pragma unroll
         for (int p = 0; p < D; ++p) acc[p] = fix::to_double(s[p], E - fix::kFixUnit + 2);
+    } else if (each) {
+#pragma unroll
+        for (int p = 0; p < D; ++p) {
+            const int E = max((int)(kr[p] >> 20), fix::kExpLo);
+            fix::i64 s = 0;
+#pragma unroll
+            for (int c = 0; c < NK; ++c)
+#pragma unroll
+                for (int q = 0; q < D; ++q) {
+                    const fix::i64 v = fix::to_fix<5>(sv[c][vslot<D>(p, q)], E);
+                    s += ((c >> q) & 1) ? -v : v;
+                }
+            acc[p] = fix::to_double(s, E - fix::kFixUnit + 2);
+        }
     } else {
 #pragma unroll
         for (int p = 0; p < D; ++p) {

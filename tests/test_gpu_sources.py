@@ -73,6 +73,27 @@ def test_source_terms_parity(built, dim, n):
             assert not got.any()
 
 
+@pytest.mark.parametrize("dim,n", [(2, (37, 29, 1)), (3, (17, 13, 11))])
+@pytest.mark.parametrize("small", [0.5, 0.1, 1e-3, 1e-12, 1e-30, 1e-200])
+def test_rows_of_the_stress_of_different_size(built, dim, n, small):
+    """Without coupling between the axes the last row of the eigenstrain's stress is 1 / small of the
+    others: each component of the load is as accurate as its own row."""
+    h, moduli = 1.0 / (n[0] - 1), (1.0, 0.0, 0.5)
+    P = oracle.Problem(dim, n, h, *moduli)
+    g = _grid(dim, n, h, moduli)
+    psi, eps0, _, _ = _inputs(P, 930 + dim)
+    e = eps0.reshape(-1, P.ncells)                # Voigt slots 2D xx yy xy, 3D xx yy zz yz xz xy
+    e[:dim - 1] *= small
+    if dim == 2:
+        e[2] = 0.0
+    else:
+        e[3:5] = 0.0
+        e[5] *= small
+    ref = oracle.source_terms(P, psi, eps0=e.reshape(-1)).reshape(dim, -1)
+    got = host(g.source_terms(cuda(psi), eps0=cuda(e.reshape(-1)))).reshape(dim, -1)
+    assert np.all(np.abs(got - ref).max(axis=1) <= 1e-13 * np.abs(ref).max(axis=1))
+
+
 def test_source_terms_parity_129_cubed(built):
     """The 129^3 grid of the damage workload (6.4 M dofs), its psi, a random
     eigenstrain, body force and traction: every entry against the oracle."""
