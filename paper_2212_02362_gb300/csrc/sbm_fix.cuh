@@ -205,7 +205,7 @@ __host__ __device__ __forceinline__ void cell_consts(i64 pm, const Consts &c, Fr
 // before they are added.
 constexpr int kNodeBits3 = 2, kNodeBits2 = 1;
 
-// psi the scheme takes: 0, or positive and within 2^+-200.
+// psi the scheme takes: 0 of either sign, or positive and within 2^+-200.
 __host__ __device__ __forceinline__ bool psi_ok(double psi)
 {
     const unsigned h = (unsigned)(bits_of(psi) >> 52);      // sign and exponent
@@ -217,7 +217,7 @@ __host__ __device__ __forceinline__ i64 psi_mantissa(double psi, int &e)
 {
     const i64 b = bits_of(psi);
     e = (int)((unsigned)(b >> 52) & 0x7ffu) - 1022;
-    return b == 0 ? 0 : (i64)((((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull) << 10);
+    return (b << 1) == 0 ? 0 : (i64)((((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull) << 10);
 }
 
 // The upper word of v's magnitude (less one for v < 0).

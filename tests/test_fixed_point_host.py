@@ -108,3 +108,8 @@ def test_values_outside_the_range_are_refused(cell3):
     for psi in (-1.0, np.nan, np.inf, 1e-90, 1e90):
         assert cell3(1.0, (1.0, 0.6, 0.5), u, psi)[0] == 1
     assert cell3(1e-40, (1.0, 0.6, 0.5), u, 1.0)[0] == 1
+
+
+def test_psi_of_negative_zero(cell3):
+    st, F = cell3(1.0, (1.0, 0.6, 0.5), W.uniform(42, 24, -1, 1), -0.0)
+    assert st == 0 and np.all(F == 0.0)

@@ -257,3 +257,19 @@ def test_fields_of_many_sizes_in_a_tile(field):
     free = ~oracle.dirichlet_mask(P)
     assert free.sum() == P.ndofs
     assert (np.abs(r - ref) / scale).max() <= LOCAL
+
+
+@pytest.mark.parametrize("dim,n", [(2, (49, 33)), (3, (35, 13, 29))])
+def test_psi_of_negative_zero(dim, n):
+    """psi as given may be a zero of either sign: no force."""
+    wk = random_workload(dim, n, 160)
+    u = W.uniform(161, dim * wk.nnodes, -1, 1)
+    psi = wk.psi.copy()
+    psi[::3] = 0.0
+    neg = np.where(psi == 0.0, -0.0, psi)
+    (r, nrm), (r0, nrm0) = _residual(wk, neg, u), _residual(wk, psi, u)
+    assert np.array_equal(r, r0) and nrm == nrm0
+    assert _rel(r, oracle.residual(oracle_problem(wk), psi, wk.f, u)) <= 1e-13
+    r, _ = _residual(wk, 0.0 * psi * -1.0, u)
+    free = ~oracle.dirichlet_mask(oracle_problem(wk))
+    assert np.array_equal(r[free], wk.f[free])
