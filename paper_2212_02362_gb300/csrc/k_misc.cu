@@ -263,6 +263,16 @@ __global__ void k_add(long long n, const TE *__restrict__ e, double *__restrict_
     if (t < n) u[t] += double(e[t]);
 }
 
+// The correction of adaptive inner cycles: e0 or e1, the buffer that the gate noted where it
+// closed (state of k_inner_gate), `last` where it did not.
+__global__ void k_add_gated(long long n, const float *e0, const float *e1, int last, const int *state, double *__restrict__ u)
+{
+    pdl_begin();
+    const float *e = (state[0] ? state[2] : last) ? e1 : e0;
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (t < n) u[t] += double(e[t]);
+}
+
 // out = a x + b y (+ c z): the vector updates of the adjoint Krylov solver.
 __global__ void k_lincomb(long long n, double a, const double *x, double b, const double *y, double c,
                           const double *z, double *out)
@@ -322,11 +332,14 @@ __global__ void k_norm_final(const double *__restrict__ part, int n, double *sca
     }
 }
 
+// Adaptive inner cycles: closes the gate once the FP32 residual is small enough, noting which of
+// the two buffers holds the iterate (later sweeps are skipped, so the host's count of them no
+// longer tells).  state = {closed, V-cycles run, buffer}.
 __global__ void k_inner_gate(const double *__restrict__ part, int n, const double *scal, double rtol,
-                             double tol_frac, int *gate, int *count)
+                             double tol_frac, int buffer, int *state)
 {
     pdl_begin();
-    if (*gate) return;
+    if (state[0]) return;
     __shared__ double red[kThreads];
     double s = 0.0;
     for (int i = threadIdx.x; i < n; i += kThreads) s += part[i];
@@ -339,8 +352,9 @@ __global__ void k_inner_gate(const double *__restrict__ part, int n, const doubl
     if (threadIdx.x == 0) {
         const double rn = sqrt(red[0]);
         const double thr = fmax(rtol * scal[7], tol_frac * scal[1]);
-        *count += 1;
-        if (rn <= thr) *gate = 1;
+        state[1] += 1;
+        state[2] = buffer;
+        if (rn <= thr) state[0] = 1;
     }
 }
 
@@ -828,6 +842,15 @@ cudaError_t launch_add(long long n, const TE *e, double *u, cudaStream_t s)
 template cudaError_t launch_add<float>(long long, const float *, double *, cudaStream_t);
 template cudaError_t launch_add<double>(long long, const double *, double *, cudaStream_t);
 
+cudaError_t launch_add_gated(long long n, const float *e0, const float *e1, int last, const int *state, double *u,
+                             cudaStream_t s)
+{
+    cudaError_t err = launch_pdl(k_add_gated, dim3(nblk(n)), dim3(kThreads), 0, s, n, e0, e1, last, state, u);
+    if (err != cudaSuccess) return err;
+    ++g_launches;
+    return cudaGetLastError();
+}
+
 cudaError_t launch_norm_final(const double *part, int nparts, double *scal, int which, cudaStream_t s,
                               const int *gate)
 {
@@ -855,9 +878,9 @@ cudaError_t launch_copy_gated(long long n, const double *src, double *dst, const
 }
 
 cudaError_t launch_inner_gate(const double *part, int nparts, const double *scal, double rtol, double tol_frac,
-                              int *gate, int *count, cudaStream_t s)
+                              int buffer, int *state, cudaStream_t s)
 {
-    cudaError_t e = launch_pdl(k_inner_gate, dim3(1), dim3(kThreads), 0, s, part, nparts, scal, rtol, tol_frac, gate, count);
+    cudaError_t e = launch_pdl(k_inner_gate, dim3(1), dim3(kThreads), 0, s, part, nparts, scal, rtol, tol_frac, buffer, state);
     if (e != cudaSuccess) return e;
     ++g_launches;
     return cudaGetLastError();

@@ -118,7 +118,7 @@ struct sbm_grid_s {
     double *part = nullptr;
     long long npart = 0;
     int *derr = nullptr;        // device error flag of the TMA kernels
-    int *dgate = nullptr;       // adaptive inner cycles: [0] gate flag, [1] FP32 V-cycles run
+    int *dgate = nullptr;       // adaptive inner cycles: [0] gate flag, [1] FP32 V-cycles run, [2] buffer of the iterate
     const int *cur_gate = nullptr;   // gate applied to the launches being enqueued (or null)
     int cur_ctas = 0;           // CTAs of the persistent sweeps being enqueued (0: one per SM)
     double gate_rtol = 0, gate_tol = 0;
@@ -423,7 +423,7 @@ cudaError_t vcycle(sbm_grid G, int l, int &cur, const sbm_opts &o, const T *f, i
         // FP32 V-cycles of the outer iteration go on
         CKE(sweep<T>(G, l, kResidual, P<T>::u(L, cur), f, P<T>::r(L), G->part, 0.0));
         CKE(launch_inner_gate(G->part, (int)sweep_nblocks(G, l, true, P<T>::u(L, cur), f), G->scal, G->gate_rtol,
-                              G->gate_tol, G->dgate, G->dgate + 1, G->st));
+                              G->gate_tol, cur, G->dgate, G->st));
     } else if (!restricted) {
         CKE(sweep<T>(G, l, kResidual, P<T>::u(L, cur), f, P<T>::r(L), nullptr, 0.0));
     }
@@ -490,7 +490,9 @@ cudaError_t enqueue_body(sbm_grid G, const sbm_opts &o, const double *rhs)
             e = vcycle<float>(G, fine, cur, o, L.sf, it == 0 ? pre : 0);
         G->cur_gate = nullptr;
         CKE(e);
-        CKE(launch_add<float>((long long)L.g.dim * L.g.cs, L.su[cur], L.du[0], G->st));
+        const long long n = (long long)L.g.dim * L.g.cs;
+        if (o.inner_rtol > 0.0) CKE(launch_add_gated(n, L.su[0], L.su[1], cur, G->dgate, L.du[0], G->st));
+        else CKE(launch_add<float>(n, L.su[cur], L.du[0], G->st));
         return residual64(G, rhs, 1, 2);
     }
     int cur = 0;
@@ -1707,8 +1709,8 @@ static sbm_status grid_create_impl(const sbm_grid_desc *d, sbm_grid G)
                              sweep_blocks_f2(G->L[l].g)});
     CK(gmalloc(G, (void **)&G->part, sizeof(double) * G->npart));
     CK(gmalloc(G, (void **)&G->derr, sizeof(int)));
-    CK(gmalloc(G, (void **)&G->dgate, 2 * sizeof(int)));
-    CK(cudaMemset(G->dgate, 0, 2 * sizeof(int)));
+    CK(gmalloc(G, (void **)&G->dgate, 3 * sizeof(int)));
+    CK(cudaMemset(G->dgate, 0, 3 * sizeof(int)));
     CK(cudaMemset(G->derr, 0, sizeof(int)));
     CK(gmalloc(G, (void **)&G->scal, sizeof(double) * 16));
     CK(cudaMemset(G->scal, 0, sizeof(double) * 16));

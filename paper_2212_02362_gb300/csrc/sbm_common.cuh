@@ -272,6 +272,10 @@ cudaError_t launch_set_face(const Geom &g, int face, int comp, double value, dou
 // u64 += e (FP32 or FP64) over n elements
 template <typename TE>
 cudaError_t launch_add(long long n, const TE *e, double *u, cudaStream_t s);
+// u += e0 or e1, after adaptive inner cycles (state of launch_inner_gate; last: the buffer if the
+// gate did not close).
+cudaError_t launch_add_gated(long long n, const float *e0, const float *e1, int last, const int *state, double *u,
+                             cudaStream_t s);
 // deterministic final reduction of block partials: out[0] = sum, optional relres
 cudaError_t launch_norm_final(const double *part, int nparts, double *scal, int which,
                               cudaStream_t s, const int *gate = nullptr);
@@ -308,11 +312,11 @@ template <typename T>
 cudaError_t launch_bottom_apply(int n, const T *Ainv, const int *gather, const T *b, T *u,
                                 int accumulate, cudaStream_t s, const int *gate = nullptr);
 // Adaptive inner cycles: sum the partial sums of the FP32 residual of this V-cycle
-// and set *gate when its norm <= max(rtol * scal[7], tol_frac * scal[1]) (scal[7]:
-// the latest FP64 residual norm, scal[1]: the initial one); counts the V-cycles
-// run in *count.  Skipped itself once the gate is set.
+// and close the gate when its norm <= max(rtol * scal[7], tol_frac * scal[1]) (scal[7]:
+// the latest FP64 residual norm, scal[1]: the initial one).  state = {closed, V-cycles
+// run, buffer of the iterate}; skipped itself once closed.
 cudaError_t launch_inner_gate(const double *part, int nparts, const double *scal, double rtol, double tol_frac,
-                              int *gate, int *count, cudaStream_t s);
+                              int buffer, int *state, cudaStream_t s);
 // dJ/dpsi_c = -lambda_c^T S_c u_c (packed u, lambda; packed cell output) and the
 // optional chain rule through the SIMP map or the psi_min floor.
 cudaError_t launch_dJdpsi(const Geom &g, const Coef<double> &c, const double *u, const double *lam,
