@@ -273,3 +273,91 @@ def test_psi_of_negative_zero(dim, n):
     r, _ = _residual(wk, 0.0 * psi * -1.0, u)
     free = ~oracle.dirichlet_mask(oracle_problem(wk))
     assert np.array_equal(r[free], wk.f[free])
+
+
+def _check_local(wk, psi, u):
+    """The residual dof by dof where it is finite, and its norm."""
+    P = oracle_problem(wk)
+    with np.errstate(invalid="ignore", over="ignore"):
+        ref = oracle.residual(P, psi, wk.f, u)
+        norm = oracle.norm_free(P, ref)
+        scale = np.nan_to_num(_scale(P, np.abs(psi), np.abs(u), wk.n), posinf=np.inf)   # fixed dofs beside a NaN: exact
+    r, nrm = _residual(wk, psi, u)
+    fin = np.isfinite(ref)
+    assert np.array_equal(fin, np.isfinite(r))
+    assert np.all(np.abs(r - ref)[fin] <= (LOCAL * scale + 2.0 ** -51 * np.abs(wk.f))[fin])
+    assert np.isclose(nrm, norm, rtol=1e-13) if np.isfinite(norm) else not np.isfinite(nrm)
+
+
+# the tiled sweep: 24 tiles of 32 x 10 cells, six or seven planes a block
+TILED = (129, 61, 40)
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan, 1e250, 1e-250])
+@pytest.mark.parametrize("plane", [0, 17, 39])
+def test_tiled_values_that_do_not_fit(value, plane):
+    """A cell that does not fit, at the bottom, inside and at the top of the blocks' ranges: the blocks
+    that hold it finish with FP64 instructions, their partial norms in two parts."""
+    wk = random_workload(3, TILED, 200)
+    u = W.uniform(201, 3 * wk.nnodes, -1, 1)
+    v = u.reshape(3, 40, 61, 129)
+    if value == 1e-250:
+        v[:, max(plane - 2, 0):plane + 3, 26:33, 60:68] = 0.0
+    v[1, plane, 29, 64] = value                   # a corner of four tiles
+    _check_local(wk, wk.psi, u)
+
+
+@pytest.mark.parametrize("value", [-0.5, np.inf, np.nan, 1e-70, 1e70])
+@pytest.mark.parametrize("layer", [0, 17, 38])
+def test_tiled_psi_that_does_not_fit(value, layer):
+    wk = random_workload(3, TILED, 202)
+    psi = wk.psi.copy()
+    psi.reshape(39, 60, 128)[layer, 29, 63] = value
+    _check_local(wk, psi, W.uniform(203, 3 * wk.nnodes, -1, 1))
+
+
+@pytest.mark.parametrize("moduli", [(1e70, 0.6e70, 0.5e70), (1e-70, 0.6e-70, 0.5e-70), (1.0, 0.0, 1e-3)])
+def test_moduli_that_do_not_fit(moduli):
+    for n in ((97, 41, 25), (65, 49, 1)):
+        wk = random_workload(3 if n[2] > 1 else 2, n, 204, moduli=moduli)
+        wk.f = moduli[0] * wk.f
+        P, u = oracle_problem(wk), W.uniform(205, (3 if n[2] > 1 else 2) * wk.nnodes, -1, 1)
+        if wk.dim == 3:
+            _check_local(wk, wk.psi, u)
+        else:
+            r, nrm = _residual(wk, wk.psi, u)
+            ref = oracle.residual(P, wk.psi, wk.f, u)
+            assert _rel(r, ref) <= 1e-13 and np.isclose(nrm, oracle.norm_free(P, ref), rtol=1e-13)
+
+
+def test_wide_psi_and_rigid_motion_on_tiles():
+    """psi over eight decades, cells without force beside full ones; a translation gives none."""
+    wk = random_workload(3, TILED, 206)
+    psi = 10.0 ** W.uniform(207, wk.ncells, -8, 0)
+    psi[::5] = 0.0
+    _check_local(wk, psi, W.uniform(208, 3 * wk.nnodes, -1, 1))
+    r, _ = _residual(wk, psi, np.repeat([0.3, -0.7, 1.1], wk.nnodes))
+    free = ~oracle.dirichlet_mask(oracle_problem(wk))
+    assert np.array_equal(r[free], wk.f[free])
+
+
+@pytest.mark.parametrize("scale", [1e-150, 1e-120, 1.0, 1e140, 1e150])
+def test_tiled_magnitudes(scale):
+    wk = random_workload(3, (97, 41, 25), 210)
+    wk.f = scale * wk.f
+    P, u = oracle_problem(wk), scale * W.uniform(211, 3 * wk.nnodes, -1, 1)
+    r, _ = _residual(wk, wk.psi, u)
+    assert _rel(r / scale, oracle.residual(P, wk.psi, wk.f, u) / scale) <= 1e-13
+
+
+def test_hand_over_with_fp32_output():
+    """The residual of a mixed solve is written in FP32: a start with a value below the range of
+    the integer form gives the iterates of one without."""
+    wk = random_workload(3, (65, 33, 41), 212, moduli=W.iso_cubic(1.0, 0.2))
+    g = gpu_grid(wk, precision="mixed")
+    kw = dict(omega=0.5, tol=0.0, max_cycles=2, raise_on_fail=False)
+    u = cuda(wk.u0)
+    v = u.clone()
+    v.view(3, 41, 33, 65)[1, 20, 16, 32] = 1e-140
+    a, b = g.solve(u, **kw), g.solve(v, **kw)
+    assert np.allclose(a.history, b.history, rtol=1e-6) and _rel(host(v), host(u)) <= 1e-6
