@@ -1,10 +1,13 @@
 """V-cycle options that the default V(2,2) cycle does not reach: adaptive inner cycles that
-stop after any number of sweeps."""
+stop after any number of sweeps, other counts of sweeps on levels of every kind (fused
+small ones, per-node, tiled), and cycles whose arithmetic is all FP64 instructions."""
 import numpy as np
 import pytest
 
 import oracle
 import workloads as W
+import test_gpu_amr as amr
+from _amr import dense_solve
 from _sbm import cuda, gpu_grid, host, oracle_problem, random_workload
 
 pytestmark = pytest.mark.gpu
@@ -67,3 +70,63 @@ def test_gate_that_closes_after_the_pre_smoothing(dim, n, nu1, nu2, use_graph):
             break
     assert info.vcycles == 2
     check(u, _sweeps(g, r, e1, nu1, omega))
+
+
+COUNTS = [(0, 1), (1, 0), (0, 2), (2, 0), (1, 1), (1, 2), (2, 1), (3, 2), (1, 3)]
+# 2D: fused levels only, and unfused ones above them; 3D: per-node levels and a tiled one
+GRIDS = [(2, (33, 49)), (2, (161, 193)), (3, (17, 25, 17)), (3, (33, 33, 25))]
+
+
+def _err(u, ref, u0):
+    return np.abs(u - ref).max() / np.abs(ref - u0).max()
+
+
+@pytest.mark.parametrize("nu1,nu2", COUNTS)
+@pytest.mark.parametrize("dim,n", GRIDS)
+def test_sweep_counts(dim, n, nu1, nu2):
+    """Two cycles from the boundary data, as the oracle's."""
+    wk = random_workload(dim, n, 180, moduli=W.iso_cubic(1.0, 0.2))
+    P, psi = oracle_problem(wk), oracle.floor_psi(wk.psi, wk.psi_min)
+    for smoother in ("jacobi", "gs"):
+        kw = dict(nu1=nu1, nu2=nu2, omega=0.5, smoother=smoother, tol=0.0, max_cycles=2)
+        ref = oracle.mg_solve(P, psi, wk.f, wk.u0, **kw)
+        for precision, tol in (("fp64", 1e-11), ("mixed", 1e-4)):
+            g = gpu_grid(wk, precision=precision)
+            u = cuda(wk.u0)
+            info = g.solve(u, raise_on_fail=False, **kw)
+            assert _err(host(u), ref.u, wk.u0) <= tol, (smoother, precision)
+            assert np.allclose(info.history, ref.history[:3], rtol=1e-9 if precision == "fp64" else 1e-3)
+
+
+@pytest.mark.parametrize("nu1,nu2", [(0, 2), (1, 1), (1, 2), (2, 1), (3, 0)])
+@pytest.mark.parametrize("case", ["2d_multibox", "3d_two_slabs"])
+@pytest.mark.parametrize("precision,inner", [("fp64", 1), ("mixed", 1), ("mixed", 4)])
+def test_sweep_counts_on_patches(case, precision, inner, nu1, nu2):
+    wk = amr.SMALL[case]()
+    A, psis = amr._oracle(wk)
+    us0 = [np.ascontiguousarray(wk.level_u0(a)) for a in range(A.nlev)]
+    ref = dense_solve(A, psis, amr._zeros_f(A), us0)
+    for smoother in ("jacobi", wk.smoother):
+        g = amr._gpu(wk, precision)
+        us = [cuda(u) for u in us0]
+        g.amr_solve(us, tol=1e-10, omega=wk.omega, smoother=smoother, nu1=nu1, nu2=nu2, inner_cycles=inner)
+        num = np.sqrt(sum(((host(us[a]) - ref[a]) ** 2).sum() for a in range(A.nlev)))
+        assert num <= 1e-8 * np.sqrt(sum((r ** 2).sum() for r in ref))
+
+
+@pytest.mark.parametrize("smoother", ["jacobi", "gs"])
+@pytest.mark.parametrize("dim,n", GRIDS)
+def test_cycles_in_fp64_instructions(dim, n, smoother):
+    """Moduli beyond the integer form's range: every kernel of the cycle takes its FP64 branch, and
+    with the load scaled alike the iterates are those of moderate moduli."""
+    wk = random_workload(dim, n, 190, moduli=W.iso_cubic(1.0, 0.2))
+    kw = dict(omega=0.5, smoother=smoother, tol=0.0, max_cycles=3, raise_on_fail=False)
+    g = gpu_grid(wk)
+    u = cuda(wk.u0)
+    info = g.solve(u, **kw)
+    wk.moduli, wk.f = tuple(1e70 * m for m in wk.moduli), 1e70 * wk.f
+    g = gpu_grid(wk)
+    v = cuda(wk.u0)
+    big = g.solve(v, **kw)
+    assert _err(host(v), host(u), wk.u0) <= 1e-12
+    assert np.allclose(big.history, info.history, rtol=1e-9)
