@@ -483,24 +483,11 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned nblocks, un
 // before), of which the pivot chain is 0.16 and 0.30.
 constexpr int kGJB = 16;
 
-// 1 / d, d > 0, to an ulp: the hardware's approximate reciprocal (PTX rcp.approx.ftz.f64,
-// 2^-20) and one cubic Newton step r <- r + r (e + e^2), e = 1 - d r.  The inversion below
-// is a chain of these; extreme exponents take the division.
-__device__ __forceinline__ double pivot_rcp(double d)
-{
-    const int ex = (int)(__double_as_longlong(d) >> 52);
-    if (ex < 64 || ex > 1980) return 1.0 / d;
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    const double e = fma(-d, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-
 // Inverse of the kGJB x kGJB SPD matrix in shared memory by threads 0 .. 127.  An SM
 // sub-partition issues one FP64 instruction of a warp in 64 cycles, dependent or not, so the
-// matrix is spread over four warps (thread: row tid / 8, two columns) and a step costs each
-// of them six: the reciprocal (3), the scaled column and two updates.  By symmetry the pivot
-// row is the pivot column, which its owners hand round through colbuf[2][kGJB].
+// matrix is spread over four warps (thread: row tid / 8, two columns): a step costs each of
+// them the division, the scaled column and two updates.  By symmetry the pivot row is the
+// pivot column, which its owners hand round through colbuf[2][kGJB].
 __device__ __forceinline__ void invert_pivot(double (*P)[kGJB + 1], double (*colbuf)[kGJB], int tid)
 {
     const int r = tid >> 3, c0 = 2 * (tid & 7);
@@ -510,7 +497,7 @@ __device__ __forceinline__ void invert_pivot(double (*P)[kGJB + 1], double (*col
 #pragma unroll
     for (int q = 0; q < kGJB; ++q) {
         const double *col = colbuf[q & 1];
-        const double ip = pivot_rcp(col[q]);
+        const double ip = 1.0 / col[q];
         const double t = col[r] * ip;                              // S_rq / S_qq
 #pragma unroll
         for (int e = 0; e < 2; ++e) {

@@ -433,3 +433,25 @@ def test_full_size_damage_129_apply_samples_and_residual(built):
         assert info.converged
         assert oracle.norm_free(P, r) / oracle.norm_free(P, r0) <= 2e-10
         del g
+
+
+@pytest.mark.parametrize("n", [(4, 4, 4), (4, 5, 6), (6, 6, 8), (8, 8, 6), (8, 8, 8), (4, 4, 1), (6, 8, 1), (20, 30, 1)])
+def test_bottom_inverse_is_as_close_as_lapacks(built, n):
+    """Single-level grids of 32 to 1536 dofs, multiples of the pivot blocks' 16 and not, the largest
+    with its panel outside shared memory: A (A^-1 f) against f, beside an inverse by LAPACK."""
+    dim = 3 if n[2] > 1 else 2
+    wk = random_workload(dim, n, 220)
+    g, P = gpu_grid(wk), oracle_problem(wk)
+    assert g.nlevels == 1
+    free = ~oracle.dirichlet_mask(P)
+    A = oracle.assemble_dense(P, oracle.floor_psi(wk.psi, wk.psi_min))[np.ix_(free, free)]
+    inv = np.linalg.inv(A)
+    worst = {"lib": 0.0, "lapack": 0.0}
+    for seed in range(5):
+        f = W.uniform(221 + seed, P.ndofs, -1, 1) * free
+        x = host(g.bottom_correct(cuda(f), cuda(np.zeros(P.ndofs))))[free]
+        for k, y in (("lib", x), ("lapack", inv @ f[free])):
+            y = y.astype(np.longdouble)
+            r = np.abs(A.astype(np.longdouble) @ y - f[free]).max() / (np.abs(A) @ np.abs(y)).max()
+            worst[k] = max(worst[k], float(r))
+    assert worst["lib"] <= 4 * worst["lapack"], worst
