@@ -164,7 +164,12 @@ sbm_status sbm_source_terms(sbm_grid grid, int level, const double *psi, const d
  * the solution on return; Dirichlet dofs are set from the face conditions and
  * never changed by the iteration.  opts may be NULL (defaults); info may be NULL.
  * Synchronises the grid stream.  Returns SBM_OK, SBM_ERR_NOCONV or
- * SBM_ERR_DIVERGED (info is filled in all three cases). */
+ * SBM_ERR_DIVERGED (info is filled in all three cases).
+ * Device memory: the first solve of a grid with FP64 cycles and Jacobi smoothing allocates
+ * 8 bytes a node of every level but the coarsest for the levels' Jacobi scaling, and the
+ * grid keeps them; a level for which that fails is smoothed without (same values, a division a
+ * node and sweep more).  The first FP64 solve with inner_cycles > 1 allocates 8 (max_cycles + 1)
+ * bytes, and fails with SBM_ERR_OOM without them. */
 sbm_status sbm_solve(sbm_grid grid, double *u, const sbm_opts *opts, sbm_info *info);
 
 /* Adjoint of a solve: lambda solves K lambda = dJdu with homogeneous Dirichlet
@@ -283,7 +288,8 @@ sbm_status sbm_jacobi_product(sbm_grid grid, int variant, const double *psi, con
  * sbm_set_alloc_limit: from now on, a grid creation (or patch addition) whose
  * device allocations would exceed `bytes` in total fails with SBM_ERR_OOM, as if
  * cudaMalloc had run out of memory; a failed creation frees what it allocated and
- * reports through sbm_last_error(NULL).  0 removes the cap.  Process-wide.
+ * reports through sbm_last_error(NULL).  0 removes the cap.  Process-wide.  The Jacobi
+ * scaling of an FP64 solve (see sbm_solve) counts against it too, but is done without.
  * sbm_set_wait_limit: polls each block makes at one grid barrier of the
  * bottom-level inversion (one cooperative launch, run by the first solve after
  * psi or the moduli change) before it gives up; on a timeout every block leaves

@@ -484,9 +484,10 @@ __global__ void __launch_bounds__(kNode64Threads) k_sweep3_node64(const SweepArg
         Ku = p == 0 ? f[0] : p == 1 ? f[1] : f[2];
     }
     if (MODE == kJacobi && !a.dinv) {
-        double s = psi;
-#pragma unroll
-        for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        double s = psi;                                   // over z, x, y: the order of dinv
+        s += __shfl_xor_sync(0xffffffffu, s, 4);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
         ip = 1.0 / s;
     }
     if (!valid || c >= 3) return;

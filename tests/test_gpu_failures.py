@@ -121,3 +121,21 @@ def test_refinement_boxes_must_nest(built):
             g.amr_add_level(lo, hi)
         assert e.value.status == _capi.SBM_ERR_ARG
     g.amr_add_level((10, 10), (36, 36))   # one parent cell inside on every side
+
+
+@pytest.mark.parametrize("wk", [W.plate_hole(65), W.damage3d(33)], ids=["2d", "3d"])
+def test_solve_at_the_allocation_cap_gives_the_same_values(built, wk):
+    """The Jacobi scaling of FP64 cycles is allocated by the first solve; without room for it the
+    sweeps divide, and a later psi takes it up again."""
+    g, ref = gpu_grid(wk), cuda(wk.u0)
+    want = gpu_grid(wk).solve(ref, omega=wk.omega)
+    sbm.lib().sbm_set_alloc_limit(1)
+    try:
+        u = cuda(wk.u0)
+        info = g.solve(u, omega=wk.omega)
+    finally:
+        sbm.lib().sbm_set_alloc_limit(0)
+    assert info.cycles == want.cycles and torch.equal(u, ref)
+    g.set_psi(cuda(wk.psi), wk.psi_min)
+    v = cuda(wk.u0)
+    assert g.solve(v, omega=wk.omega).cycles == want.cycles and torch.equal(v, ref)
