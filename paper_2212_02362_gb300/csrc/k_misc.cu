@@ -479,8 +479,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned nblocks, un
 // orders the passes.  In a pass four warps invert the pivot block (a chain of kGJB
 // reciprocals, which bounds a pass on small n) while the others bring the panel to
 // shared memory; then the warps share the 32-column pieces of the block's rows.  375
-// dofs 0.66 -> 0.31 ms, 720 dofs 2.05 -> 0.74 ms (the Gauss-Jordan form by 256 threads
-// before), of which the pivot chain is 0.16 and 0.30.
+// dofs 0.66 -> 0.32 ms, 720 dofs 2.05 -> 0.75 ms (the Gauss-Jordan form by 256 threads
+// before), about half of it the pivot chain.
 constexpr int kGJB = 16;
 
 // Inverse of the kGJB x kGJB SPD matrix in shared memory by threads 0 .. 127.  An SM
@@ -648,7 +648,7 @@ __global__ void k_bottom_apply(int n, const T *__restrict__ Ainv, const int *__r
 // density != 0: dJ/drho = dJ/dpsi (1 - psi_min) q rho^(q-1);  density == 0 and
 // grho != null: dJ/dpsi_raw = dJ/dpsi where psi_raw > psi_min, else 0.  The 3D product is
 // formed in integers (sbm_fix.cuh): in FP64 its 220 instructions a cell took 1.58 ms on
-// 4.2 M cells, bound by their issue; 0.60 ms in integers.
+// 4.2 M cells, bound by their issue; 0.63 ms in integers.
 __global__ void k_dJdpsi(const Geom g, const Coef<double> c, const fix::Consts fc, const double *__restrict__ u,
                          const double *__restrict__ lam, double *__restrict__ gout, double *__restrict__ grho,
                          const double *__restrict__ rho, const double *__restrict__ praw, double psi_min,

@@ -31,8 +31,8 @@
 // of cells far below the tile's largest value.
 //
 // Measured (kernel time, FP64 instructions -> this form): residual with norm at 129^3
-// 812 -> 212 us (0.76 TB/s), Jacobi sweep at 65^3 155 -> 40 us, at 33^3 46 -> 12.5 us; issue
-// and latency of one block of 12 warps per SM (registers).
+// 812 -> 204 us (0.84 TB/s), Jacobi sweep with kept scaling at 65^3 155 -> 35 us, at 33^3 46 ->
+// 11.5 us; issue and latency of one block of 12 warps per SM (registers).
 #include <algorithm>
 
 #include "sbm_common.cuh"
@@ -421,8 +421,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep3_fix(const SweepArgs<double, TO
 // the node is corner c; exponents and forces are combined by shuffles and the first three
 // lanes finalise a component each.  A cell that does not fit sends its warp to FP64
 // instructions.  No shared memory, no barrier, no plane ring: what is left is one round
-// of loads and one cell's chain.  A sweep at 9^3 and 17^3: 12 us with the tiled kernel, 5
-// and 7 us here; at 33^3 14 and 24 us, hence the limit kNode64MaxNodes.
+// of loads and one cell's chain (7 us at 17^3 against 12 us tiled; see kNode64MaxNodes).
 constexpr int kNode64Threads = 128;
 
 template <int MODE>
@@ -507,7 +506,7 @@ __global__ void __launch_bounds__(kNode64Threads) k_sweep3_node64(const SweepArg
 // value that does not fit evaluates its cells with FP64 instructions.  What is left is
 // latency (one round of loads, one barrier), so small grids take the flat tile, which
 // spreads the FP64 instructions of the update over twice as many SMs.  A Jacobi sweep took
-// 9.6 us at 65^2 and 40 us at 513^2 with FP64 instructions; 4 and 13 us here.
+// 9.6 us at 65^2 and 40 us at 513^2 with FP64 instructions; 2.9 and 12 us here.
 constexpr int TX2 = 32;
 
 // PRO: u is taken as u + P ec, ec the correction on the coarse level gc (a prolongation
@@ -764,7 +763,7 @@ __global__ void __launch_bounds__(kRrThreads) k_resid_restrict2(const SweepArgs<
 // The diagonal blocks follow from psi sums: every corner of the unit-psi cell matrix has
 // the same diagonal entry, and the same coupling up to its sign (+ at corners 0 and 3).
 // A sweep of the refinement levels (1 to 49 tiles) took 51 us with FP64 instructions and a
-// thread per node, 14 us here; what is left is the four phases' chain.
+// thread per node, 11 to 14 us here; what is left is the four phases' chain.
 constexpr int kGsThreads = 512;
 
 template <int TILE>

@@ -83,8 +83,10 @@ struct Patch {
 
 constexpr int kBranches = 8;   // side streams for concurrent patches
 // CTAs handed out to the patches in flight: two per SM's worth, since a sweep's CTAs finish at
-// different times (refined 3D voids: 29.0 ms without shares, 30.1 with 152, 28.1 with 228,
-// 27.7 with 304).
+// different times.  Composite solves with 152, 228, 304, 608 CTAs and without shares, in ms, five
+// layouts of 3 to 8 patches: 65^3 + 2 levels 28.7, 26.9, 26.5, 26.9, 27.6; 49^3 + 2 11.25, 10.80, 10.69, 10.79,
+// 10.81; 57^3 + 1 8.45, 8.24, 8.09, 8.19, 8.21; 33^3 + 2 9.46, 9.71, 9.51, 9.64, 9.71; 41^3 + 2 8.61, 8.55, 8.57,
+// 8.77, 8.79.
 constexpr double kShareCtas = 304;
 
 struct GraphSlot {

@@ -202,8 +202,11 @@ long long sweep_blocks_fix(const Geom &g);
 // small levels (no partial sums).
 cudaError_t launch_sweep_node64(int mode, const SweepArgs<double, double> &a, cudaStream_t s);
 // Levels with at most this many nodes use it: there the tiled sweep's few blocks and the
-// latency of its plane ring cost more than evaluating every cell eight times (9^3 and 17^3:
-// 12 against 5 us a sweep; 33^3: 14 against 24 us).
+// latency of its plane ring cost more than evaluating every cell eight times.  A Jacobi sweep
+// per node / tiled, in us: 13^3 3.6 / 11.6, 17^3 7.1 / 11.7, 21^3 7.4 / 11.9, 23^3 (12 167 nodes)
+// 9.9 / 11.9, 25^3 (15 625) 11.8 / 11.8, 27^3 14.3 / 11.9, 33^3 21.8 / 11.6; 129 x 9 x 9 (10 449) 8.9 /
+// 11.3.  The per-node kernel goes up by waves (9 728 nodes fill the chip once), so the line is
+// kept below the crossing.
 constexpr long long kNode64MaxNodes = 12000;
 // dinv[node] = 1 / (sum of psi over the node's cells), summed in the sweeps' order.
 cudaError_t launch_inv_psi(const Geom &g, const double *psi, double *dinv, cudaStream_t s);
@@ -300,7 +303,10 @@ cudaError_t launch_resid_restrict(const SweepArgs<double, double> &a, const Geom
                                   const FirstSweep<double> &first, cudaStream_t s);
 cudaError_t launch_prolong_sweep(const SweepArgs<float, float> &a, const Geom &gc, const float *ec, cudaStream_t s);
 cudaError_t launch_prolong_sweep(const SweepArgs<double, double> &a, const Geom &gc, const double *ec, cudaStream_t s);
-// 2D FP64 levels with at most this many nodes take the fused steps.
+// 2D FP64 levels with at most this many nodes take the fused steps.  A V(2,2) cycle, finest
+// level fused / not, in us: 65^2 79.8 / 92 (all levels not), 145^2 (21 025 nodes) 87.9 / 92.5, 161^2
+// (25 921) 100.4 / 104.5, 193^2 (37 249) 104.4 / 105.0, 257^2 132.4 / 130.9, 513^2 215.6 / 203.5: they cross
+// near 37 000 nodes, and between there and the line lies little.
 constexpr long long kFuse2MaxNodes = 20000;
 
 // Inverse of the coarsest-level matrix (half bandwidth bw) in place (one cooperative launch);
