@@ -3,9 +3,9 @@
 //
 // What bounds it (3D).  With FP64 instructions the sweep is bound by their issue rate (about
 // two lanes per SM and clock on GB300): some 180 of them per cell.  In block floating
-// point the same cell takes about 800 integer instructions, which issue 64 times as
-// fast, and leaves some ten FP64 instructions per node (the conversion of the node's
-// force, f - K u, the norm), which run on the FP64 pipe beside them.
+// point a cell takes some 1100 integer instructions, conversions included, which issue 64
+// times as fast, and leaves some ten FP64 instructions per node (the conversion of the
+// node's force, f - K u, the norm), which run on the FP64 pipe beside them.
 //
 // Work split.  A block owns a tile of 32 x 10 cells in x/y (33 x 11 threads, one per cell
 // column with the halo column and row; 12 warps, so 168 registers a thread) and a
@@ -27,7 +27,7 @@
 // body below, which also runs when the level's constants do not fit.
 //
 // A unit per staged plane and tile instead (values converted once, in place, instead of by
-// the four cells around a column) took 200 us for the 129^3 residual, but lost the digits
+// the four cells around a column) took 213 us for a 129^3 residual call, 231 now, but lost the digits
 // of cells far below the tile's largest value.
 //
 // Measured (kernel time, FP64 instructions -> this form): residual with norm at 129^3
