@@ -480,7 +480,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned nblocks, un
 // reciprocals, which bounds a pass on small n) while the others bring the panel to
 // shared memory; then the warps share the 32-column pieces of the block's rows.  375
 // dofs 0.66 -> 0.32 ms, 720 dofs 2.05 -> 0.75 ms (the Gauss-Jordan form by 256 threads
-// before), about half of it the pivot chain.
+// before).
 constexpr int kGJB = 16;
 
 // Inverse of the kGJB x kGJB SPD matrix in shared memory by threads 0 .. 127.  An SM
